@@ -859,7 +859,7 @@ static size_t carve_select(int B, int M, int N, int K, Scratch* s, char* base,
                            R0State* r0s = nullptr, int wide_pool = 0, WideState* ws = nullptr) {
   Carver c{base};
   Scratch t{};
-  t.nSel = 64;
+  t.nSel = 512;  // blocks of the copy and total pass per image (about three per SM)
   t.status = c.take<uint32_t>(4);
   t.C = c.take<float>((size_t)B * M * N);
   t.scol = c.take<uint16_t>((size_t)B * M * N);
@@ -923,10 +923,7 @@ int gmc_select(const float* clients, int B, int M, int N, int K, const gmc_param
     GMC_TRY(cudaMemsetAsync(trace, 0, (size_t)B * L.bytes_per_image, st));
   }
   GMC_TRY(cudaMemsetAsync(s.status, 0, sizeof(uint32_t), st));
-  GMC_TRY(cudaMemcpyAsync(s.C, clients, sizeof(float) * B * (size_t)M * N,
-                          cudaMemcpyDeviceToDevice, st));
-  GMC_TRY(cudaMemsetAsync(s.u0, 0, sizeof(long long) * B * (size_t)N, st));
-  GMC_TRY(launch_select_prep(s.C, B, M, N, s, st));
+  GMC_TRY(launch_select_prep(clients, B, M, N, s, st));  // copies the clients into s.C
   if (wp || !select_fits(B, N, M, p.pool_mult * p.batch_b)) {
     WideGeom wg{};
     wg.B = B; wg.N = N; wg.K = K; wg.Mstride = M;

@@ -110,7 +110,7 @@ struct Scratch {
   int32_t* pi;       // [B][N]
   uint32_t* mbits;   // [B][K][ceil(N/32)] members of each carrier slot, bit i = token i
   float* mass;       // [B][N]
-  double* selpart;   // [B][64]        select-path total mass partials
+  double* selpart;   // [B][nSel]      select-path total mass partials
   int32_t* fexp;     // [B]            select-path fixed-point exponents
   __nv_bfloat16* Qp; // [B][Hkv][RQ][d] packed text queries of each KV group (tcgen05 path)
   int nP, nHG, nA, nSel, nE, nRS;
@@ -189,7 +189,9 @@ cudaError_t launch_select(const R0State&, int B, int N, int K, int M, const int3
                           uint16_t* scol, const long long* u0, int32_t* order, int32_t* support,
                           int32_t* slot, int32_t* out_idx, uint32_t* status, const TraceView&,
                           cudaStream_t, int I = 1);
-cudaError_t launch_select_prep(const float* C, int B, int M, int N, Scratch&, cudaStream_t);
+// gmc_select: copies the caller's clients into s.C, then the per-image total,
+// fixed-point exponent (s.fexp) and column sums (s.u0)
+cudaError_t launch_select_prep(const float* clients, int B, int M, int N, Scratch& s, cudaStream_t);
 // Whether the cluster solver's per-CTA state (a copy of every token's gain,
 // bucket and pool slot, and its share of the client rows) fits one CTA's
 // shared memory for this problem on this device; where it does not, every
