@@ -191,8 +191,8 @@ size_t carve_compress(const Dims& dm, Scratch* s, char* base, R0State* r0s = nul
   t.zn2 = c.take<float>(V * t.vzn);
   t.sigpart = c.take<float>(V * t.vsp);
   t.sigma = c.take<float>(V * t.vsg);
-  t.hgpart = c.take<double>(V * t.vhp);
-  t.HG = c.take<double>(V * t.vHG);
+  t.hgpart = c.take<float>(V * t.vhp);
+  t.HG = c.take<float>(V * t.vHG);
   t.W2 = c.take<float>(V * t.vW2);
   t.omega = c.take<float>(B * H);
   t.ebar = c.take<float>(B * N);

@@ -8,176 +8,274 @@
 // so the H x H Gram is accumulated token block by token block without ever
 // forming the (T N (r+1))-long patterns.  The mean atom norm of head h is
 // sum_t rs[h,t] / (T N) (rs from the message kernel).
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 
 namespace gmc {
 
-constexpr int HG_TC = 32;                       // queries per staged chunk
-constexpr int HG_HB = 4;                        // heads per register tile side
-
 __device__ __forceinline__ float query_weight(int t, int Tb, float wq) {
   return (t == Tb - 1 ? wq : 1.f) / ((float)(Tb - 1) + wq);
 }
 
-__device__ __forceinline__ int pair_index(int h, int g, int H) {  // h <= g, h-major
-  return h * H - h * (h - 1) / 2 + (g - h);
+// Sums n values over the warp's 32 lanes, halving the values each lane holds at
+// every step (51 shuffles for 49 values instead of 5 each).  On return v[0],
+// v[1] hold the totals number index(lane, 0) and index(lane, 1) of the n
+// (LaneSum::index; -1: none).  A fixed tree: the same on every call.
+template <int n, int o>
+struct LaneSum {
+  static constexpr int K = (n + 1) / 2;
+  static __device__ __forceinline__ void run(float* v, int lane) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int q = 0; q < K; ++q) {
+      const float hi = K + q < n ? v[K + q] : 0.f;
+      v[q] = (up ? hi : v[q]) + __shfl_xor_sync(FULL, up ? v[q] : hi, o);
+    }
+    if constexpr (o > 1) LaneSum<K, o / 2>::run(v, lane);
+  }
+  static __device__ __forceinline__ int index(int lane, int f) {
+    int i;
+    if constexpr (o > 1) i = LaneSum<K, o / 2>::index(lane, f);
+    else i = f < K ? f : -1;
+    if (i < 0) return -1;
+    i += (lane & o) ? K : 0;
+    return i < n ? i : -1;
+  }
+};
+
+// A 16-byte shared load that is issued where it stands: the weights of a pair
+// re-read their probe values instead of holding 2 HB of them in registers
+// beside the sums.
+__device__ __forceinline__ float4 lds4(unsigned a) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+               : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+               : "r"(a));
+  return v;
 }
 
-// Per block: TOK tokens (8, or 9 where that puts one image's blocks in one wave), all head
-// pairs (h <= g).  Writes the block's part
-// of the pattern Gram (an fp32 sum over its TOK tokens, stored as fp64 for
-// the cross-block sum) and W2[h,i] = sum_t nu_t A[h,t,i]^2.  The per-token
-// sums over queries are register tiles of 4 x 4 head pairs: 8 shared loads
-// feed 16 FMAs.
-template <int TOK>
-__global__ void k_head_stats(const float* __restrict__ A, const float* __restrict__ Z,
-                             const float* __restrict__ sigma, const int32_t* toff, int B, int N,
-                             int Tmax, int H, float wq, double* hgpart, int nHG, float* W2,
-                             uint32_t* status) {
+constexpr int HS_WARPS = 10;  // warps per block: the 10 head-block pairs of 28 or 32 heads
+constexpr int HS_TC = 8;      // queries of a stage per lane group (TT groups)
+// Words between the staged rows of two queries: every head block padded to HB,
+// and TT > 1 query groups of a warp on distinct banks.
+__host__ __device__ constexpr int hs_stride(int H, int HB, int TT) {
+  return (ceil_div(H, HB) * HB * (32 / TT) + 31) / 32 * 32 + (TT > 1 ? 32 / TT : 0);
+}
+
+// Pattern Gram and query-weighted squares of a group of tokens.
+//
+// Work split: a block takes TOK = 32 / TT consecutive tokens of an image; a
+// warp takes one pair of head blocks (HB heads each) and keeps the HB x HB sums
+// sum_t A[h,t,i] A[g,t,i] in registers, lane = (query t mod TT, token).  A
+// passes once through shared memory (cp.async, two stages of TC queries), laid
+// out [query][head][token], so a lane's 2 HB operands of a query lie at fixed
+// offsets from one address and feed HB^2 FMAs.  Then every lane applies its
+// token's weights Z_h . Z_g + sigma_h sigma_g and the lanes are added.  With fewer
+// pairs than HS_WARPS the queries are dealt to `ts` slices of warps.
+// TT: 1 reads whole 128-byte lines; 2 and 4 make more, smaller blocks for a
+// single small image (head_tokens).  Bound by the shared-memory and FMA issue
+// of 14 loads against 49 FMAs and the two stages' barriers.  The 4 x 4 tiles
+// over [head][query][token] stages that it replaced used half the threads and 8
+// shared loads for 16 FMAs: 656 -> 299 us at 32 ragged images of N = 1,296 (T <=
+// 256), 229 -> 110 us at N = 15,876, T = 128, 64 -> 32 us at N = 4,096, T = 128,
+// 17.1 -> 13.6 us at N = 1,296, T = 64 (H = 28).
+template <int HB, int TT>
+__global__ void __launch_bounds__(32 * HS_WARPS, HB == 8 ? 1 : 2)
+    k_head_stats(const float* __restrict__ A, const float* __restrict__ Z,
+                 const float* __restrict__ sigma, const int32_t* toff, int B, int N, int Tmax,
+                 int H, float wq, float* hgpart, int nHG, float* W2, int ts, uint32_t* status) {
   grid_dep_wait();
-  constexpr int RS = HG_TC * TOK + 2;  // row stride of a staged head: 4 rows apart land 8 banks apart
-  extern __shared__ float sm_hs[];
-  __shared__ float sgm[GMC_MAX_HEADS];  // sigma_h of the image
+  constexpr int TOK = 32 / TT, NV = HB * HB, TC = HS_TC * TT;
+  extern __shared__ __align__(16) float sm_hs[];  // [2][TC][stride], then Z [nb HB][TOK]
+  __shared__ float sgm[GMC_MAX_HEADS + 8];       // sigma_h of the image
+  __shared__ float part[HS_WARPS][NV];        // slices' sums of a pair (ts > 1)
+  __shared__ float w2s[HS_WARPS][HB][TOK];    // slices' query-weighted squares (ts > 1)
   const int b = blockIdx.y;
   const TextGeom tg = text_geom(toff, b, B, Tmax, status);
   if (tg.T == 0) return;
-  for (int h = threadIdx.x; h < H; h += blockDim.x) sgm[h] = sigma[(size_t)b * H + h];
   const int Tb = tg.T;
-  const int npairs = H * (H + 1) / 2;
-  const int nhb = (H + HG_HB - 1) / HG_HB, Hp = nhb * HG_HB;
-  const int ntiles = nhb * (nhb + 1) / 2;
-  float* Abuf = sm_hs;                          // [2][Hp][RS], rows >= H stay zero
-  float* acc = Abuf + 2 * (size_t)Hp * RS;   // [2][npairs][TOK], one per block half
-  float* w2 = acc + 2 * (size_t)npairs * TOK;  // [2][H][TOK]
-  float4* zs = reinterpret_cast<float4*>(w2 + 2 * H * TOK);  // [H][TOK] probe values
-  unsigned short* tiles = reinterpret_cast<unsigned short*>(zs + H * TOK);  // [ntiles]
-  const int i0 = blockIdx.x * TOK;
-  for (int p = threadIdx.x; p < 2 * npairs * TOK; p += blockDim.x) acc[p] = 0.f;
-  for (int p = threadIdx.x; p < 2 * H * TOK; p += blockDim.x) w2[p] = 0.f;
-  for (int p = H * RS + threadIdx.x; p < Hp * RS; p += blockDim.x) {
-    Abuf[p] = 0.f;
-    Abuf[(size_t)Hp * RS + p] = 0.f;
-  }
-  if (threadIdx.x == 0) {
-    int p = 0;
-    for (int hb = 0; hb < nhb; ++hb)
-      for (int gb = hb; gb < nhb; ++gb) tiles[p++] = (unsigned short)(hb * 256 + gb);
-  }
-  // the block's probe values Z_h[i] for every head (used by the output step)
-  for (int q = threadIdx.x; q < H * TOK; q += blockDim.x) {
-    const int h = q / TOK, i = i0 + q % TOK;
-    zs[q] = i < N ? reinterpret_cast<const float4*>(Z)[((size_t)b * H + h) * N + i]
-                  : make_float4(0.f, 0.f, 0.f, 0.f);
-  }
-  // Queries in pairs of HG_TC-chunks: both are staged, then the two halves of
-  // the block work on one chunk each into their own sums.  The TOK tokens
-  // of one (head, query) row are read as 16-byte loads when the rows of A
-  // start on 16 bytes (N % 4 == 0) and the block is not the ragged last one
-  // (the padded shared rows are not 16-byte aligned, so these go through
-  // registers); otherwise as 4-byte cp.async copies.
-  const bool vec = TOK % 4 == 0 && (N & 3) == 0 && i0 + TOK <= N;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int nb = ceil_div(H, HB), npair = nb * (nb + 1) / 2;
+  const int stride = hs_stride(H, HB, TT);
+  const int i0 = blockIdx.x * TOK, tt = lane / TOK;
+  const int i = i0 + lane % TOK;
+  const bool tok = i < N;
+  float* out = hgpart + ((size_t)b * nHG + blockIdx.x) * H * H;
+  const float nu = 1.f / ((float)(Tb - 1) + wq);
+  const float* Ab = A + (size_t)b * H * Tmax * N + i0;
+  // rows of A start on 16 bytes when N % 4 == 0 (then four tokens are all
+  // inside or all past the image); queries and tokens past the end are zero
+  const bool vec = (N & 3) == 0;
+  // thread's piece of a staged row (16 or 4 bytes) and its first (query, head) row;
+  // a step moves `rstep` rows on, without a division
+  const int pieces = vec ? TOK / 4 : TOK, pw = vec ? 4 : 1;
+  const int pv = (int)threadIdx.x % pieces * pw, r0 = (int)threadIdx.x / pieces;
+  const int rstep = 32 * HS_WARPS / pieces, dt = rstep / H, dh = rstep % H;
+  const int rt = r0 / H, rh = r0 % H;
+  const bool pin = i0 + pv < N;
   auto stage = [&](int t0, float* buf) {
-    const int tc = min(HG_TC, Tb - t0);
-    if (vec) {
-      constexpr int V = TOK / 4;  // 16-byte pieces per row
-      for (int idx = threadIdx.x; idx < H * HG_TC * V; idx += blockDim.x) {
-        const int h = idx / (HG_TC * V), tt = (idx / V) % HG_TC, v = idx % V;
-        float* dst = buf + h * RS + tt * TOK + 4 * v;
-        float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-        if (tt < tc)
-          x = *reinterpret_cast<const float4*>(A + (((size_t)b * H + h) * Tmax + t0 + tt) * N + i0 +
-                                               4 * v);
-        dst[0] = x.x;
-        dst[1] = x.y;
-        dst[2] = x.z;
-        dst[3] = x.w;
-      }
-    } else {
-      for (int idx = threadIdx.x; idx < H * HG_TC * TOK; idx += blockDim.x) {
-        const int h = idx / (HG_TC * TOK), tt = (idx / TOK) % HG_TC, ii = idx % TOK;
-        const bool in = tt < tc && i0 + ii < N;
-        const float* src = in ? A + (((size_t)b * H + h) * Tmax + t0 + tt) * N + i0 + ii : A;
-        cp_async4(buf + h * RS + tt * TOK + ii, src, in);
+    int t = rt, h = rh;
+#pragma unroll 1
+    while (t < TC) {
+      const bool in = pin && t0 + t < Tb;
+      const float* src = in ? Ab + ((size_t)h * Tmax + t0 + t) * N + pv : A;
+      float* dst = buf + t * stride + h * TOK + pv;
+      if (vec) cp_async16(dst, src, in);
+      else cp_async4(dst, src, in);
+      t += dt;
+      h += dh;
+      if (h >= H) {
+        h -= H;
+        ++t;
       }
     }
     cp_async_commit();
   };
-  const int hsz = blockDim.x / 2, half = threadIdx.x / hsz, ht = threadIdx.x % hsz;
-  float* accH = acc + (size_t)half * npairs * TOK;
-  float* w2H = w2 + (size_t)half * H * TOK;
-  for (int tp = 0; tp < Tb; tp += 2 * HG_TC) {
-    __syncthreads();  // both buffers are free
-    stage(tp, Abuf);
-    stage(tp + HG_TC, Abuf + (size_t)Hp * RS);
-    cp_async_wait<0>();
-    __syncthreads();
-    const int t0 = tp + half * HG_TC;
-    const int tc = max(0, min(HG_TC, Tb - t0));
-    const float* Ablk = Abuf + (size_t)half * Hp * RS;
-    for (int task = ht; task < ntiles * TOK; task += hsz) {
-      const int tile = task / TOK, ii = task % TOK;
-      const int hb = tiles[tile] >> 8, gb = tiles[tile] & 255;
-      const float* ah = Ablk + (size_t)hb * HG_HB * RS + ii;
-      const float* ag = Ablk + (size_t)gb * HG_HB * RS + ii;
-      float sacc[HG_HB][HG_HB];
-#pragma unroll
-      for (int u = 0; u < HG_HB; ++u)
-#pragma unroll
-        for (int v = 0; v < HG_HB; ++v) sacc[u][v] = 0.f;
-      for (int tt = 0; tt < tc; ++tt) {
-        float x[HG_HB], y[HG_HB];
-#pragma unroll
-        for (int u = 0; u < HG_HB; ++u) {
-          x[u] = ah[u * RS + tt * TOK];
-          y[u] = ag[u * RS + tt * TOK];
-        }
-#pragma unroll
-        for (int u = 0; u < HG_HB; ++u)
-#pragma unroll
-          for (int v = 0; v < HG_HB; ++v) sacc[u][v] = fmaf(x[u], y[v], sacc[u][v]);
-      }
-#pragma unroll
-      for (int u = 0; u < HG_HB; ++u)
-#pragma unroll
-        for (int v = 0; v < HG_HB; ++v) {
-          const int h = hb * HG_HB + u, g = gb * HG_HB + v;
-          if (h <= g && g < H) accH[pair_index(h, g, H) * TOK + ii] += sacc[u][v];
-        }
-    }
-    for (int q = ht; q < H * TOK; q += hsz) {
-      const int h = q / TOK, ii = q % TOK;
-      const float* ah = Ablk + h * RS;
-      float sw = 0.f;
-      for (int tt = 0; tt < tc; ++tt) {
-        const float a = ah[tt * TOK + ii];
-        sw = fmaf(query_weight(t0 + tt, Tb, wq) * a, a, sw);
-      }
-      w2H[q] += sw;
-    }
-  }
-  __syncthreads();
-  double* out = hgpart + ((size_t)b * nHG + blockIdx.x) * H * H;
-  for (int p = threadIdx.x; p < H * H; p += blockDim.x) {
-    const int h = p / H, g = p % H;
-    if (h > g) continue;
-    const int pi = pair_index(h, g, H);
-    const float sh = sgm[h], sgv = sgm[g];
-    float v = 0.f;
-    for (int ii = 0; ii < TOK; ++ii) {
-      const int i = i0 + ii;
-      if (i >= N) break;
-      const float4 zh = zs[h * TOK + ii];
-      const float4 zg = zs[g * TOK + ii];
-      const float w = fmaf(zh.x, zg.x, fmaf(zh.y, zg.y, fmaf(zh.z, zg.z, fmaf(zh.w, zg.w, sh * sgv))));
-      v = fmaf(w, acc[pi * TOK + ii] + acc[((size_t)npairs + pi) * TOK + ii], v);
-    }
-    out[h * H + g] = v;
-    out[g * H + h] = v;
-  }
+  // the tokens' probe values and the heads' mass coordinates, beside the stages
+  float4* zs = reinterpret_cast<float4*>(sm_hs + 2 * (size_t)TC * stride);
+#pragma unroll 1
   for (int q = threadIdx.x; q < H * TOK; q += blockDim.x) {
-    const int h = q / TOK, i = i0 + q % TOK;
-    if (i < N) W2[((size_t)b * H + h) * N + i] = w2[q] + w2[H * TOK + q];
+    const int h = q / TOK, k = q % TOK;
+    cp_async16(&zs[q],
+               reinterpret_cast<const float4*>(Z) + ((size_t)b * H + h) * N + min(i0 + k, N - 1));
+  }
+  for (int h = threadIdx.x; h < H; h += blockDim.x) sgm[h] = sigma[(size_t)b * H + h];
+  const int nst = ceil_div(Tb, TC);  // stages
+  // ts slices of npair warps; ts == 1: the warps walk the pairs, in one pass
+  // over the queries for every HS_WARPS pairs
+  const int slice = ts > 1 ? w / npair : 0, wp = ts > 1 ? w % npair : w;
+  const int npass = ts > 1 ? 1 : ceil_div(npair, HS_WARPS);
+  for (int pass = 0; pass < npass; ++pass) {
+    const int p = wp + pass * HS_WARPS;
+    const bool mine = p < npair && slice < ts;
+    int hb = 0, q = mine ? p : 0;  // pair p of the upper triangle, row by row
+    while (q >= nb - hb) {
+      q -= nb - hb;
+      ++hb;
+    }
+    const int gb = hb + q, h0 = hb * HB, g0 = gb * HB;
+    const bool diag = hb == gb;
+    const int nh = min(HB, H - h0), ng = min(HB, H - g0);
+    float acc[NV], w2[HB];
+#pragma unroll
+    for (int k = 0; k < NV; ++k) acc[k] = 0.f;
+#pragma unroll
+    for (int u = 0; u < HB; ++u) w2[u] = 0.f;
+    stage(0, sm_hs);
+    for (int st = 0; st < nst; ++st) {
+      if (st + 1 < nst) {
+        stage((st + 1) * TC, sm_hs + (size_t)((st + 1) & 1) * TC * stride);
+        cp_async_wait<1>();
+      } else {
+        cp_async_wait<0>();
+      }
+      __syncthreads();
+      if (mine) {
+        const int tend = min(TC, Tb - st * TC);  // staged queries of the image
+        const float* row = sm_hs + (size_t)(st & 1) * TC * stride + (slice * TT + tt) * stride +
+                           lane % TOK;
+        if (diag) {
+#pragma unroll 1
+          for (int t0 = slice * TT; t0 < tend; t0 += ts * TT, row += ts * TT * stride) {
+            const float wt = st * TC + t0 + tt == Tb - 1 ? wq * nu : nu;
+            float x[HB];
+#pragma unroll
+            for (int u = 0; u < HB; ++u) x[u] = row[(h0 + u) * TOK];
+#pragma unroll
+            for (int u = 0; u < HB; ++u) {
+              w2[u] = fmaf(wt * x[u], x[u], w2[u]);
+#pragma unroll
+              for (int v = 0; v < HB; ++v) acc[u * HB + v] = fmaf(x[u], x[v], acc[u * HB + v]);
+            }
+          }
+        } else {
+#pragma unroll 1
+          for (int t0 = slice * TT; t0 < tend; t0 += ts * TT, row += ts * TT * stride) {
+            float x[HB], y[HB];
+#pragma unroll
+            for (int u = 0; u < HB; ++u) {
+              x[u] = row[(h0 + u) * TOK];
+              y[u] = row[(g0 + u) * TOK];
+            }
+#pragma unroll
+            for (int u = 0; u < HB; ++u)
+#pragma unroll
+              for (int v = 0; v < HB; ++v) acc[u * HB + v] = fmaf(x[u], y[v], acc[u * HB + v]);
+          }
+        }
+      }
+      __syncthreads();  // the stage's buffer is free
+    }
+    if (!mine) continue;
+    if (diag) {  // sum_t nu_t A[h,t,i]^2 of the block's heads
+#pragma unroll
+      for (int u = 0; u < HB; ++u) {
+#pragma unroll
+        for (int o = TOK; o < 32; o <<= 1) w2[u] += __shfl_xor_sync(FULL, w2[u], o);
+        if (ts > 1) {
+          if (tt == 0) w2s[w][u][lane % TOK] = w2[u];
+        } else if (tt == 0 && tok && u < nh) {
+          W2[((size_t)b * H + h0 + u) * N + i] = w2[u];
+        }
+      }
+    }
+    // the token's weights (heads past H: whatever the padding holds, never written)
+    const unsigned zh0 = (unsigned)__cvta_generic_to_shared(zs + h0 * TOK + lane % TOK);
+    const unsigned zg0 = (unsigned)__cvta_generic_to_shared(zs + g0 * TOK + lane % TOK);
+#pragma unroll
+    for (int v = 0; v < HB; ++v) {
+      const float4 zg = lds4(zg0 + v * TOK * 16);
+      const float sg = sgm[g0 + v];
+#pragma unroll
+      for (int u = 0; u < HB; ++u) {
+        const float4 zh = lds4(zh0 + u * TOK * 16);
+        const float wgt =
+            fmaf(zh.x, zg.x, fmaf(zh.y, zg.y, fmaf(zh.z, zg.z, fmaf(zh.w, zg.w, sgm[h0 + u] * sg))));
+        acc[u * HB + v] = tok ? wgt * acc[u * HB + v] : 0.f;
+      }
+    }
+    LaneSum<NV, 16>::run(acc, lane);
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const int k = LaneSum<NV, 16>::index(lane, f);
+      if (k < 0) continue;
+      const int u = k / HB, v = k % HB;
+      if (u >= nh || v >= ng) continue;
+      if (ts > 1) {
+        part[w][k] = acc[f];
+      } else {
+        out[(h0 + u) * H + g0 + v] = acc[f];
+        if (!diag) out[(g0 + v) * H + h0 + u] = acc[f];
+      }
+    }
+  }
+  if (ts == 1) return;
+  // the slices in order
+  __syncthreads();
+  for (int e = threadIdx.x; e < npair * NV; e += blockDim.x) {
+    const int p = e / NV, k = e % NV;
+    int hb = 0, q = p;
+    while (q >= nb - hb) {
+      q -= nb - hb;
+      ++hb;
+    }
+    const int h = hb * HB + k / HB, g = (hb + q) * HB + k % HB;
+    if (h >= H || g >= H) continue;
+    float s = 0.f;
+    for (int x = 0; x < ts; ++x) s += part[x * npair + p][k];
+    out[h * H + g] = s;
+    if (q > 0) out[g * H + h] = s;
+  }
+  for (int e = threadIdx.x; e < nb * HB * TOK; e += blockDim.x) {
+    const int hb = e / (HB * TOK), u = e / TOK % HB, k = e % TOK;
+    const int h = hb * HB + u, tk = blockIdx.x * TOK + k;
+    if (h >= H || tk >= N) continue;
+    const int p = hb * nb - hb * (hb - 1) / 2;  // the diagonal pair of head block hb
+    float s = 0.f;
+    for (int x = 0; x < ts; ++x) s += w2s[x * npair + p][u][k];
+    W2[((size_t)b * H + h) * N + tk] = s;
   }
 }
 
@@ -196,12 +294,12 @@ __device__ __forceinline__ void warp_argbest(float& v, int& idx, bool want_max) 
 }
 
 // Farthest-first head clusters and head weights of image b from its reduced
-// pattern Gram (fp64 sums, read past L1: other blocks wrote them).  The
-// cosines, dispersions and weights are fp32: the weights enter as
+// pattern Gram (read past L1: other blocks wrote it).  The cosines, dispersions and weights are fp32: the weights enter as
 // 1 / (dispersion + head_eps) with head_eps = 0.05 by default, far above the
-// fp32 rounding of a cosine.  One block of 256 threads, one warp for the
-// centres (two heads per lane, H <= 64).
-__device__ void cluster_heads(const double* hgb, int b, int T, int N, int H, int max_clusters,
+// fp32 rounding of a cosine.  One block, one warp for the centres (two heads
+// per lane, H <= 64).  A chain of short steps between barriers: with one view
+// the Gram is read once into shared memory, all loads in flight together.
+__device__ void cluster_heads(const float* hgb, int b, int T, int N, int H, int max_clusters,
                               float head_eps, float* omega, const TraceView& tv, float* sm,
                               const ViewGrams& vg) {
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -223,9 +321,9 @@ __device__ void cluster_heads(const double* hgb, int b, int T, int N, int H, int
     for (int h = threadIdx.x; h < H; h += blockDim.x) {
       float a = 0.f;
       for (int v = 0; v < vg.n; ++v) {
-        const double* hv = vg.HG[v] + (size_t)b * HE;
-        const float m = (float)__ldcg(&hv[H * H + h]) / TN;
-        if (m > 0.f) a += vg.beta[v] * (float)__ldcg(&hv[h * H + h]) / (m * m);
+        const float* hv = vg.HG[v] + (size_t)b * HE;
+        const float m = __ldcg(&hv[H * H + h]) / TN;
+        if (m > 0.f) a += vg.beta[v] * __ldcg(&hv[h * H + h]) / (m * m);
       }
       pre[h] = a > 0.f ? sqrtf(a) : 0.f;
       dot[h] = a > 0.f ? 1.f / sqrtf(a) : 0.f;
@@ -235,25 +333,25 @@ __device__ void cluster_heads(const double* hgb, int b, int T, int N, int H, int
       const int h = p / H, g = p % H;
       float x = 0.f;
       for (int v = 0; v < vg.n; ++v) {
-        const double* hv = vg.HG[v] + (size_t)b * HE;
-        const float mh = (float)__ldcg(&hv[H * H + h]) / TN, mg = (float)__ldcg(&hv[H * H + g]) / TN;
-        if (mh > 0.f && mg > 0.f) x += vg.beta[v] * (float)__ldcg(&hv[p]) / (mh * mg);
+        const float* hv = vg.HG[v] + (size_t)b * HE;
+        const float mh = __ldcg(&hv[H * H + h]) / TN, mg = __ldcg(&hv[H * H + g]) / TN;
+        if (mh > 0.f && mg > 0.f) x += vg.beta[v] * __ldcg(&hv[p]) / (mh * mg);
       }
       cs[p] = x * dot[h] * dot[g];
     }
     __syncthreads();
   } else {
+    for (int p = threadIdx.x; p < H * H; p += blockDim.x) cs[p] = __ldcg(&hgb[p]);
+    for (int h = threadIdx.x; h < H; h += blockDim.x) inv[h] = __ldcg(&hgb[H * H + h]);
+    __syncthreads();
     for (int h = threadIdx.x; h < H; h += blockDim.x) {
-      const float a = (float)__ldcg(&hgb[h * H + h]);
-      const float mean = (float)__ldcg(&hgb[H * H + h]) / TN;  // sum_t rs / (T N)
+      const float a = cs[h * H + h];
+      const float mean = inv[h] / TN;  // sum_t rs / (T N)
       pre[h] = (mean > 0.f && a > 0.f) ? sqrtf(a) / mean : 0.f;
       dot[h] = a > 0.f ? 1.f / sqrtf(a) : 0.f;  // 1 / ||U_h||, 0 for a zero pattern
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < H * H; p += blockDim.x) {
-      const int h = p / H, g = p % H;
-      cs[p] = (float)__ldcg(&hgb[p]) * dot[h] * dot[g];
-    }
+    for (int p = threadIdx.x; p < H * H; p += blockDim.x) cs[p] = cs[p] * dot[p / H] * dot[p % H];
     __syncthreads();
   }
   const int nc = min(max_clusters, H);
@@ -354,40 +452,99 @@ __device__ void cluster_heads(const double* hgb, int b, int T, int N, int H, int
   }
 }
 
-// The pattern Gram of image blockIdx.y: sum of the token-block partials, one
-// warp per entry, lanes over the blocks (fixed order, so the sum is
-// reproducible); further warps sum every head's atom norms sum_t rs[h,t] (rs
-// in nRS parts per query).  HG[b] holds the H*H Gram followed by the H
-// atom-norm totals.  The image's last block to finish (ticket zeroed with the
-// status word) clusters the heads.
-__global__ void __launch_bounds__(256) k_hg_reduce(const double* __restrict__ hgpart, int nHG,
-                                                     int B, int N, int H,
-                                                     const float* __restrict__ rs, int nRS,
-                                                     const int32_t* toff, int Tmax, double* HG,
-                                                     uint32_t* tick, int max_clusters,
-                                                     float head_eps, float* omega, TraceView tv,
-                                                     int cluster, const ViewGrams vg,
-                                                     uint32_t* status) {
+// A sum held as hi + lo, every addition's rounding error kept in lo (Knuth's
+// two-sum): about 48 bits, on the fp32 pipe.  fp64 additions run at a small
+// fraction of its rate on this GPU: with them the reduction below took 15.3
+// instead of 10.3 us at the 162 partials of N = 1,296, H = 28.
+struct Sum2 {
+  float hi = 0.f, lo = 0.f;
+  __device__ __forceinline__ void add(float x) {
+    const float t = hi + x, z = t - hi;
+    lo += (hi - (t - z)) + (x - z);
+    hi = t;
+  }
+  __device__ __forceinline__ void add(const Sum2& o) {
+    add(o.hi);
+    lo += o.lo;
+  }
+  // the sum over the lanes that differ in the bits below `n` (a fixed tree)
+  __device__ __forceinline__ void reduce(int n) {
+    for (int o = n / 2; o > 0; o >>= 1) {
+      Sum2 y;
+      y.hi = __shfl_xor_sync(FULL, hi, o);
+      y.lo = __shfl_xor_sync(FULL, lo, o);
+      add(y);
+    }
+  }
+  __device__ __forceinline__ float value() const { return hi + lo; }
+};
+
+// The pattern Gram of image blockIdx.y: the token blocks' partials added up.
+// The first gridDim.x - nrb blocks take 32 Gram entries each, one per lane (a
+// warp reads one line of a partial), and their warps every HR_WARPS-th partial,
+// twelve loads in flight (one round trip for the 162 partials of N = 1,296).
+// The last nrb blocks sum every head's atom norms sum_t rs[h,t] (rs in nRS
+// parts per query), a warp per head.  HG[b] holds the H*H Gram followed by the
+// H atom-norm totals.  The image's last block to finish (ticket zeroed with
+// the status word) clusters the heads.
+constexpr int HR_WARPS = 16;
+__global__ void __launch_bounds__(32 * HR_WARPS)
+    k_hg_reduce(const float* __restrict__ hgpart, int nHG, int B, int N, int H,
+                const float* __restrict__ rs, int nRS, const int32_t* toff, int Tmax, float* HG,
+                uint32_t* tick, int max_clusters, float head_eps, float* omega, TraceView tv,
+                int cluster, const ViewGrams vg, int nrb, uint32_t* status) {
   grid_dep_wait();
   extern __shared__ float sm_hc[];
+  __shared__ Sum2 psum[HR_WARPS][33];
   __shared__ int last;
-  const int lane = threadIdx.x & 31, b = blockIdx.y;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, b = blockIdx.y;
   const int HH = H * H, HE = HH + H;
   const TextGeom tg = text_geom(toff, b, B, Tmax, status);
   if (tg.T == 0) return;  // uniform over the image
-  const int p = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-  if (p < HE) {
-    double s = 0.0;
+  const int ngb = gridDim.x - nrb;
+  if ((int)blockIdx.x < ngb) {
+    const int p = blockIdx.x * 32 + lane;
+    const float* src = hgpart + (size_t)b * nHG * HH + p;
+    Sum2 s;
     if (p < HH) {
-      for (int k = lane; k < nHG; k += 32) s += hgpart[((size_t)b * nHG + k) * HH + p];
-    } else {
-      const int h = p - HH;
-      const float* r = rs + ((size_t)b * H + h) * nRS * Tmax;
-      for (int k = lane; k < nRS * Tmax; k += 32)
-        if (k % Tmax < tg.T) s += r[k];
+      constexpr int U = 12;
+      for (int k0 = w; k0 < nHG; k0 += U * HR_WARPS) {
+        float v[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int k = k0 + u * HR_WARPS;
+          v[u] = k < nHG ? src[(size_t)k * HH] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < U; ++u) s.add(v[u]);
+      }
     }
-    s = warp_sum(s);
-    if (lane == 0) HG[(size_t)b * HE + p] = s;
+    psum[w][lane] = s;
+    __syncthreads();
+    // half-warp: one entry, lane = source warp
+    const int pe = 2 * w + (lane >> 4), p2 = blockIdx.x * 32 + pe;
+    Sum2 t = psum[lane & 15][pe];
+    t.reduce(HR_WARPS);
+    if ((lane & 15) == 0 && p2 < HH) HG[(size_t)b * HE + p2] = t.value();
+  } else {
+    const int h = (blockIdx.x - ngb) * HR_WARPS + w;
+    if (h < H) {
+      Sum2 s;
+      const float* r = rs + ((size_t)b * H + h) * nRS * Tmax;
+      const int n = nRS * tg.T;  // (part, query) pairs, eight per lane in flight
+      for (int k0 = lane; k0 < n; k0 += 32 * 8) {
+        float v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = k0 + 32 * u;
+          v[u] = k < n ? r[(size_t)(k / tg.T) * Tmax + k % tg.T] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) s.add(v[u]);
+      }
+      s.reduce(32);
+      if (lane == 0) HG[(size_t)b * HE + HH + h] = s.value();
+    }
   }
   __threadfence();
   __syncthreads();
@@ -398,18 +555,22 @@ __global__ void __launch_bounds__(256) k_hg_reduce(const double* __restrict__ hg
   cluster_heads(HG + (size_t)b * HE, b, tg.T, N, H, max_clusters, head_eps, omega, tv, sm_hc, vg);
 }
 
-// Dynamic shared memory of k_head_stats for H heads: both staged query
-// chunks, both halves' pair sums and query-weighted squares, the probe values
-// and the tile list.
-static size_t head_stats_smem(int H, int tok) {
-  const int npairs = H * (H + 1) / 2;
-  const int nhb = (H + HG_HB - 1) / HG_HB;
-  const int rs = HG_TC * tok + 2;
-  return sizeof(float) * (2 * (size_t)nhb * HG_HB * rs + 2 * (size_t)npairs * tok + 2 * H * tok) +
-         sizeof(float4) * H * tok + sizeof(unsigned short) * (nhb * (nhb + 1) / 2) + 16;
+namespace {
+// Heads per register block: the one that pads H least (28 -> 7, 32 -> 8), the
+// larger among equals.
+int head_block(int H) {
+  int best = 8;
+  for (int hb : {7, 4})
+    if (ceil_div(H, hb) * hb < ceil_div(H, best) * best) best = hb;
+  return best;
 }
+}  // namespace
 
+// Tokens per head-statistics block.  32 (whole lines) once those blocks fill
+// the SMs twice over; below that smaller blocks keep more SMs busy: at one
+// image of N = 1,296 the 162 blocks of 8 tokens, at N = 4,096 the 256 of 16.
 int head_tokens(int B, int N, int H) {
+  (void)H;
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
@@ -419,36 +580,43 @@ int head_tokens(int B, int N, int H) {
       sms = 152;
     }
   }
-  const long long b8 = (long long)B * ceil_div(N, 8), b9 = (long long)B * ceil_div(N, 9);
-  return b8 > sms && b9 <= sms && head_stats_smem(H, 9) <= 227 * 1024 ? 9 : 8;
+  for (int tok : {32, 16})
+    if ((long long)B * ceil_div(N, tok) >= (tok == 32 ? 2LL : 1LL) * sms) return tok;
+  return 8;
 }
 
-// Whether the head statistics of H heads fit one block's shared memory
-// (227 KB on sm_103a): H <= 56.
-bool heads_supported(int H) { return H >= 1 && head_stats_smem(H, 8) <= 227 * 1024; }
+// The documented head limit of the library (include/gmc.h).
+bool heads_supported(int H) { return H >= 1 && H <= 56; }
 
 cudaError_t launch_heads(const Dims& dm, const gmc_params& p, Scratch& s, const TraceView& tv,
                          cudaStream_t st, int cluster, const ViewGrams* views) {
   const int H = dm.H;
-  const int tok = s.hgtok;
-  const size_t smem = head_stats_smem(H, tok);
-  const void* kf = tok == 9 ? (const void*)k_head_stats<9> : (const void*)k_head_stats<8>;
-  cudaError_t e = set_smem_limit(kf, smem);
-  if (e != cudaSuccess) return e;
-  if (tok == 9)
-    launch_k(k_head_stats<9>, dim3(s.nHG, dm.B), 512, smem, st, 1, s.A, s.Z, s.sigma, dm.toff, dm.B,
-             dm.N, dm.T, H, p.terminal_q_weight, s.hgpart, s.nHG, s.W2, s.status);
-  else
-    launch_k(k_head_stats<8>, dim3(s.nHG, dm.B), 512, smem, st, 1, s.A, s.Z, s.sigma, dm.toff, dm.B,
-             dm.N, dm.T, H, p.terminal_q_weight, s.hgpart, s.nHG, s.W2, s.status);
+  cudaError_t e;
+  const int hb = head_block(H), nb = ceil_div(H, hb), npair = nb * (nb + 1) / 2;
+  // few pairs of head blocks: the queries in slices, one per group of warps
+  const int ts = std::max(1, HS_WARPS / npair);
+  const int tt = 32 / s.hgtok;
+  const size_t smem = sizeof(float) * 2 * (size_t)HS_TC * tt * hs_stride(H, hb, tt) +
+                      sizeof(float4) * (size_t)nb * hb * s.hgtok;
+  auto kern = [&]() {
+    switch (hb) {
+      case 7: return s.hgtok == 32 ? k_head_stats<7, 1> : s.hgtok == 16 ? k_head_stats<7, 2> : k_head_stats<7, 4>;
+      case 4: return s.hgtok == 32 ? k_head_stats<4, 1> : s.hgtok == 16 ? k_head_stats<4, 2> : k_head_stats<4, 4>;
+      default: return s.hgtok == 32 ? k_head_stats<8, 1> : s.hgtok == 16 ? k_head_stats<8, 2> : k_head_stats<8, 4>;
+    }
+  }();
+  if ((e = set_smem_limit((const void*)kern, smem)) != cudaSuccess) return e;
+  launch_k(kern, dim3(s.nHG, dm.B), 32 * HS_WARPS, smem, st, 1, s.A, s.Z, s.sigma, dm.toff, dm.B,
+           dm.N, dm.T, H, p.terminal_q_weight, s.hgpart, s.nHG, s.W2, ts, s.status);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const size_t smem2 = sizeof(float) * ((size_t)H * H + 3 * H + 2 * GMC_MAX_HEADS) +
                        sizeof(int) * (H + 2 * GMC_MAX_HEADS);
   if ((e = set_smem_limit((const void*)k_hg_reduce, smem2)) != cudaSuccess) return e;
-  launch_k(k_hg_reduce, dim3(ceil_div(H * H + H, 8), dm.B), 256, smem2, st, 1,
-           (const double*)s.hgpart, s.nHG, dm.B, dm.N, H, (const float*)s.rs, s.nRS, dm.toff, dm.T,
+  const int nrb = ceil_div(H, HR_WARPS);
+  launch_k(k_hg_reduce, dim3(ceil_div(H * H, 32) + nrb, dm.B), 32 * HR_WARPS, smem2, st, 1,
+           (const float*)s.hgpart, s.nHG, dm.B, dm.N, H, (const float*)s.rs, s.nRS, dm.toff, dm.T,
            s.HG, s.tick3, p.max_head_clusters, p.head_eps, s.omega, tv, cluster,
-           views ? *views : ViewGrams{}, s.status);
+           views ? *views : ViewGrams{}, nrb, s.status);
   return cudaGetLastError();
 }
 

@@ -64,7 +64,7 @@ struct ViewRows {
 // HG[v] holds [B][H*H + H] (Gram, then sum_t rs[h,t] per head).
 struct ViewGrams {
   int n;
-  const double* HG[MAX_VIEWS];
+  const float* HG[MAX_VIEWS];
   float beta[MAX_VIEWS];
 };
 
@@ -90,8 +90,8 @@ struct Scratch {
   uint32_t* tick3;   // [B]            last-block tickets of the head-Gram reduction (same)
   float* gatev;      // [B][4]         Delta_bar, s_x, mean message energy
   float* sigma;      // [B][H]         mass coordinate sigma_h
-  double* hgpart;    // [B][nHG][H*H]  block partials of the head-pattern Gram
-  double* HG;        // [B][H*H + H]   head-pattern Gram, then sum_t rs[h,t] per head
+  float* hgpart;     // [B][nHG][H*H]  block partials of the head-pattern Gram
+  float* HG;         // [B][H*H + H]   head-pattern Gram, then sum_t rs[h,t] per head
   float* W2;         // [B][H][N]      sum_t nu_t A[h,t,i]^2
   float* omega;      // [B][H]
   float* ebar;       // [B][N]  message energy e_i (the assignment divides by its mean)
@@ -130,8 +130,7 @@ struct Scratch {
 };
 
 constexpr int ROWS_PER_BLOCK = 8;  // rownorm / probe / client builder blocks
-int head_tokens(int B, int N, int H);  // tokens per head-statistics block: 8, or 9 where
-                                      // that puts every block in one wave
+int head_tokens(int B, int N, int H);  // tokens per head-statistics block: 8, 16 or 32
 constexpr int ASSIGN_WARPS = 16;   // warps per assignment block (32 tokens, one per lane)
 int assign_blocks(int N);          // assignment blocks per image
 constexpr int PROBE_TOK = 32;       // tokens per probe block
