@@ -246,7 +246,7 @@ R0State carve_round0(Carver& c, size_t B, size_t N, size_t M) {
   r.s0 = c.take<long long>(B * GMC_MAX_POOL);
   r.u1 = c.take<long long>(B * N);
   r.u2 = c.take<long long>(B * N);
-  r.ugain = sparse_gpu_rounds((int)N) % 2 == 0 ? r.u1 : r.u2;
+  r.ugain = nullptr;
   r.bcov = c.take<float>(B * M);
   r.cnt = c.take<int32_t>(B * M);
   r.fv = c.take<long long>(B * 4);
@@ -677,7 +677,7 @@ static int compress_impl(const gmc_problem* prob, const gmc_params* params,
       g_launches += 1;
     }
   } else {
-    GMC_STAGE("rounds_gpu", 3 + 3 * sparse_gpu_rounds(N),
+    GMC_STAGE("rounds_gpu", 3 + 3 * sparse_gpu_rounds(N, dm.B, Ke, p.batch_b, dm.I),
               launch_round0(r0, dm.B, N, Ke, dm.M, dm.toff, HV, T, LS, p, fx, nullptr, s.C,
                             s.scol, s.u0, s.order, s.status, tv, st, dm.I));
     GMC_STAGE("select", 1,
@@ -942,7 +942,7 @@ int gmc_select(const float* clients, int B, int M, int N, int K, const gmc_param
                         s.order, s.status, tv, st));
   GMC_TRY(launch_select(r0, B, N, K, M, nullptr, 0, 1, 0, p, 0, s.fexp, s.C, s.scol, s.u0,
                         s.order, s.support, s.slot, out_idx, s.status, tv, st));
-  g_launches += 7 + 3 * sparse_gpu_rounds(N);
+  g_launches += 7 + 3 * sparse_gpu_rounds(N, B, K, p.batch_b, 1);
   return GMC_OK;
 }
 

@@ -8,7 +8,7 @@
 //               b_m = max over the batch, and the row's survivors
 //               {i : Cbar_mi > b_m} compacted in place; the next round's gains
 //               are summed in fixed point (global atomics).
-// The next sparse_gpu_rounds(N) rounds run the same three steps over the survivor
+// The next sparse_gpu_rounds() rounds run the same three steps over the survivor
 // lists left in place by the previous round (row m: values Cbar[m][0..cnt_m),
 // tokens scol[m][0..cnt_m), ascending):
 //   k_rg_pool   the pool of the current gains among the unselected tokens;
@@ -646,7 +646,8 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   if ((e = set_smem_limit((const void*)k_rg_rho<ROWS>, rsm)) != cudaSuccess) return e;
   const size_t gsm = sizeof(unsigned long long) * (size_t)N + (size_t)N;
   if ((e = set_smem_limit((const void*)k_rg_filter<ROWS>, gsm)) != cudaSuccess) return e;
-  for (int rr = 1; rr <= sparse_gpu_rounds(N); ++rr) {
+  const int rounds = sparse_gpu_rounds(N, B, K, p.batch_b, I);
+  for (int rr = 1; rr <= rounds; ++rr) {
     long long* ucur = rr % 2 == 1 ? r0.u1 : r0.u2;
     long long* unext = rr % 2 == 1 ? r0.u2 : r0.u1;
     launch_k(k_rg_pool, B, 512, psm, st, 1, (const long long*)ucur, unext, B, N, K, P,
@@ -665,12 +666,13 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   return cudaSuccess;
 }
 
-cudaError_t launch_round0(const R0State& r0, int B, int N, int K, int M, const int32_t* toff,
+cudaError_t launch_round0(R0State& r0, int B, int N, int K, int M, const int32_t* toff,
                           int H, int T, int L2, const gmc_params& p, int fx_exp,
                           const int32_t* fexp, float* C, uint16_t* scol, const long long* u0,
                           int32_t* order, uint32_t* status, const TraceView& tv,
                           cudaStream_t st, int I) {
   const int P = p.pool_mult * p.batch_b;
+  r0.ugain = sparse_gpu_rounds(N, B, K, p.batch_b, I) % 2 == 0 ? r0.u1 : r0.u2;
   cudaError_t e;
   const size_t smem =
       sizeof(long long) * (size_t)N + sizeof(int) * (sel::HBINS + N + 32 + 8 + sel::CBINS + P) +

@@ -154,12 +154,21 @@ cudaError_t launch_build_clients(const Dims&, const gmc_params&, int fx_exp, Scr
                                  const ViewRows& views, const float* app,
                                  cudaStream_t, int part = 0);
 // State left by the first (dense) selection round, run over the whole GPU.
-// Rounds of the solver run on the whole GPU before the cluster kernel takes
-// over: the dense first round, then sparse_gpu_rounds(N) sparse rounds (an
-// even count: the cluster kernel starts from the gains in u1).  Larger images
-// keep more survivors per round, so more rounds stay on the whole GPU; the
-// counts were chosen by measurement.
-__host__ __device__ inline int sparse_gpu_rounds(int N) { return N > 2048 ? 8 : 4; }
+// Sparse rounds of the solver run on the whole GPU, after the dense first one
+// and before the cluster kernel takes over: until the survivor lists fit the
+// cluster's shared memory, and no more than the budget has rounds left.  Larger
+// images keep more survivors, and a batch leaves fewer CTAs per image.  A round
+// costs about 21 us on the whole GPU and 9-18 us in a cluster that holds its
+// lists, but 50 us and more in one that does not (they stay in global memory).
+// Measured calls by sparse rounds on the GPU: N = 1,296: 0 525 us, 1 320, 2 327,
+// 4 328; N = 2,592: 2 937, 3 956, 4 716, 5 686, 8 709; N = 4,096: 6 924, 8 889, 10
+// 907; 32 images of N = 1,296: 1 4.31 ms, 2 4.15, 4 3.99, 6 3.98.
+inline int sparse_gpu_rounds(int N, int B, int K, int batch_b, int images) {
+  const int base = (N > 3072 ? 8 : (N > 1536 ? 5 : 1)) + (B > 38 ? 5 : (B > 19 ? 4 : (B > 9 ? 2 : 0)));
+  const int left = K - (images > 1 ? images : batch_b);
+  const int most = left > 0 ? (left + batch_b - 1) / batch_b : 0;
+  return base < most ? base : most;
+}
 
 // per-image words of R0State::info
 constexpr int INFO_W = 8;
@@ -174,12 +183,12 @@ struct R0State {
   long long* s0;   // [B][P]  scores of the current round (fixed point)
   long long* u1;   // [B][N]  gains (fixed point), written by rounds 0, 2, ...
   long long* u2;   // [B][N]  gains written by rounds 1, 3, ...
-  long long* ugain;  // u1 or u2: the gains the cluster kernel starts from
+  long long* ugain;  // u1 or u2: the gains the cluster kernel starts from (set by launch_round0)
   float* bcov;     // [B][M]  coverage b_m after the last whole-GPU round
   int32_t* cnt;    // [B][M]  survivors per row (lists in place over Cbar / scol)
   long long* fv;   // [B][4]  F_b(V) per bank (fixed point)
 };
-cudaError_t launch_round0(const R0State&, int B, int N, int K, int M, const int32_t* toff, int H,
+cudaError_t launch_round0(R0State&, int B, int N, int K, int M, const int32_t* toff, int H,
                           int T, int L2, const gmc_params&, int fx_exp, const int32_t* fexp,
                           float* C, uint16_t* scol, const long long* u0, int32_t* order,
                           uint32_t* status, const TraceView&, cudaStream_t, int I = 1);

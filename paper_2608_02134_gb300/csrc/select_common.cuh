@@ -19,6 +19,24 @@ __device__ __forceinline__ unsigned lanemask_lt() {
   return m;
 }
 
+// 64-bit sums in shared memory as three 32-bit limbs of LIMB bits.  A 64-bit
+// shared-memory addition is a compare-and-swap loop that retries once for every
+// other thread on the same word, and popular tokens are on many rows; 32-bit
+// additions without a result are native.  A word takes up to LIMB_ADDS values
+// below 2^63 before its limbs are put together.
+constexpr int LIMB = 21;
+constexpr int LIMB_ADDS = (1 << (32 - LIMB)) - 1;
+__device__ __forceinline__ void limb_add(uint32_t* w, int stride, unsigned long long v) {
+  constexpr unsigned M = (1u << LIMB) - 1;
+  atomicAdd(w, (unsigned)v & M);
+  atomicAdd(w + stride, (unsigned)(v >> LIMB) & M);
+  atomicAdd(w + 2 * stride, (unsigned)(v >> (2 * LIMB)));
+}
+__device__ __forceinline__ unsigned long long limb_value(const uint32_t* w, int stride) {
+  return (unsigned long long)w[0] + ((unsigned long long)w[stride] << LIMB) +
+         ((unsigned long long)w[2 * stride] << (2 * LIMB));
+}
+
 // Monotone 11-bit bucket of a positive 64-bit gain: exponent and 5 mantissa bits.
 __device__ __forceinline__ int gain_bucket(long long u) {
   const int lz = __clzll(u);                                      // 1..63 for 0 < u < 2^63
