@@ -29,14 +29,13 @@
 namespace gmc {
 
 namespace {
-// Warps per block of the responsibility and filter kernels (ROWS, a template
-// parameter: 16 for one image, 8 for a batch; the responsibility kernels take
-// one row per warp).  The filters take `rpw` rows per warp (rows m0 + w +
-// ROWS * i).  More rows
-// per block mean fewer global atomics for the next gains (one per block and
-// column) but less parallelism: one row per warp is faster while the blocks
-// fit on the GPU at once, four when there are many more blocks than that.
-int filter_rows_per_warp(int B, int M, int rows) {
+// The responsibility and filter kernels have ROWS warps a block (a template
+// parameter: 16 for one image, 8 for a batch) and take `rpw` consecutive rows per
+// warp.  Every block pays for tables of N tokens, and the filters end with a global
+// addition per touched token, so a batch takes more rows per block; the next row
+// is loaded while one is worked on.  At most eight: with 32 the images of a ragged
+// batch that have the most rows ran alone at the end.
+int rows_per_warp(int B, int M, int rows) {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
@@ -46,10 +45,29 @@ int filter_rows_per_warp(int B, int M, int rows) {
       sms = 152;
     }
   }
-  const long long blocks = (long long)B * ceil_div(M, rows);
-  return blocks > 32LL * sms ? 4 : 1;
+  const long long rpw = (long long)B * M / ((long long)rows * 4 * sms);
+  return rpw < 1 ? 1 : (rpw > 8 ? 8 : (int)rpw);
 }
-}
+
+// The first 64 entries of a row's survivor list, loaded ahead of their use by the
+// kernels with several rows per warp (a batch).  With one row per warp there is
+// nothing to load ahead of, and the registers cost a block per SM (document page:
+// the eight responsibility launches 71 us without, 91 us with them).
+template <bool AHEAD>
+struct RowHead {
+  static constexpr int U = AHEAD ? 2 : 0;
+  int j[2];
+  float v[2];
+  __device__ __forceinline__ void load(const float* vals, const uint16_t* cols, int n, int lane) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int e = 32 * u + lane;
+      j[u] = e < n ? (int)cols[e] : -1;
+      v[u] = e < n ? vals[e] : 0.f;
+    }
+  }
+};
+}  // namespace
 
 __global__ void __launch_bounds__(512) k_r0_pool(const long long* __restrict__ u0, int B, int N,
                                                    int P, const int32_t* toff, int Tmax, int I,
@@ -131,40 +149,54 @@ __global__ void __launch_bounds__(512) k_r0_pool(const long long* __restrict__ u
   }
 }
 
+// A lane keeps the sums of its pool slots in registers over the warp's rows; the
+// warps are added in shared memory once (8 warps adding every row's 64 scores to
+// the same shared words took a batch of 32 images 115 us, R0RHO us now).
 template <int ROWS>
 __global__ void __launch_bounds__(32 * ROWS) k_r0_rho(
     const float* __restrict__ C, int B, int N, int Mstride, int H, int L2, const int32_t* toff,
     int Tmax, int uniform_rows, const int32_t* __restrict__ pool0, const int32_t* __restrict__ info,
-    int P, float resp_temp, float resp_eps, int fx_exp, const int32_t* fexp, int I, long long* s0) {
+    int P, float resp_temp, float resp_eps, int fx_exp, const int32_t* fexp, int I, int rpw,
+    long long* s0) {
   grid_dep_wait();
   if (I > 1) return;  // a seed round: no responsibilities
-  __shared__ int pool[GMC_MAX_POOL];
-  __shared__ long long sblk[GMC_MAX_POOL];
+  constexpr int U = GMC_MAX_POOL / 32;
+  __shared__ unsigned long long sblk[ROWS][GMC_MAX_POOL];
   const int b = blockIdx.y;
   const int Pt = info[b * INFO_W];
   if (Pt == 0) return;
   int Mb = Mstride;
   if (!uniform_rows) Mb = H * text_geom(toff, b, B, Tmax, nullptr).T + N + L2;
-  const int m0 = blockIdx.x * ROWS;
+  const int m0 = blockIdx.x * ROWS * rpw;
   if (m0 >= Mb) return;
   const float fxs = ldexpf(1.f, fexp ? fexp[b] : fx_exp);
-  for (int k = threadIdx.x; k < P; k += blockDim.x) {
-    pool[k] = pool0[(size_t)b * P + k];
-    sblk[k] = 0;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int pool[U];
+  unsigned long long acc[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) {
+    const int k = lane + 32 * u;
+    pool[u] = k < Pt ? pool0[(size_t)b * P + k] : -1;
+    acc[u] = 0;
   }
-  __syncthreads();
-  const int lane = threadIdx.x & 31, m = m0 + (threadIdx.x >> 5);
-  if (m < Mb) {
-    const float* row = C + ((size_t)b * Mstride + m) * N;
-    float Rd[GMC_MAX_POOL / 32];
+  const int mw = m0 + w * rpw, nr = min(rpw, Mb - mw);  // this warp's rows
+  const float* row = C + ((size_t)b * Mstride + mw) * N;
+  float next[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) next[u] = nr > 0 && pool[u] >= 0 ? row[pool[u]] : 0.f;
+  for (int ir = 0; ir < nr; ++ir) {
+    float Rd[U];
+    row += N;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {  // b = 0: the residual is the client value
+      Rd[u] = next[u];
+      next[u] = ir + 1 < nr && pool[u] >= 0 ? row[pool[u]] : 0.f;
+    }
     float rmax = 0.f;
     int npool = 0;
 #pragma unroll
-    for (int u = 0; u < GMC_MAX_POOL / 32; ++u) {
-      const int k = lane + 32 * u;
-      Rd[u] = k < Pt ? row[pool[k]] : 0.f;  // b = 0: the residual is the client value
+    for (int u = 0; u < U; ++u)
       if (Rd[u] > 0.f) { rmax = fmaxf(rmax, Rd[u]); ++npool; }
-    }
     rmax = warp_max(rmax);
     npool = warp_sum_int(npool);
     if (npool > 0) {
@@ -172,22 +204,28 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_rho(
       // exponential is at most 1, whatever resp_temp
       const float tau = resp_temp * rmax + resp_eps;
       const float e0 = expf(-rmax / tau);  // a pool token with R = 0
-      float z = 0.f;
+      float ex[U], z = 0.f;
 #pragma unroll
-      for (int u = 0; u < GMC_MAX_POOL / 32; ++u)
-        if (Rd[u] > 0.f) z += expf((Rd[u] - rmax) / tau);
+      for (int u = 0; u < U; ++u) {
+        ex[u] = Rd[u] > 0.f ? expf((Rd[u] - rmax) / tau) : 0.f;
+        z += ex[u];
+      }
       z = warp_sum(z) + (float)(Pt - npool) * e0;
       const float invz = 1.f / z;
 #pragma unroll
-      for (int u = 0; u < GMC_MAX_POOL / 32; ++u)
-        if (Rd[u] > 0.f)
-          atomicAdd((unsigned long long*)&sblk[lane + 32 * u],
-                    (unsigned long long)to_fix(expf((Rd[u] - rmax) / tau) * invz * Rd[u], fxs));
+      for (int u = 0; u < U; ++u)
+        if (Rd[u] > 0.f) acc[u] += (unsigned long long)to_fix(ex[u] * invz * Rd[u], fxs);
     }
   }
+#pragma unroll
+  for (int u = 0; u < U; ++u) sblk[w][lane + 32 * u] = acc[u];
   __syncthreads();
-  for (int k = threadIdx.x; k < Pt; k += blockDim.x)
-    if (sblk[k]) atomicAdd((unsigned long long*)&s0[(size_t)b * P + k], (unsigned long long)sblk[k]);
+  for (int k = threadIdx.x; k < Pt; k += blockDim.x) {
+    unsigned long long v = 0;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) v += sblk[q][k];
+    if (v) atomicAdd((unsigned long long*)&s0[(size_t)b * P + k], v);
+  }
 }
 
 template <int ROWS>
@@ -202,8 +240,9 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_filter(
   __shared__ long long sc[GMC_MAX_POOL];
   __shared__ int batch[GMC_MAX_POOL];
   __shared__ long long fb[3];
-  // the block's contributions to the next gains, one global atomic per column at the end
-  extern __shared__ unsigned long long uacc[];  // [N]
+  // the warps' tiles, then the block's contributions to the next gains (N <= 8,192),
+  // one global addition per column at the end
+  extern __shared__ float4 sm_r0f[];
   const int b = blockIdx.y;
   const int Pt = info[b * INFO_W];
   if (Pt == 0) return;
@@ -221,7 +260,9 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_filter(
     sc[k] = s0[(size_t)b * P + k];
   }
   if (threadIdx.x < 3) fb[threadIdx.x] = 0;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) uacc[j] = 0;
+  constexpr int TILE = sel::ROW_STEP / 4;
+  const sel::GainSums<true> sums{reinterpret_cast<uint32_t*>(sm_r0f + ROWS * TILE), N};
+  sums.clear();
   __syncthreads();
   {
     const int lane = threadIdx.x & 31, gl = lane & 7;
@@ -246,7 +287,7 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_filter(
   }
   const int lane = threadIdx.x & 31;
   for (int ir = 0; ir < rpw; ++ir) {
-    const int m = m0 + (threadIdx.x >> 5) + ROWS * ir;
+    const int m = m0 + (threadIdx.x >> 5) * rpw + ir;
     if (m >= Mb) break;
     float* vals = C + ((size_t)b * Mstride + m) * N;
     uint16_t* cols = scol + ((size_t)b * Mstride + m) * N;
@@ -254,83 +295,25 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_filter(
     for (int t = lane; t < nb; t += 32) bnew = fmaxf(bnew, vals[batch[t]]);
     bnew = warp_max(bnew);
     const long long fb_new = to_fix(bnew, fxs);
-    int w = 0;
-    float rowmax = 0.f;
-    const unsigned lt = sel::lanemask_lt();
-    if ((N & 3) == 0) {
-      // 32 lanes x 8 float4 = 1024 columns per step; all loads issued before any
-      // survivor is written back in place
-      const float4* row4 = reinterpret_cast<const float4*>(vals);
-      const int n4 = N >> 2;
-      for (int base4 = 0; base4 < n4; base4 += 32 * 8) {
-        float4 buf[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k4 = base4 + u * 32 + lane;
-          buf[u] = k4 < n4 ? row4[k4] : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k4 = base4 + u * 32 + lane;
-          const float c4[4] = {buf[u].x, buf[u].y, buf[u].z, buf[u].w};
-          // survivors before this lane's: one ballot per element of the float4
-          int pre = 0, tot = 0;
-#pragma unroll
-          for (int e2 = 0; e2 < 4; ++e2) {
-            rowmax = fmaxf(rowmax, c4[e2]);
-            const unsigned bal = __ballot_sync(FULL, k4 < n4 && c4[e2] > bnew);
-            pre += __popc(bal & lt);
-            tot += __popc(bal);
-          }
-          int pos = w + pre;
-          if (k4 < n4) {
-#pragma unroll
-            for (int e2 = 0; e2 < 4; ++e2)
-              if (c4[e2] > bnew) {
-                const int j = 4 * k4 + e2;
-                vals[pos] = c4[e2];
-                cols[pos] = (uint16_t)j;
-                atomicAdd(&uacc[j], (unsigned long long)(to_fix(c4[e2], fxs) - fb_new));
-                ++pos;
-              }
-          }
-          w += tot;
-        }
-        __syncwarp();
-      }
-    } else {
-      for (int base = 0; base < N; base += 32) {
-        const int k = base + lane;
-        const float c = k < N ? vals[k] : 0.f;
-        rowmax = fmaxf(rowmax, c);
-        const bool keep = k < N && c > bnew;
-        const unsigned msk = __ballot_sync(FULL, keep);
-        __syncwarp();
-        if (keep) {
-          const int pos = w + __popc(msk & sel::lanemask_lt());
-          vals[pos] = c;
-          cols[pos] = (uint16_t)k;
-          atomicAdd(&uacc[k], (unsigned long long)(to_fix(c, fxs) - fb_new));
-        }
-        w += __popc(msk);
-      }
-    }
-    rowmax = warp_max(rowmax);
+    float4* tile = sm_r0f + (threadIdx.x >> 5) * TILE;
+    float rowmax = 0.f;  // only the trace reports F(V)
+    const int w =
+        tv.base ? sel::filter_dense_row<true>(vals, cols, N, bnew, fb_new, fxs, sums, tile, &rowmax)
+                : sel::filter_dense_row<false>(vals, cols, N, bnew, fb_new, fxs, sums, tile, &rowmax);
     if (lane == 0) {
       bcov[(size_t)b * Mstride + m] = bnew;
       cnt[(size_t)b * Mstride + m] = w;
-      const int bank = m < MG ? 0 : (m < MG + N ? 1 : 2);
-      atomicAdd((unsigned long long*)&fb[bank], (unsigned long long)to_fix(rowmax, fxs));
-      if (tv.base) atomicAdd(tv.cover(b, 0), (unsigned long long)fb_new);  // F after the round
+      if (tv.base) {
+        const int bank = m < MG ? 0 : (m < MG + N ? 1 : 2);
+        atomicAdd((unsigned long long*)&fb[bank], (unsigned long long)to_fix(rowmax, fxs));
+        atomicAdd(tv.cover(b, 0), (unsigned long long)fb_new);  // F after the round
+      }
     }
   }
   __syncthreads();
   if (threadIdx.x < 3 && fb[threadIdx.x])
     atomicAdd((unsigned long long*)&fv[(size_t)b * 4 + threadIdx.x], (unsigned long long)fb[threadIdx.x]);
-  unsigned long long* ub = reinterpret_cast<unsigned long long*>(u1 + (size_t)b * N);
-  for (int j = threadIdx.x; j < N; j += blockDim.x)
-    if (uacc[j]) atomicAdd(&ub[j], uacc[j]);
+  sums.flush(reinterpret_cast<unsigned long long*>(u1 + (size_t)b * N), false);
 }
 
 // ---- sparse rounds on the whole GPU -------------------------------------------
@@ -405,14 +388,14 @@ __global__ void __launch_bounds__(512) k_rg_pool(const long long* __restrict__ u
 }
 
 template <int ROWS>
-__global__ void __launch_bounds__(32 * ROWS) k_rg_rho(
+__global__ void __launch_bounds__(32 * ROWS, ROWS == 16 ? 4 : 5) k_rg_rho(
     const float* __restrict__ C, const uint16_t* __restrict__ scol,
     const float* __restrict__ bcov, const int32_t* __restrict__ cnt, int B, int N, int Mstride,
     int H, int L2, const int32_t* toff, int Tmax, int uniform_rows,
     const int32_t* __restrict__ pool0, const int32_t* __restrict__ info, int P, float resp_temp,
-    float resp_eps, int fx_exp, const int32_t* fexp, long long* sc) {
+    float resp_eps, int fx_exp, const int32_t* fexp, int rpw, long long* sc) {
   grid_dep_wait();
-  __shared__ long long sblk[GMC_MAX_POOL];
+  __shared__ uint32_t sblk[3 * GMC_MAX_POOL];  // limbs: at most ROWS * rpw additions per slot
   __shared__ int fslot[ROWS][GMC_MAX_POOL];  // a row's pool entries: slot and residual
   __shared__ float fres[ROWS][GMC_MAX_POOL];
   extern __shared__ short pslot[];              // [N] pool slot of every token or -1
@@ -421,26 +404,58 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_rho(
   if (Pt == 0) return;
   int Mb = Mstride;
   if (!uniform_rows) Mb = H * text_geom(toff, b, B, Tmax, nullptr).T + N + L2;
-  const int m0 = blockIdx.x * ROWS;
+  const int m0 = blockIdx.x * ROWS * rpw;
   if (m0 >= Mb) return;
   const float fxs = ldexpf(1.f, fexp ? fexp[b] : fx_exp);
   for (int j = threadIdx.x; j < N; j += blockDim.x) pslot[j] = -1;
-  for (int k = threadIdx.x; k < P; k += blockDim.x) sblk[k] = 0;
+  for (int k = threadIdx.x; k < 3 * GMC_MAX_POOL; k += blockDim.x) sblk[k] = 0;
   __syncthreads();
   for (int k = threadIdx.x; k < Pt; k += blockDim.x) pslot[pool0[(size_t)b * P + k]] = (short)k;
   __syncthreads();
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, m = m0 + w;
-  if (m < Mb) {
-    const size_t row = (size_t)b * Mstride + m;
-    const int n = cnt[row];
-    const float bm = bcov[row];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int mw = m0 + w * rpw, nr = min(rpw, Mb - mw);  // this warp's rows (rpw <= 32)
+  const size_t row0 = (size_t)b * Mstride + mw;
+  constexpr bool AHEAD = ROWS == 8;
+  using Head = RowHead<AHEAD>;
+  Head next;
+  int cnts = 0;  // AHEAD: the rows' counts and coverages, one per lane
+  float covs = 0.f;
+  if constexpr (AHEAD) {
+    if (lane < nr) {
+      cnts = cnt[row0 + lane];
+      covs = bcov[row0 + lane];
+    }
+    next.load(C + row0 * N, scol + row0 * N, __shfl_sync(FULL, cnts, 0), lane);
+  }
+  const unsigned lt = sel::lanemask_lt();
+  for (int ir = 0; ir < nr; ++ir) {
+    const size_t row = row0 + ir;
+    const int n = AHEAD ? __shfl_sync(FULL, cnts, ir) : cnt[row];
+    const float bm = AHEAD ? __shfl_sync(FULL, covs, ir) : bcov[row];
     const float* vals = C + row * N;
     const uint16_t* cols = scol + row * N;
-    const unsigned lt = sel::lanemask_lt();
+    const Head head = next;
+    if constexpr (AHEAD) {
+      const int n1 = __shfl_sync(FULL, cnts, min(ir + 1, 31));
+      next.load(vals + N, cols + N, ir + 1 < nr ? n1 : 0, lane);
+    }
     int nf = 0;
     float rmax = 0.f;
+    auto take = [&](int ps, float R) {  // a pool entry of the row: its slot and residual
+      const unsigned bal = __ballot_sync(FULL, ps >= 0);
+      if (ps >= 0) {
+        const int at = nf + __popc(bal & lt);
+        fslot[w][at] = ps;
+        fres[w][at] = R;
+        rmax = fmaxf(rmax, R);
+      }
+      nf += __popc(bal);
+    };
+#pragma unroll
+    for (int u = 0; u < Head::U; ++u)
+      if (32 * u < n) take(head.j[u] >= 0 ? (int)pslot[head.j[u]] : -1, head.v[u] - bm);
     constexpr int RU = 4;  // chunks of 32 entries whose loads are in flight together
-    for (int e00 = 0; e00 < n; e00 += 32 * RU) {
+    for (int e00 = 32 * Head::U; e00 < n; e00 += 32 * RU) {
       int ps[RU];
       float R[RU];
 #pragma unroll
@@ -454,16 +469,7 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_rho(
         R[u] = ps[u] >= 0 ? vals[e00 + 32 * u + lane] - bm : 0.f;  // > 0: exceeds its coverage
       }
 #pragma unroll
-      for (int u = 0; u < RU; ++u) {
-        const unsigned bal = __ballot_sync(FULL, ps[u] >= 0);
-        if (ps[u] >= 0) {
-          const int at = nf + __popc(bal & lt);
-          fslot[w][at] = ps[u];
-          fres[w][at] = R[u];
-          rmax = fmaxf(rmax, R[u]);
-        }
-        nf += __popc(bal);
-      }
+      for (int u = 0; u < RU; ++u) take(ps[u], R[u]);
     }
     rmax = warp_max(rmax);
     __syncwarp();
@@ -477,18 +483,21 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_rho(
       const float invz = 1.f / z;
       for (int q = lane; q < nf; q += 32) {
         const float R = fres[w][q];
-        atomicAdd((unsigned long long*)&sblk[fslot[w][q]],
-                  (unsigned long long)to_fix(expf((R - rmax) / tau) * invz * R, fxs));
+        sel::limb_add(&sblk[fslot[w][q]], GMC_MAX_POOL,
+                      (unsigned long long)to_fix(expf((R - rmax) / tau) * invz * R, fxs));
       }
+      __syncwarp();  // the next row refills the warp's entries
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < Pt; k += blockDim.x)
-    if (sblk[k]) atomicAdd((unsigned long long*)&sc[(size_t)b * P + k], (unsigned long long)sblk[k]);
+  for (int k = threadIdx.x; k < Pt; k += blockDim.x) {
+    const unsigned long long v = sel::limb_value(sblk + k, GMC_MAX_POOL);
+    if (v) atomicAdd((unsigned long long*)&sc[(size_t)b * P + k], v);
+  }
 }
 
 template <int ROWS>
-__global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
+__global__ void __launch_bounds__(32 * ROWS, ROWS == 16 ? 3 : 4) k_rg_filter(
     float* C, uint16_t* scol, int B, int N, int K, int Mstride, int H, int L2,
     const int32_t* toff, int Tmax, int uniform_rows, const int32_t* __restrict__ pool0,
     int32_t* info, const long long* __restrict__ sc0, int P, int bsz, int fx_exp,
@@ -498,8 +507,9 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
   __shared__ int pool[GMC_MAX_POOL];
   __shared__ long long sc[GMC_MAX_POOL];
   __shared__ int batch[GMC_MAX_POOL];
-  extern __shared__ unsigned long long uacc[];  // [N] then the batch flags [N] (bytes)
-  unsigned char* inb = reinterpret_cast<unsigned char*>(uacc + N);
+  extern __shared__ __align__(16) char sm_rgf[];  // the falls of the gains, then the batch flags [N]
+  const sel::GainSums<true> sums{reinterpret_cast<uint32_t*>(sm_rgf), N};
+  unsigned char* inb = reinterpret_cast<unsigned char*>(sm_rgf) + sel::gain_sums_bytes(N);
   const int b = blockIdx.y;
   const int Pt = info[b * INFO_W];
   if (Pt == 0) return;
@@ -514,10 +524,8 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
     pool[k] = pool0[(size_t)b * P + k];
     sc[k] = sc0[(size_t)b * P + k];
   }
-  for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    uacc[j] = 0;
-    inb[j] = 0;
-  }
+  sums.clear();
+  for (int j = threadIdx.x; j < N; j += blockDim.x) inb[j] = 0;
   __syncthreads();
   {
     const int lane = threadIdx.x & 31, gl = lane & 7;
@@ -539,20 +547,41 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
   }
   __syncthreads();
   const int lane = threadIdx.x & 31;
-  for (int ir = 0; ir < rpw; ++ir) {
-    const int m = m0 + (threadIdx.x >> 5) + ROWS * ir;
-    if (m >= Mb) break;
-    const size_t row = (size_t)b * Mstride + m;
-    const int n = cnt[row];
+  const int mw = m0 + (threadIdx.x >> 5) * rpw, nr = min(rpw, Mb - mw);  // this warp's rows
+  const size_t row0 = (size_t)b * Mstride + mw;
+  constexpr bool AHEAD = ROWS == 8;
+  using Head = RowHead<AHEAD>;
+  Head next;
+  int cnts = 0;  // AHEAD: the rows' counts and coverages, one per lane
+  float covs = 0.f;
+  if constexpr (AHEAD) {
+    if (lane < nr) {
+      cnts = cnt[row0 + lane];
+      covs = bcov[row0 + lane];
+    }
+    next.load(C + row0 * N, scol + row0 * N, __shfl_sync(FULL, cnts, 0), lane);
+  }
+  const unsigned lt = sel::lanemask_lt();
+  for (int ir = 0; ir < nr; ++ir) {
+    const size_t row = row0 + ir;
+    const int n = AHEAD ? __shfl_sync(FULL, cnts, ir) : cnt[row];
+    const float bold = AHEAD ? __shfl_sync(FULL, covs, ir) : bcov[row];
     float* vals = C + row * N;
     uint16_t* cols = scol + row * N;
+    const Head head = next;
+    if constexpr (AHEAD) {
+      const int n1 = __shfl_sync(FULL, cnts, min(ir + 1, 31));
+      next.load(vals + N, cols + N, ir + 1 < nr ? n1 : 0, lane);
+    }
     // The list is walked FU chunks of 32 entries at a time, every load of the
     // chunks issued before the first use (and, below, before any survivor is
     // written back in place: a chunk's survivors land below its end).
     constexpr int FU = 4;
-    const float bold = bcov[row];
     float bnew = bold;
-    for (int e00 = 0; e00 < n; e00 += 32 * FU) {
+#pragma unroll
+    for (int u = 0; u < Head::U; ++u)
+      if (head.j[u] >= 0 && inb[head.j[u]]) bnew = fmaxf(bnew, head.v[u]);
+    for (int e00 = 32 * Head::U; e00 < n; e00 += 32 * FU) {
       int jj[FU];
 #pragma unroll
       for (int u = 0; u < FU; ++u) {
@@ -570,9 +599,24 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
       continue;
     }
     const long long fb_old = to_fix(bold, fxs);
-    const unsigned lt = sel::lanemask_lt();
     int wr = 0;
-    for (int e00 = 0; e00 < n; e00 += 32 * FU) {
+    // an entry's residual moves from C - b_old to C - b_new, or to zero (exact:
+    // integers modulo 2^64); survivors move down in order
+    auto settle = [&](bool in, int j, float c) {
+      const bool keep = in && c > bnew;
+      const unsigned bal = __ballot_sync(FULL, keep);
+      if (in) sums.add(j, (unsigned long long)((keep ? fb_new : to_fix(c, fxs)) - fb_old));
+      if (keep) {
+        const int pos = wr + __popc(bal & lt);
+        vals[pos] = c;
+        cols[pos] = (uint16_t)j;
+      }
+      wr += __popc(bal);
+    };
+#pragma unroll
+    for (int u = 0; u < Head::U; ++u)
+      if (32 * u < n) settle(head.j[u] >= 0, head.j[u], head.v[u]);
+    for (int e00 = 32 * Head::U; e00 < n; e00 += 32 * FU) {
       float cc[FU];
       int jj[FU];
 #pragma unroll
@@ -587,22 +631,7 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
       }
       __syncwarp();  // the chunks are read before any survivor moves down into them
 #pragma unroll
-      for (int u = 0; u < FU; ++u) {
-        const bool in = e00 + 32 * u + lane < n;
-        const bool keep = in && cc[u] > bnew;
-        const unsigned bal = __ballot_sync(FULL, keep);
-        // the entry's residual moves from C - b_old to C - b_new, or to zero
-        // (exact: integers modulo 2^64)
-        if (in)
-          atomicAdd(&uacc[jj[u]], (unsigned long long)(keep ? fb_old - fb_new
-                                                             : fb_old - to_fix(cc[u], fxs)));
-        if (keep) {
-          const int pos = wr + __popc(bal & lt);
-          vals[pos] = cc[u];
-          cols[pos] = (uint16_t)jj[u];
-        }
-        wr += __popc(bal);
-      }
+      for (int u = 0; u < FU; ++u) settle(e00 + 32 * u + lane < n, jj[u], cc[u]);
     }
     if (lane == 0) {
       bcov[row] = bnew;
@@ -611,12 +640,10 @@ __global__ void __launch_bounds__(32 * ROWS) k_rg_filter(
     }
   }
   __syncthreads();
-  unsigned long long* ub = reinterpret_cast<unsigned long long*>(unext + (size_t)b * N);
-  for (int j = threadIdx.x; j < N; j += blockDim.x)
-    if (uacc[j]) atomicAdd(&ub[j], uacc[j]);
+  sums.flush(reinterpret_cast<unsigned long long*>(unext + (size_t)b * N), true);
 }
 
-// The responsibility and filter launches of every whole-GPU round, ROWS rows per block.
+// The responsibility and filter launches of every whole-GPU round, ROWS warps per block.
 template <int ROWS>
 static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, int M,
                                       const int32_t* toff, int H, int T, int L2,
@@ -626,16 +653,15 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   const int P = p.pool_mult * p.batch_b;
   const int uniform = (H == 0);
   cudaError_t e;
-  dim3 grid(ceil_div(M, ROWS), B);
+  const int rpw = rows_per_warp(B, M, ROWS);
+  const dim3 grid(ceil_div(M, ROWS * rpw), B);
   launch_k(k_r0_rho<ROWS>, grid, 32 * ROWS, 0, st, 1, C, B, N, M, H, L2, toff, T, uniform, r0.pool,
-           r0.info, P, p.resp_temp, p.resp_eps, fx_exp, fexp, I, r0.s0);
+           r0.info, P, p.resp_temp, p.resp_eps, fx_exp, fexp, I, rpw, r0.s0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const size_t fsm = sizeof(unsigned long long) * (size_t)N;
+  const size_t fsm = sizeof(float) * ROWS * sel::ROW_STEP + sel::gain_sums_bytes(N);
   if ((e = set_smem_limit((const void*)k_r0_filter<ROWS>, fsm)) != cudaSuccess) return e;
-  const int rpw = filter_rows_per_warp(B, M, ROWS);
-  const dim3 fgrid(ceil_div(M, ROWS * rpw), B);
-  launch_k(k_r0_filter<ROWS>, fgrid, 32 * ROWS, fsm, st, 1, C, scol, B, N, K, M, H, L2, toff, T,
-           uniform, r0.pool, r0.info, r0.s0, P, p.batch_b, fx_exp, fexp, r0.u1, r0.bcov, r0.cnt,
+  launch_k(k_r0_filter<ROWS>, grid, 32 * ROWS, fsm, st, 1, C, scol, B, N, K, M, H, L2, toff,
+           T, uniform, r0.pool, r0.info, r0.s0, P, p.batch_b, fx_exp, fexp, r0.u1, r0.bcov, r0.cnt,
            r0.fv, order, rpw, I, tv);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // sparse rounds: gains alternate between u1 and u2
@@ -644,7 +670,7 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   if ((e = set_smem_limit((const void*)k_rg_pool, psm)) != cudaSuccess) return e;
   const size_t rsm = sizeof(short) * (size_t)N;
   if ((e = set_smem_limit((const void*)k_rg_rho<ROWS>, rsm)) != cudaSuccess) return e;
-  const size_t gsm = sizeof(unsigned long long) * (size_t)N + (size_t)N;
+  const size_t gsm = sel::gain_sums_bytes(N) + (size_t)N;
   if ((e = set_smem_limit((const void*)k_rg_filter<ROWS>, gsm)) != cudaSuccess) return e;
   const int rounds = sparse_gpu_rounds(N, B, K, p.batch_b, I);
   for (int rr = 1; rr <= rounds; ++rr) {
@@ -656,10 +682,10 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
     launch_k(k_rg_rho<ROWS>, grid, 32 * ROWS, rsm, st, 1, (const float*)C, (const uint16_t*)scol,
              (const float*)r0.bcov, (const int32_t*)r0.cnt, B, N, M, H, L2, toff, T, uniform,
              (const int32_t*)r0.pool, (const int32_t*)r0.info, P, p.resp_temp, p.resp_eps, fx_exp,
-             fexp, r0.s0);
+             fexp, rpw, r0.s0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    launch_k(k_rg_filter<ROWS>, fgrid, 32 * ROWS, gsm, st, 1, C, scol, B, N, K, M, H, L2, toff, T,
-             uniform, (const int32_t*)r0.pool, r0.info, (const long long*)r0.s0, P, p.batch_b,
+    launch_k(k_rg_filter<ROWS>, grid, 32 * ROWS, gsm, st, 1, C, scol, B, N, K, M, H, L2, toff,
+             T, uniform, (const int32_t*)r0.pool, r0.info, (const long long*)r0.s0, P, p.batch_b,
              fx_exp, fexp, unext, r0.bcov, r0.cnt, order, rpw, tv);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -682,13 +708,9 @@ cudaError_t launch_round0(R0State& r0, int B, int N, int K, int M, const int32_t
   launch_k(k_r0_pool, B, 512, smem, st, 1, u0, B, N, P, uniform ? nullptr : toff, T, I, r0.pool, r0.info,
                                   r0.s0, r0.u1, r0.fv, status, tv);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  // one image: 16 rows per block (fewer, larger blocks finish the rounds
-  // sooner); a batch: 8
-  if (B == 1)
-    return launch_rounds_rows<16>(r0, B, N, K, M, toff, H, T, L2, p, fx_exp, fexp, C, scol, order,
-                                  tv, st, I, smem);
-  return launch_rounds_rows<8>(r0, B, N, K, M, toff, H, T, L2, p, fx_exp, fexp, C, scol, order, tv,
-                               st, I, smem);
+  // one image: 16 warps per block (fewer, larger blocks finish the rounds sooner); a
+  // batch: 8
+  return (B == 1 ? launch_rounds_rows<16> : launch_rounds_rows<8>)(r0, B, N, K, M, toff, H, T, L2, p, fx_exp, fexp, C, scol, order, tv, st, I, smem);
 }
 
 }  // namespace gmc

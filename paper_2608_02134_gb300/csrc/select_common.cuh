@@ -37,6 +37,114 @@ __device__ __forceinline__ unsigned long long limb_value(const uint32_t* w, int 
          ((unsigned long long)w[2 * stride] << (2 * LIMB));
 }
 
+// Sums of a block's changes of the gains, one per token: limbs, or 64-bit words
+// where the limbs of N tokens would not leave room for two blocks on an SM.
+constexpr int LIMB_MAX_N = 8192;
+__host__ __device__ inline size_t gain_sums_bytes(int N) {
+  return (N <= LIMB_MAX_N ? 12 : 8) * (size_t)N;
+}
+template <bool LIMBS>
+struct GainSums {
+  uint32_t* w;
+  int N;
+  __device__ __forceinline__ void clear() const {
+    for (int k = threadIdx.x; k < (LIMBS ? 3 : 2) * N; k += blockDim.x) w[k] = 0;
+  }
+  __device__ __forceinline__ void add(int j, unsigned long long v) const {
+    if constexpr (LIMBS) limb_add(w + j, N, v);
+    else atomicAdd(reinterpret_cast<unsigned long long*>(w) + j, v);
+  }
+  // every nonzero sum, its sign applied, into the global gains
+  __device__ __forceinline__ void flush(unsigned long long* gains, bool negative) const {
+    for (int j = threadIdx.x; j < N; j += blockDim.x) {
+      unsigned long long v;
+      if constexpr (LIMBS) v = limb_value(w + j, N);
+      else v = reinterpret_cast<const unsigned long long*>(w)[j];
+      if (v) atomicAdd(&gains[j], negative ? 0ull - v : v);
+    }
+  }
+};
+
+// One dense client row of N values, by one warp: the entries above `cover`
+// (residual survivors) move to the front of the row in place, with their tokens
+// in cols; their residuals are added to `sums`.  Returns the survivors; *rowmax
+// (MAX) the row's largest value in every lane.
+//
+// A warp takes ROW_STEP values a step: 16 per lane, compared into a bit mask; one scan of the counts places every lane's
+// survivors (lane by lane, ascending within a lane), and only they take the slow
+// part, one per lane and turn, read back from the warp's tile in shared memory.
+// With one survivor in sixteen, doing that part at every position instead cost a
+// warp about four times the instructions.
+constexpr int ROW_STEP = 512;  // values a step (2 KB of tile per warp)
+constexpr int ROW_U = ROW_STEP / 128;  // 16-byte loads in flight per lane
+template <bool MAX, class Sums>
+__device__ __forceinline__ int filter_dense_row(float* vals, uint16_t* cols, int N, float cover,
+                                                long long cover_fix, float fxs, const Sums& sums,
+                                                float4* tile, float* rowmax) {
+  const int lane = threadIdx.x & 31;
+  const bool vec = (N & 3) == 0;  // rows start on 16 bytes
+  float mx = 0.f;
+  int w = 0;
+  for (int base = 0; base < N; base += ROW_STEP) {
+    if (vec) {
+      float4 buf[ROW_U];
+#pragma unroll
+      for (int u = 0; u < ROW_U; ++u) {
+        const int k = base + 4 * (u * 32 + lane);
+        buf[u] = k < N ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+      }
+      __syncwarp();  // the last step's survivors are out of the tile
+#pragma unroll
+      for (int u = 0; u < ROW_U; ++u) tile[u * 32 + lane] = buf[u];
+    } else {
+      float b1[8];
+      __syncwarp();
+#pragma unroll
+      for (int h = 0; h < ROW_STEP / 256; ++h) {
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+          const int k = base + (h * 8 + u) * 32 + lane;
+          b1[u] = k < N ? vals[k] : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          reinterpret_cast<float*>(tile)[(h * 8 + u) * 32 + lane] = b1[u];
+      }
+    }
+    __syncwarp();
+    unsigned mask = 0;
+#pragma unroll
+    for (int u = 0; u < ROW_U; ++u) {  // values past N are zero: never above a coverage
+      const float4 x = tile[u * 32 + lane];
+      mask |= (x.x > cover ? 1u : 0u) << (4 * u) | (x.y > cover ? 2u : 0u) << (4 * u) |
+              (x.z > cover ? 4u : 0u) << (4 * u) | (x.w > cover ? 8u : 0u) << (4 * u);
+      if (MAX) mx = fmaxf(fmaxf(mx, fmaxf(x.x, x.y)), fmaxf(x.z, x.w));
+    }
+    const int c = __popc(mask);
+    int incl = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(FULL, incl, o);
+      if (lane >= o) incl += y;
+    }
+    int pos = w + incl - c;
+    w += __shfl_sync(FULL, incl, 31);
+    while (mask) {
+      const int bit = __ffs(mask) - 1;
+      mask &= mask - 1;
+      const int at = 4 * ((bit >> 2) * 32 + lane) + (bit & 3);
+      const float x = reinterpret_cast<const float*>(tile)[at];
+      vals[pos] = x;  // at or below the step's last value, which every lane has read
+      cols[pos] = (uint16_t)(base + at);
+      ++pos;
+      sums.add(base + at, (unsigned long long)(to_fix(x, fxs) - cover_fix));
+    }
+  }
+  if (MAX) *rowmax = warp_max(mx);
+  __syncwarp();  // the next row reuses the tile
+  return w;
+}
+
 // Monotone 11-bit bucket of a positive 64-bit gain: exponent and 5 mantissa bits.
 __device__ __forceinline__ int gain_bucket(long long u) {
   const int lz = __clzll(u);                                      // 1..63 for 0 < u < 2^63
