@@ -61,3 +61,56 @@ def _clients(kind, B, M, N, seed):
 def test_cluster_solver_sizes(kind, B, M, N, K, b, mult):
     from tests.test_gpu_stages import _check_select
     _check_select(_clients(kind, B, M, N, 5 + N), K, batch_b=b, pool_mult=mult)
+
+
+# transport: fewer and more member rows than a thread has in flight, lists of more
+# than 64 members (one carrier takes every token), one list for the block (N above
+# 4,096), a row that is one CTA and one that is eight, more text rows than carriers,
+# K/V rows wider than the threads, both types; from a caller's assignment
+@pytest.mark.parametrize("B,gh,gw,T,K,D,Hkv,d,dtype,spread", [
+    (1, 5, 7, 3, 4, 64, 2, 32, "bf16", "all"), (2, 9, 31, 40, 11, 1032, 1, 8, "f32", "even"),
+    (1, 66, 64, 5, 700, 256, 2, 32, "bf16", "even"), (1, 128, 64, 9, 3, 8192, 32, 128, "bf16", "all"),
+    (3, 20, 13, 17, 260, 3584, 4, 128, "bf16", "even"), (1, 64, 64, 2, 33, 4096, 16, 64, "f32", "skew")])
+def test_transport_sizes(B, gh, gw, T, K, D, Hkv, d, dtype, spread):
+    from paper_2608_02134_gb300 import gmc
+    N = gh * gw
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + D)
+    tdt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    hid = torch.randn((B, N + T, D), generator=g, device="cuda").to(tdt)
+    kv = torch.randn((B, 2, N + T, Hkv, d), generator=g, device="cuda").to(tdt)
+    pos = torch.randint(0, 1000, (B, 3, N + T), generator=g, device="cuda", dtype=torch.int32)
+    sup = torch.stack([torch.randperm(N, generator=g, device="cuda")[:K].sort().values
+                       for _ in range(B)])
+    u = torch.rand((B, N), generator=g, device="cuda")
+    slot = {"all": torch.zeros_like(u), "even": u * K, "skew": u ** 3 * K}[spread].long().clamp(max=K - 1)
+    slot.scatter_(1, sup, torch.arange(K, device="cuda").expand(B, K))
+    pi = sup.gather(1, slot)
+    w = 0.5 + torch.rand((B, N), generator=g, device="cuda")
+    prob = gmc.problem(B, gh, gw, Hkv, gmc.GMC_BF16 if dtype == "bf16" else gmc.GMC_F32)
+    ws = gmc.alloc_workspace(gmc.transport_workspace_size(prob, N, T, K))
+    oi = torch.empty(B * K, dtype=torch.int32, device="cuda")
+    oh = torch.empty((B, K + T, D), dtype=tdt, device="cuda")
+    okv = torch.empty((B, 2, K + T, Hkv, d), dtype=tdt, device="cuda")
+    op = torch.empty((B, 3, K + T), dtype=torch.int32, device="cuda")
+    gmc.transport(prob, gmc.default_params(), hid, kv, pos, sup.int().contiguous(),
+                  pi.int().contiguous(), w, N, T, d, D, K, oi, oh, okv, op, ws)
+    torch.cuda.synchronize()
+    assert gmc.read_status(ws) == 0
+    assert torch.equal(oi.view(B, K).long(), sup)
+    for b in range(B):
+        rows = torch.cat([sup[b], N + torch.arange(T, device="cuda")])
+        assert torch.equal(okv[b], kv[b][:, rows]) and torch.equal(op[b], pos[b][:, rows])
+        assert torch.equal(oh[b, K:], hid[b, N:])
+        h, m = hid[b, :N].double(), w[b].double()
+        acc = torch.zeros((K, D), dtype=torch.float64, device="cuda").index_add_(0, slot[b], m[:, None] * h)
+        cen = acc / torch.zeros(K, dtype=torch.float64, device="cuda").index_add_(0, slot[b], m)[:, None]
+        rms = lambda v: v.square().mean(1, keepdim=True).sqrt()  # noqa: E731
+        ref = cen * rms(h[sup[b]]) / (rms(cen) + 1e-6)
+        # fp32 sums of up to N terms, each rounded once (N 2^-24 of the terms' magnitude), and
+        # the cast of the output: half an ulp of bf16
+        terms = torch.zeros_like(acc).index_add_(0, slot[b], m[:, None] * h.abs()) / (acc.abs() + 1e-300)
+        bound = (N * 2.0 ** -24) * (terms * ref.abs()) + 2e-6 * ref.abs() + 1e-7
+        if dtype == "bf16":
+            bound = bound + ref.abs() * 2.0 ** -8
+        assert bool(((oh[b, :K].double() - ref).abs() <= bound).all())
