@@ -54,13 +54,19 @@ struct MsgCtl {
   float stat_m[EPI_PARTS][BM];
   float stat_l[EPI_PARTS][BM];
   float rsum[EPI_PARTS][BM];
+  int arow[BM];  // row of A of every tile row, -1: none
 };
+// the write launch's staging tiles, one 32 x 32 fp32 tile per epilogue warp
+constexpr int WRITE_STAGE_BYTES = EPI_WARPS * 32 * 32 * 4;
 
 // Fused kernel: 16 epilogue warps (warp w reads TMEM lanes 32*(w%4).. and the
 // 32-column quarter w/4 of every tile), then the TMA producer and MMA warps.
 constexpr int FE_WARPS = 16, FT_THREADS = 32 * (FE_WARPS + 2);
 
-constexpr int FUSED_MAX_CLUSTER = 8;  // portable cluster size
+constexpr int FUSED_PORTABLE = 8;      // portable cluster size
+constexpr int FUSED_MAX_CLUSTER = 16;  // with the non-portable attribute
+
+constexpr int FUSED_MAX_TILES = 4;  // key tiles a CTA keeps in TMEM (4 x 128 columns)
 
 // Control block of the fused kernel: barriers, this CTA's per-row statistics
 // and the statistics of every split of the cluster.
@@ -78,12 +84,12 @@ struct FusedCtl {
   // each CTA of the cluster by the split that owns them
   float all_m[FUSED_MAX_CLUSTER][BM];
   float all_l[FUSED_MAX_CLUSTER][BM];
+  int arow[BM];  // row of A of every tile row, -1: none
 };
 
 __device__ __forceinline__ void fused_epi_barrier() {
   asm volatile("bar.sync 1, %0;" ::"n"(FE_WARPS * 32) : "memory");
 }
-constexpr int FUSED_MAX_TILES = 4;     // key tiles a CTA keeps in TMEM (4 x 128 columns)
 constexpr int FUSED_STAGE_BYTES = FE_WARPS * 32 * 32 * 4;  // one 32 x 32 fp32 tile per warp
 
 // Bytes before the control block: the operand tiles (query tile and key ring)
@@ -94,22 +100,43 @@ __host__ __device__ inline size_t fused_region_bytes(int nkb) {
 }
 
 struct MsgSplit {
-  int kt_per;  // key tiles per split
+  int kt_per;  // key tiles per split at the widest image (an image's own: split_tiles)
   int n;       // splits
 };
 
+// Key splits of a query tile.  Few query tiles: enough splits for one wave of
+// CTAs.  Many: one split would do, but the fused kernel writes A from logits
+// it keeps in TMEM, in whole 128-byte lines, where the two launches compute every
+// logit twice and store row by row; so the splits are at least as many as
+// hold an image's keys in TMEM (FUSED_MAX_TILES each) while a cluster can span
+// them, and at most a portable cluster where that is enough.  Measured, two
+// launches -> fused: 32 ragged images of N = 1,296 (13 key tiles, T <= 256)
+// 695 us -> 492, N = 4,096 at T = 128 (33 tiles, 9 splits) 69 us ->
+// 47.
 MsgSplit msg_split(int B, int Hkv, int RQ, int N, int T) {
   const int nkt = (N + T + BM - 1) / BM;
   const int base = (RQ / BM) * Hkv * B;
-  const int target = SPLIT_TARGET_CTAS / base > 1 ? SPLIT_TARGET_CTAS / base : 1;
+  int target = SPLIT_TARGET_CTAS / base > 1 ? SPLIT_TARGET_CTAS / base : 1;
+  const int need = (nkt + FUSED_MAX_TILES - 1) / FUSED_MAX_TILES;
+  if (need <= FUSED_MAX_CLUSTER) {
+    if (target > FUSED_PORTABLE) target = FUSED_PORTABLE;
+    if (target < need) target = need;
+  }
   MsgSplit sp;
   sp.kt_per = (nkt + target - 1) / target;
   sp.n = (nkt + sp.kt_per - 1) / sp.kt_per;
   return sp;
 }
 
-size_t msg_smem_bytes(int nkb) {
-  return 1024 + (size_t)nkb * TILE_BYTES * (1 + STAGES) + sizeof(MsgCtl);
+// Key tiles per split of an image with nkt tiles: spread evenly, so that an
+// image with fewer keys than the widest one leaves no split empty.
+__device__ __forceinline__ int split_tiles(int nkt, int nsplit) { return ceil_div(nkt, nsplit); }
+
+__host__ __device__ inline size_t msg_ctl_bytes() { return (sizeof(MsgCtl) + 127) & ~(size_t)127; }
+// the write launch (mode 1) has the staging tiles besides
+size_t msg_smem_bytes(int nkb, int mode) {
+  return 1024 + (size_t)nkb * TILE_BYTES * (1 + STAGES) + msg_ctl_bytes() +
+         (mode ? WRITE_STAGE_BYTES : 0);
 }
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -123,7 +150,7 @@ __device__ __forceinline__ void epi_barrier() {
 __global__ void __launch_bounds__(THREADS, 1)
     k_message_tc(const __grid_constant__ CUtensorMap qmap, const __grid_constant__ CUtensorMap kmap,
                  const int32_t* toff, int B, int N, int Tmax, int H, int Hkv, int d, int RQ,
-                 int mode, int kt_per, int nsplit, float2* part,
+                 int mode, int nsplit, float2* part,
                  const float* __restrict__ zn2, const float* __restrict__ sigma, float* A,
                  float* rs, uint32_t* status) {
   grid_dep_wait();
@@ -141,8 +168,8 @@ __global__ void __launch_bounds__(THREADS, 1)
   if (tg.T == 0 || tile * BM >= grp * tg.T) return;  // uniform per CTA
   const int Tb = tg.T;
   const int nkeys = N + Tb;
-  const int nkt = ceil_div(nkeys, BM);
-  const int c0 = split * kt_per, c1 = min(nkt, c0 + kt_per);
+  const int nkt = ceil_div(nkeys, BM), kt = split_tiles(nkt, nsplit);
+  const int c0 = split * kt, c1 = min(nkt, c0 + kt);
   const int iters = max(0, c1 - c0);  // an image with fewer keys than the widest one
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qrow0 = (int)(((size_t)b * Hkv + g) * RQ + (size_t)tile * BM);
@@ -238,7 +265,10 @@ __global__ void __launch_bounds__(THREADS, 1)
     const float sg = sigma[(size_t)b * H + h];
     const float sg2 = sg * sg;
     const float* zr = zn2 + ((size_t)b * H + h) * N;
-    float* arow = A + (((size_t)b * H + h) * Tmax + t) * N;
+    float* stg = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(ctl) + msg_ctl_bytes()) +
+                 warp * 32 * 32;
+    if (cpart == 0) ctl->arow[r] = valid ? (b * H + h) * Tmax + t : -1;
+    epi_barrier();
     const int kvis = N + t + 1;                  // keys this query may see
     float2* prow = part + ((((size_t)b * Hkv + g) * RQ) + (size_t)tile * BM + r) * nsplit;
     float m = -INFINITY, l = 0.f, rsum = 0.f, M = 0.f, invL = 0.f;
@@ -283,32 +313,49 @@ __global__ void __launch_bounds__(THREADS, 1)
           l = acc;
           m = mn;
         }
-      } else if (valid && k0 < N) {  // normalised visual columns
+      } else if (k0 < N) {  // normalised visual columns; uniform over the warp
         const int nv = min(32, N - k0);
+#pragma unroll
+        for (int q = 0; q < 32; ++q) v[q] = expf(v[q] * scale - M) * invL;
         if (nv == 32 && (N & 3) == 0) {
 #pragma unroll
           for (int q = 0; q < 32; q += 4) {
             const float4 z = *reinterpret_cast<const float4*>(zr + k0 + q);
-            float4 o;
-            o.x = expf(v[q] * scale - M) * invL;
-            o.y = expf(v[q + 1] * scale - M) * invL;
-            o.z = expf(v[q + 2] * scale - M) * invL;
-            o.w = expf(v[q + 3] * scale - M) * invL;
-            *reinterpret_cast<float4*>(arow + k0 + q) = o;
-            rsum = fmaf(o.x, sqrtf(z.x + sg2), rsum);
-            rsum = fmaf(o.y, sqrtf(z.y + sg2), rsum);
-            rsum = fmaf(o.z, sqrtf(z.z + sg2), rsum);
-            rsum = fmaf(o.w, sqrtf(z.w + sg2), rsum);
+            rsum = fmaf(v[q], sqrtf(z.x + sg2), rsum);
+            rsum = fmaf(v[q + 1], sqrtf(z.y + sg2), rsum);
+            rsum = fmaf(v[q + 2], sqrtf(z.z + sg2), rsum);
+            rsum = fmaf(v[q + 3], sqrtf(z.w + sg2), rsum);
           }
         } else {
 #pragma unroll
           for (int q = 0; q < 32; ++q)  // unrolled: v stays in registers
-            if (q < nv) {
-              const float p = expf(v[q] * scale - M) * invL;
-              arow[k0 + q] = p;
-              rsum = fmaf(p, sqrtf(zr[k0 + q] + sg2), rsum);
-            }
+            if (q < nv) rsum = fmaf(v[q], sqrtf(zr[k0 + q] + sg2), rsum);
         }
+        // transpose through shared memory, as in the fused kernel: eight lanes write
+        // each row's 128-byte line
+#pragma unroll
+        for (int c4 = 0; c4 < 8; ++c4)
+          *reinterpret_cast<float4*>(stg + lane * 32 + ((c4 ^ (lane & 7)) << 2)) =
+              make_float4(v[4 * c4], v[4 * c4 + 1], v[4 * c4 + 2], v[4 * c4 + 3]);
+        __syncwarp();
+        const int c4 = lane & 7, col = k0 + 4 * c4;
+#pragma unroll
+        for (int rr = 0; rr < 32; rr += 4) {
+          const int row = rr + (lane >> 3);
+          const float4 o = *reinterpret_cast<const float4*>(stg + row * 32 + ((c4 ^ (row & 7)) << 2));
+          const int ar = ctl->arow[quarter * 32 + row];
+          if (ar < 0 || col >= N) continue;
+          float* ap = A + (size_t)ar * N + col;
+          if ((N & 3) == 0 && col + 4 <= N) {
+            *reinterpret_cast<float4*>(ap) = o;
+          } else {
+            ap[0] = o.x;
+            if (col + 1 < N) ap[1] = o.y;
+            if (col + 2 < N) ap[2] = o.z;
+            if (col + 3 < N) ap[3] = o.w;
+          }
+        }
+        __syncwarp();  // the next tile reuses the staging
       }
     }
     if (mode == 0) {  // combine the column parts of every row, in a fixed order
@@ -379,8 +426,8 @@ __global__ void __launch_bounds__(FT_THREADS, 1)
   // written by the others once every CTA has arrived)
   asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");
   const int Tb = tg.T;
-  const int nkt = ceil_div(N + Tb, BM);
-  const int c0 = split * kt_per, c1 = min(nkt, c0 + kt_per);
+  const int nkt = ceil_div(N + Tb, BM), kt = split_tiles(nkt, nsplit);
+  const int c0 = split * kt, c1 = min(nkt, c0 + kt);
   const int iters = max(0, c1 - c0);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int qrow0 = (int)(((size_t)b * Hkv + g) * RQ + (size_t)tile * BM);
@@ -415,6 +462,11 @@ __global__ void __launch_bounds__(FT_THREADS, 1)
   const int j = valid ? R / Tb : 0, t = valid ? R % Tb : 0;
   const int h = g * grp + j;
   const int kvis = N + t + 1;
+
+  // the tile rows' places in A, once: the write pass stores every row in pieces by
+  // other lanes, and a division per piece cost more than the rest of that pass
+  if (warp < FE_WARPS && cq == 0)
+    ctl->arow[r] = valid ? (b * H + h) * Tmax + t : -1;
 
   if (warp == FE_WARPS) {  // ---------------- TMA producer
     int issued = 0;
@@ -580,9 +632,9 @@ __global__ void __launch_bounds__(FT_THREADS, 1)
       for (int rr = 0; rr < 32; rr += 4) {
         const int row = rr + (lane >> 3);
         const float4 o = *reinterpret_cast<const float4*>(stg + row * 32 + ((c4 ^ (row & 7)) << 2));
-        const int Rw = tile * BM + quarter * 32 + row;
-        if (Rw >= grp * Tb || col >= N) continue;
-        float* arow = A + (((size_t)b * H + g * grp + Rw / Tb) * Tmax + Rw % Tb) * N;
+        const int ar = ctl->arow[quarter * 32 + row];
+        if (ar < 0 || col >= N) continue;
+        float* arow = A + (size_t)ar * N;
         if ((N & 3) == 0 && col + 4 <= N) {
           *reinterpret_cast<float4*>(arow + col) = o;
         } else {
@@ -636,8 +688,7 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
       cudaSuccess)
     return e;
   const int nkb = dm.d / BK;
-  const size_t smem = msg_smem_bytes(nkb);
-  if ((e = set_smem_limit((const void*)k_message_tc, smem)) != cudaSuccess) return e;
+  if ((e = set_smem_limit((const void*)k_message_tc, msg_smem_bytes(nkb, 1))) != cudaSuccess) return e;
   const MsgSplit sp = msg_split(dm.B, dm.Hkv, RQ, dm.N, dm.T);
   dim3 grid(RQ / BM, dm.Hkv, dm.B * sp.n);
   const size_t fsmem = 1024 + fused_region_bytes(nkb) + sizeof(FusedCtl) +
@@ -658,6 +709,10 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
     attr[0].val.clusterDim.z = sp.n;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
+    if (sp.n > FUSED_PORTABLE &&
+        (e = cudaFuncSetAttribute((const void*)k_message_fused,
+                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+      return e;
     int ncl = 0;
     if (cudaOccupancyMaxActiveClusters(&ncl, (void*)k_message_fused, &cfg) == cudaSuccess && ncl > 0) {
       attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_wait
@@ -671,8 +726,8 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
   }
   if (launches) *launches = 2;
   for (int mode = 0; mode < 2; ++mode) {
-    launch_k(k_message_tc, grid, THREADS, smem, st, 1, qmap, kmap, dm.toff, dm.B, dm.N, dm.T, dm.H, dm.Hkv,
-                                              dm.d, RQ, mode, sp.kt_per, sp.n, s.mpart, s.zn2,
+    launch_k(k_message_tc, grid, THREADS, msg_smem_bytes(nkb, mode), st, 1, qmap, kmap, dm.toff, dm.B, dm.N, dm.T, dm.H, dm.Hkv,
+                                              dm.d, RQ, mode, sp.n, s.mpart, s.zn2,
                                               s.sigma, s.A, s.rs, s.status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

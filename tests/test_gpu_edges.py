@@ -114,3 +114,29 @@ def test_transport_sizes(B, gh, gw, T, K, D, Hkv, d, dtype, spread):
         if dtype == "bf16":
             bound = bound + ref.abs() * 2.0 ** -8
         assert bool(((oh[b, :K].double() - ref).abs() <= bound).all())
+
+
+# message slice: key splits that fill a cluster, exceed the portable cluster size and
+# exceed the largest one (two launches); query tiles that are ragged; keys that end
+# inside a tile, rows of A on 16 bytes and not
+@pytest.mark.parametrize("gh,gw,T,H,Hkv,B", [
+    (16, 8, [40], 4, 2, 1), (23, 41, [70, 3, 33], 6, 2, 3), (36, 37, [21], 28, 28, 12),
+    (66, 64, [9], 4, 1, 1), (128, 64, [5], 2, 1, 1)])
+def test_message_slice_splits(gh, gw, T, H, Hkv, B):
+    from paper_2608_02134_gb300 import workloads
+    from tests.test_gpu_clients import _gpu_clients
+    from oracle import gmc_oracle as O
+    wl = workloads.make("qwen", B=B, T=T * (B // len(T)), gh=gh, gw=gw, D=64, d=64, H=H, Hkv=Hkv, K=9)
+    C, traces, comp = _gpu_clients(wl)
+    p = O.params()
+    f = lambda a: np.asarray(a, dtype=np.float64)  # noqa: E731
+    for b in {0, B - 1}:
+        im, tr = wl.image(b), traces[b]
+        A = O.message_slice(f(im.queries), f(im.keys), wl.N)
+        Z, sigma = O.probe_values(f(im.values)[:wl.N], f(wl.probe()), H, p)
+        P, _ = O.grounded_clients(O.atom_norms(A, Z, sigma))
+        nu = O.query_weights(im.T, p)
+        ref = 0.5 * f(tr.omega)[:, None, None] * nu[None, :, None] * P
+        got = C[b, :H * im.T].reshape(H, im.T, wl.N)
+        err = np.abs(got - ref).max(2) / ref.max(2)
+        assert err.max() <= 1e-3, err.max()   # the bar of the client parity tests
