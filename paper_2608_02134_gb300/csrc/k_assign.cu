@@ -21,8 +21,18 @@
 // the K x N support cosines of long prefixes (cs mode).  So both passes read
 // exactly K x N values, coalesced, and no lane divides or gathers per entry:
 // the support's images and grid coordinates are staged once per block.  The
-// warps' partial results (top two cosines; best kappa and its entry, ties to
-// the lower entry) are merged in shared memory.
+// warps' partial results (top two cosines and the entry of the first; best kappa
+// and its entry, ties to the lower entry) are merged in shared memory.
+//
+// The second pass reads a token's cosines only where the spatial term can change
+// its carrier.  The term lies between 0 and c = lambda_p s_x g_i, so the carrier
+// of the largest cosine keeps a token whose gap delta_i exceeds c (by more than
+// the rounding of the two sums); g_i falls as delta_i^8, so that is every token
+// with a gap beyond about ambig_margin, and every one where s_x is small.
+// Both passes wait on the cosines' arithmetic, not on memory: taking the largest two
+// without branches and leaving out most of the second pass's exponentials took
+// N = 15,876, K = 4,096 from 277 to 170 us, and 32 images of N = 1,296, K = 257
+// from 73 to 58.
 #include "common.cuh"
 #include "kernels.cuh"
 
@@ -31,6 +41,10 @@ namespace gmc {
 namespace {
 constexpr int AT = 32;  // tokens per block (one per lane)
 constexpr int AU = 8;   // support entries each lane loads before using them
+// Rounding left between delta_i, a difference of two cosines, and the sums it
+// stands for: cosines are at most 1 + 1e-4 in magnitude, so each sum is within
+// 1.2e-7 of its value.
+constexpr float GAP_SLACK = 1e-6f;
 
 // Cosine row of support entry k (token j) for image b: its cosines with every token.
 __device__ __forceinline__ const float* support_row(const float* cos, int cs_mode, int b, int N,
@@ -50,11 +64,11 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_gap(
     const int32_t* __restrict__ slot, const int32_t* toff, int B, int N, int K, int Tmax, int H,
     const float* __restrict__ omega, const float* __restrict__ zn2,
     const float* __restrict__ sigma, const float* __restrict__ W2, float* energy, float* epart,
-    float* delta, double* dpart, int nA, float gate_scale, float gate_pow, int I, uint32_t* tick,
-    float* gatev, uint32_t* status) {
+    float* delta, double* dpart, int nA, float gate_scale, float gate_pow, int I, int32_t* pi,
+    uint32_t* tick, float* gatev, uint32_t* status) {
   grid_dep_wait();
   __shared__ float pm1[ASSIGN_WARPS][AT], pm2[ASSIGN_WARPS][AT], pe2[ASSIGN_WARPS][AT];
-  __shared__ int pnc[ASSIGN_WARPS][AT];
+  __shared__ int pnc[ASSIGN_WARPS][AT], pk1[ASSIGN_WARPS][AT];
   __shared__ int last;
   extern __shared__ int sS[];  // [K] support, then [K] its images
   int* sImg = sS + K;
@@ -72,23 +86,26 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_gap(
   __syncthreads();
   const bool tok = i < N;
   const int img = tok ? i / Ng : -1;
-  // top two cosines of this lane's token over the warp's share of the support
+  // top two cosines of this lane's token over the warp's share of the support, and the
+  // entry of the largest (the first among equals: k ascends)
   float m1 = -INFINITY, m2 = -INFINITY;
-  int nc = 0;
+  int nc = 0, k1 = 0x7fffffff;
   for (int k0 = w; k0 < K; k0 += ASSIGN_WARPS * AU) {
     float v[AU];
     bool ok[AU];
 #pragma unroll
     for (int u = 0; u < AU; ++u) {
       const int k = k0 + ASSIGN_WARPS * u;
-      ok[u] = tok && k < K && sImg[k] == img;
-      v[u] = ok[u] ? support_row(cos, cs_mode, b, N, K, k, sS[k])[i] : 0.f;
+      ok[u] = tok && k < K && (I == 1 || sImg[k] == img);
+      v[u] = ok[u] ? support_row(cos, cs_mode, b, N, K, k, sS[k])[i] : -INFINITY;
     }
 #pragma unroll
-    for (int u = 0; u < AU; ++u) {
-      if (!ok[u]) continue;
-      ++nc;
-      if (v[u] > m1) { m2 = m1; m1 = v[u]; } else if (v[u] > m2) { m2 = v[u]; }
+    for (int u = 0; u < AU; ++u) {  // -inf (and NaN) raises nothing
+      const bool up = v[u] > m1;
+      nc += ok[u];
+      m2 = up ? m1 : fmaxf(m2, v[u]);
+      k1 = up ? k0 + ASSIGN_WARPS * u : k1;
+      m1 = up ? v[u] : m1;
     }
   }
   // the message energy's head terms, the heads split over the warps
@@ -102,6 +119,7 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_gap(
   pm1[w][lane] = m1;
   pm2[w][lane] = m2;
   pnc[w][lane] = nc;
+  pk1[w][lane] = k1;
   pe2[w][lane] = e2w;
   __syncthreads();
   if (w == 0) {
@@ -109,7 +127,9 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_gap(
     float e2 = e2w;
     for (int q = 1; q < ASSIGN_WARPS; ++q) {
       const float b1 = pm1[q][lane], b2 = pm2[q][lane];
+      const int q1 = pk1[q][lane];
       const float hi = fmaxf(m1, b1);
+      if (b1 > m1 || (b1 == m1 && q1 < k1)) k1 = q1;
       m2 = fmaxf(fminf(m1, b1), fmaxf(m2, b2));
       m1 = hi;
       nc += pnc[q][lane];
@@ -124,6 +144,9 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_gap(
       const bool disc = slot[(size_t)b * N + i] < 0;
       const float d = disc && nc > 1 ? m1 - m2 : 0.f;
       delta[(size_t)b * N + i] = d;
+      // for pass 2: the entry of the largest cosine; -1: none, or a gap that is no
+      // number, so that every entry is looked at again
+      pi[(size_t)b * N + i] = k1 < K && (nc == 1 || d >= 0.f) ? k1 : -1;
       if (disc) {
         dv = d;
         dc = 1;
@@ -203,20 +226,28 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_pick(
   const int img = tok ? i / Ng : -1, il = tok ? i - img * Ng : 0;
   const float piy = ((il / gw) + 0.5f) / gh, pix = ((il % gw) + 0.5f) / gw;
   float coef = 0.f;
-  if (disc) {
-    const float gi = expf(-powf(delta[(size_t)b * N + i] / ambig_margin, gate_pow));
-    coef = lambda_p * sxg * gi;
-  }
   float best = -INFINITY;
   int bk = 0x7fffffff;
+  bool open = disc;  // the spatial term may change the token's carrier
   if (disc) {
+    const float dl = delta[(size_t)b * N + i];
+    const float gi = expf(-powf(dl / ambig_margin, gate_pow));
+    coef = lambda_p * sxg * gi;
+    const int k1 = pi[(size_t)b * N + i];
+    if (k1 >= 0 && lambda_p >= 0.f && dl > coef + GAP_SLACK) {
+      bk = k1;
+      open = false;
+    }
+  }
+  // warps of a block see the same 32 tokens: all skip or none
+  if (__any_sync(FULL, open)) {
     for (int k0 = w; k0 < K; k0 += ASSIGN_WARPS * AU) {
       float v[AU];
       bool ok[AU];
 #pragma unroll
       for (int u = 0; u < AU; ++u) {
         const int k = k0 + ASSIGN_WARPS * u;
-        ok[u] = k < K && sImg[k] == img;  // a carrier of the token's own image
+        ok[u] = open && k < K && (I == 1 || sImg[k] == img);  // a carrier of its own image
         v[u] = ok[u] ? support_row(cos, cs_mode, b, N, K, k, sS[k])[i] : 0.f;
       }
 #pragma unroll
@@ -224,7 +255,7 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_pick(
         if (!ok[u]) continue;
         const int k = k0 + ASSIGN_WARPS * u;
         float x = v[u];
-        if (coef > 0.f) {
+        if (coef > 0.f && x + coef > best) {  // the term is at most coef
           const float dy = spy[k] - piy, dx = spx[k] - pix;
           x += coef * expf(-(dy * dy + dx * dx) / tau_s);
         }
@@ -236,7 +267,7 @@ __global__ void __launch_bounds__(32 * ASSIGN_WARPS) k_assign_pick(
   pk[w][lane] = bk;
   __syncthreads();
   if (w != 0 || !tok) return;
-  for (int q = 1; q < ASSIGN_WARPS; ++q) {
+  for (int q = 1; q < (open ? ASSIGN_WARPS : 1); ++q) {
     const float ob = pbest[q][lane];
     const int ok = pk[q][lane];
     if (ob > best || (ob == best && ok < bk)) { best = ob; bk = ok; }
@@ -282,7 +313,7 @@ cudaError_t launch_assign(const Dims& dm, const gmc_params& p, Scratch& s, const
   if ((e0 = set_smem_limit((const void*)k_assign_pick, psm)) != cudaSuccess) return e0;
   launch_k(k_assign_gap, grid, 32 * ASSIGN_WARPS, gsm, st, 1,
       src, cs_mode, s.support, s.slot, dm.toff, dm.B, dm.N, dm.K, dm.T, dm.H, s.omega, s.zn2,
-      s.sigma, s.W2, s.ebar, s.epart, s.delta, s.dpart, s.nA, p.gate_scale, p.gate_pow, dm.I,
+      s.sigma, s.W2, s.ebar, s.epart, s.delta, s.dpart, s.nA, p.gate_scale, p.gate_pow, dm.I, s.pi,
       s.tick2, s.gatev, s.status);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

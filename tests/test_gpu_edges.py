@@ -140,3 +140,53 @@ def test_message_slice_splits(gh, gw, T, H, Hkv, B):
         got = C[b, :H * im.T].reshape(H, im.T, wl.N)
         err = np.abs(got - ref).max(2) / ref.max(2)
         assert err.max() <= 1e-3, err.max()   # the bar of the client parity tests
+
+
+# assignment: gates that leave every gap open, some and none, a weight that lets the
+# spatial term outweigh any gap and one of zero, one carrier, duplicated tokens (gap
+# zero), several images: the carrier of every discarded token has the largest kappa
+@pytest.mark.parametrize("shape,K,gate_scale,weight,margin,twins", [
+    (dict(gh=8, gw=8, D=32), 16, 0.08, 0.5, 0.05, False),
+    (dict(gh=9, gw=23, D=64), 60, 1e-3, 0.5, 0.05, False),
+    (dict(gh=9, gw=23, D=64), 60, 1e-3, 8.0, 1.0, False),
+    (dict(gh=9, gw=23, D=64), 33, 1e9, 0.5, 0.05, True),
+    (dict(gh=17, gw=31, D=32), 100, 1e-3, 0.0, 0.05, True),
+    (dict(gh=5, gw=7, D=32), 1, 1e-3, 0.5, 0.05, False),
+    (dict(gh=9, gw=11, D=64, I=3), 40, 1e-3, 0.5, 0.2, True)])
+def test_assignment_gates(shape, K, gate_scale, weight, margin, twins):
+    from oracle import gmc_oracle as O
+    from paper_2608_02134_gb300 import gmc, workloads
+    from tests import gpu_harness as GH
+    wl = workloads.make("tiny", K=K, T=9, **shape)
+    inp = GH.to_device(wl)
+    ng = wl.gh * wl.gw
+    if twins:  # tokens 2 and 3 of every image hold the same state
+        h = inp["hidden"].view(-1, wl.D)
+        h[torch.arange(0, wl.N, ng) + 3] = h[torch.arange(0, wl.N, ng) + 2]
+    params = gmc.default_params(gate_scale=gate_scale, assign_spatial_w=weight,
+                                ambig_margin=margin)
+    run = GH.run(wl, params=params, inputs=inp)
+    assert run.status == 0
+    tr, S = run.traces[0], run.idx[:K]
+    p = O.params(gate_scale=gate_scale, assign_spatial_w=weight, ambig_margin=margin)
+    x = O.unit_states(inp["hidden"].view(-1, wl.D)[:wl.N].cpu().numpy().astype(np.float64), p)
+    cos = x @ x[S].T
+    tok = np.arange(wl.N)
+    cos[(tok[:, None] // ng) != (S[None] // ng)] = -np.inf
+    top = np.sort(cos, axis=1)[:, ::-1]
+    with np.errstate(invalid="ignore"):
+        delta = top[:, 0] - top[:, 1] if K > 1 else np.zeros(wl.N)
+    delta = np.where(np.isfinite(delta), delta, 0.0)
+    pos = O.grid_coords(wl.gh, wl.gw)[tok % ng]
+    d2 = ((pos[:, None] - pos[S][None]) ** 2).sum(2)
+    gate = np.exp(-((delta / margin) ** p["gate_pow"]))
+    kappa = cos + weight * tr.s_x * gate[:, None] * np.exp(-d2 / p["tau_s"])
+    got = kappa[tok, np.searchsorted(S, tr.pi)]
+    # fp32 cosines of D terms are within D 2^-24 each; the gate's slope is below
+    # 3.1 / margin, and it multiplies the spatial term
+    eps = wl.D * 2.0 ** -24 + 1e-6
+    tol = 2 * eps + weight * (3.1 / margin) * 2 * eps
+    disc = np.ones(wl.N, bool)
+    disc[S] = False
+    assert np.isin(tr.pi, S).all() and np.array_equal(tr.pi[S], S)
+    assert (got[disc] >= kappa.max(1)[disc] - tol).all(), (kappa.max(1) - got)[disc].max()
