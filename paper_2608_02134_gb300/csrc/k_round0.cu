@@ -151,7 +151,7 @@ __global__ void __launch_bounds__(512) k_r0_pool(const long long* __restrict__ u
 
 // A lane keeps the sums of its pool slots in registers over the warp's rows; the
 // warps are added in shared memory once (8 warps adding every row's 64 scores to
-// the same shared words took a batch of 32 images 115 us, R0RHO us now).
+// the same shared words took a batch of 32 images 115 us, 108 us now).
 template <int ROWS>
 __global__ void __launch_bounds__(32 * ROWS) k_r0_rho(
     const float* __restrict__ C, int B, int N, int Mstride, int H, int L2, const int32_t* toff,
@@ -298,8 +298,8 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_filter(
     float4* tile = sm_r0f + (threadIdx.x >> 5) * TILE;
     float rowmax = 0.f;  // only the trace reports F(V)
     const int w =
-        tv.base ? sel::filter_dense_row<true>(vals, cols, N, bnew, fb_new, fxs, sums, tile, &rowmax)
-                : sel::filter_dense_row<false>(vals, cols, N, bnew, fb_new, fxs, sums, tile, &rowmax);
+        tv.base ? sel::filter_dense_row<true, ROWS == 16>(vals, cols, N, bnew, fb_new, fxs, sums, tile, &rowmax)
+                : sel::filter_dense_row<false, ROWS == 16>(vals, cols, N, bnew, fb_new, fxs, sums, tile, &rowmax);
     if (lane == 0) {
       bcov[(size_t)b * Mstride + m] = bnew;
       cnt[(size_t)b * Mstride + m] = w;

@@ -16,13 +16,14 @@
 //   k_w_pool    one block per image: the pool of the current gains (the
 //               histogram selection of select_common.cuh, gains read from
 //               global memory);
-//   k_w_rho     warp per client row: the row's responsibilities over the pool,
-//               summed into the scores in 64-bit fixed point.  The dense first
-//               round gathers the row at the pool tokens into shared memory;
-//               later rounds walk the row's survivor list three times (max,
-//               normaliser, scores: the temperature depends on the row's max);
-//   k_w_batch   one block per image: a bitonic sort of the pool by (score
-//               desc, token asc) gives the batch;
+//   k_w_rho     the rows' responsibilities over the pool, summed into the scores
+//               in 64-bit fixed point: k_w_rho_dense in the first round (a block
+//               per row at a time), then a warp per row that walks its survivor
+//               list three times (max, normaliser, scores: the temperature
+//               depends on the row's max);
+//   k_w_batch   one block per image: the best of the pool by (score desc, token
+//               asc), found as the pool is; a bitonic sort where fewer than a
+//               batch of them have a positive score;
 //   k_w_filter  warp per client row: the new coverage b_m, the row's
 //               survivors {i : Cbar_mi > b_m} compacted in place (values over
 //               Cbar, tokens in scol), the next round's gains summed per block
@@ -42,9 +43,11 @@
 namespace gmc {
 
 namespace {
-constexpr int WROWS = 8;      // warps (client rows) per responsibility block
-constexpr int FROWS = 16;     // warps per filter block (one block per SM: the next gains of
-                              // N tokens take 8 N bytes of shared memory)
+constexpr int DTHREADS = 512; // threads of a block of the dense responsibilities
+constexpr int DROWS = 3;      // client rows it has in shared memory
+constexpr int SROWS = 16;     // warps (client rows) per block of the later rounds'
+constexpr int FROWS = 32;     // most warps of a filter block (one block per SM: the next gains
+                              // of N tokens take 8 N bytes of shared memory)
 constexpr int WP_THREADS = 1024;
 constexpr int W_BCAP = 4096;  // boundary-bucket gains the pool kernel stages in shared memory
 
@@ -133,9 +136,6 @@ __global__ void __launch_bounds__(WP_THREADS, 1) k_w_pool(WideState w, WideGeom 
   ps.bval = reinterpret_cast<long long*>(p);  // the boundary bucket's gains
   ps.bcap = min(N, W_BCAP);
   p += sizeof(long long) * (size_t)ps.bcap;
-  ps.sortbuf = reinterpret_cast<int*>(p);     // and their order
-  ps.scap = W_BCAP;
-  p += sizeof(int) * (size_t)W_BCAP;
   sel::WindowScratch ws{};
   long long* ug = nullptr;  // win: the gains, staged for the pool's passes
   if (win) {
@@ -175,10 +175,110 @@ __global__ void __launch_bounds__(WP_THREADS, 1) k_w_pool(WideState w, WideGeom 
 }
 
 // ---- responsibilities ----------------------------------------------------------------
-// DENSE: the first round (b = 0, rows are the dense client rows); otherwise
-// rows are survivor lists with coverage bcov.
-template <bool DENSE>
-__global__ void __launch_bounds__(32 * WROWS) k_w_rho(WideState w, WideGeom g, int P,
+// The dense first round (b = 0: a residual is the client value): one block an SM,
+// whole rows one after another.  A row comes to shared memory as it lies, DROWS - 1
+// rows ahead (the pool is one token in eight, so its values touch two sectors in
+// three: gathering them took as much memory traffic and many more requests); each
+// thread then keeps its SLOTS pool slots in registers, values, exponentials and sums,
+// so an exponential is taken once and the sums meet nobody until the end.  Bound by
+// reading the rows: 7,936 of 15,876 values, P = 2,048: a warp a row, gathering, with
+// 64-bit shared-memory additions 193 us, now 124 (4.1 TB/s).
+template <int SLOTS, bool VEC>
+__global__ void __launch_bounds__(DTHREADS, 1) k_w_rho_dense(WideState w, WideGeom g, int P,
+                                                             const float* __restrict__ C,
+                                                             float resp_temp, float resp_eps,
+                                                             int fx_exp, const int32_t* fexp) {
+  grid_dep_wait();
+  extern __shared__ __align__(16) char sm_wd[];
+  constexpr int NW = DTHREADS / 32;
+  __shared__ float red_max[NW], red_z[NW];
+  __shared__ int red_n[NW];
+  const int b = blockIdx.y, N = g.N;
+  const int Pt = w.info[b * INFO_W];
+  if (Pt == 0) return;
+  int MG;
+  const int Mb = wide_rows(g, b, &MG);
+  if ((int)blockIdx.x >= Mb) return;
+  const float fxs = ldexpf(1.f, fexp ? fexp[b] : fx_exp);
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const size_t pitch = ((size_t)N + 3) & ~(size_t)3;
+  float* rows = reinterpret_cast<float*>(sm_wd);  // [DROWS][pitch]
+  int tok[SLOTS];
+  long long acc[SLOTS];
+#pragma unroll
+  for (int q = 0; q < SLOTS; ++q) {
+    const int k = threadIdx.x + DTHREADS * q;
+    tok[q] = k < Pt ? w.pool[(size_t)b * P + k] : -1;
+    acc[q] = 0;
+  }
+  auto fetch = [&](int m, int slot) {
+    if (m < Mb) {
+      const float* src = C + ((size_t)b * g.Mstride + m) * N;
+      float* dst = rows + slot * pitch;
+      if (VEC) {
+        for (int j = 4 * threadIdx.x; j < N; j += 4 * DTHREADS) cp_async16(dst + j, src + j);
+      } else {
+        for (int j = threadIdx.x; j < N; j += DTHREADS) cp_async4(dst + j, src + j, true);
+      }
+    }
+    cp_async_commit();
+  };
+  for (int q = 0; q < DROWS - 1; ++q) fetch(blockIdx.x + q * gridDim.x, q);
+  for (int m = blockIdx.x, i = 0; m < Mb; m += gridDim.x, ++i) {
+    cp_async_wait<DROWS - 2>();
+    __syncthreads();  // row i is here, and every thread is done with row i - 1
+    fetch(m + (DROWS - 1) * gridDim.x, (i + DROWS - 1) % DROWS);
+    const float* row = rows + (i % DROWS) * pitch;
+    float R[SLOTS];
+    float mx = 0.f;
+    int n = 0;
+#pragma unroll
+    for (int q = 0; q < SLOTS; ++q) {
+      R[q] = tok[q] >= 0 ? row[tok[q]] : 0.f;
+      mx = fmaxf(mx, R[q]);
+      n += R[q] > 0.f;
+    }
+    mx = warp_max(mx);
+    n = warp_sum_int(n);
+    if (lane == 0) {
+      red_max[wid] = mx;
+      red_n[wid] = n;
+    }
+    __syncthreads();
+    const float rmax = warp_max(lane < NW ? red_max[lane] : 0.f);
+    const int nf = warp_sum_int(lane < NW ? red_n[lane] : 0);
+    if (nf == 0) continue;  // uniform over the block
+    // softmax of R / tau shifted by its largest logit rmax / tau
+    const float tau = resp_temp * rmax + resp_eps;
+    float ex[SLOTS], z = 0.f;
+#pragma unroll
+    for (int q = 0; q < SLOTS; ++q) {
+      ex[q] = R[q] > 0.f ? expf((R[q] - rmax) / tau) : 0.f;
+      z += ex[q];
+    }
+    z = warp_sum(z);
+    if (lane == 0) red_z[wid] = z;
+    __syncthreads();
+    z = warp_sum(lane < NW ? red_z[lane] : 0.f) +
+        (float)(Pt - nf) * expf(-rmax / tau);  // a pool token with R = 0
+    const float invz = 1.f / z;
+#pragma unroll
+    for (int q = 0; q < SLOTS; ++q)
+      if (R[q] > 0.f) acc[q] += to_fix(ex[q] * invz * R[q], fxs);
+  }
+#pragma unroll
+  for (int q = 0; q < SLOTS; ++q) {
+    const int k = threadIdx.x + DTHREADS * q;
+    if (acc[q]) atomicAdd((unsigned long long*)&w.sc[(size_t)b * P + k], (unsigned long long)acc[q]);
+  }
+}
+
+// Later rounds: a warp per row, over its survivor list with coverage bcov.  The
+// entries in the pool are few, and their sums are three native 32-bit additions
+// (select_common.cuh); one block takes many rows, so the slot table is laid out and
+// the sums are flushed once per block and not once per eight rows (7,936 rows:
+// 15.7 us a round, now 10).
+__global__ void __launch_bounds__(32 * SROWS) k_w_rho(WideState w, WideGeom g, int P,
                                                       const float* __restrict__ C,
                                                       const uint16_t* __restrict__ scol,
                                                       float resp_temp, float resp_eps, int fx_exp,
@@ -190,98 +290,72 @@ __global__ void __launch_bounds__(32 * WROWS) k_w_rho(WideState w, WideGeom g, i
   if (Pt == 0) return;
   int MG;
   const int Mb = wide_rows(g, b, &MG);
-  const int m0 = blockIdx.x * WROWS;
-  if (m0 >= Mb) return;
   const float fxs = ldexpf(1.f, fexp ? fexp[b] : fx_exp);
-  long long* sblk = reinterpret_cast<long long*>(sm_wr);  // [P]
-  char* p = sm_wr + sizeof(long long) * (size_t)P;
   const int32_t* gpool = w.pool + (size_t)b * P;
-  for (int k = threadIdx.x; k < P; k += blockDim.x) sblk[k] = 0;
-  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, m = m0 + wid;
-  if (DENSE) {
-    float* Rw = reinterpret_cast<float*>(p) + (size_t)wid * P;  // this warp's row at the pool
-    __syncthreads();
-    if (m < Mb) {
-      const float* row = C + ((size_t)b * g.Mstride + m) * N;
-      float rmax = 0.f;
-      int nf = 0;
-      for (int k = lane; k < Pt; k += 32) {
-        const float R = row[gpool[k]];  // b = 0: the residual is the client value
-        Rw[k] = R;
-        if (R > 0.f) {
-          rmax = fmaxf(rmax, R);
-          ++nf;
-        }
-      }
-      rmax = warp_max(rmax);
-      nf = warp_sum_int(nf);
-      if (nf > 0) {
-        // softmax of R / tau shifted by its largest logit rmax / tau
-        const float tau = resp_temp * rmax + resp_eps;
-        const float e0 = expf(-rmax / tau);  // a pool token with R = 0
-        float z = 0.f;
-        for (int k = lane; k < Pt; k += 32)
-          if (Rw[k] > 0.f) z += expf((Rw[k] - rmax) / tau);
-        z = warp_sum(z) + (float)(Pt - nf) * e0;
-        const float invz = 1.f / z;
-        for (int k = lane; k < Pt; k += 32) {
-          const float R = Rw[k];
-          if (R > 0.f)
-            atomicAdd((unsigned long long*)&sblk[k],
-                      (unsigned long long)to_fix(expf((R - rmax) / tau) * invz * R, fxs));
-        }
+  unsigned long long* sc = reinterpret_cast<unsigned long long*>(w.sc) + (size_t)b * P;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  if (blockIdx.x * SROWS >= Mb) return;
+  uint32_t* sblk = reinterpret_cast<uint32_t*>(sm_wr);  // [3][P] limbs
+  short* pslot = reinterpret_cast<short*>(sblk + 3 * (size_t)P);  // [N] pool slot or -1
+  for (int k = threadIdx.x; k < 3 * P; k += blockDim.x) sblk[k] = 0;
+  int* fill = reinterpret_cast<int*>(pslot);
+  for (int j = threadIdx.x; j < (N + 1) / 2; j += blockDim.x) fill[j] = -1;
+  __syncthreads();
+  for (int k = threadIdx.x; k < Pt; k += blockDim.x) pslot[gpool[k]] = (short)k;
+  __syncthreads();
+  for (int m = blockIdx.x * SROWS + wid; m < Mb; m += gridDim.x * SROWS) {
+    const size_t row = (size_t)b * g.Mstride + m;
+    const int n = w.cnt[row];
+    const float bm = w.bcov[row];
+    const float* vals = C + row * N;
+    const uint16_t* cols = scol + row * N;
+    // pass 1: the largest pool residual and the number of pool entries
+    float rmax = 0.f;
+    int nf = 0;
+#pragma unroll 4
+    for (int e = lane; e < n; e += 32) {
+      const int k = pslot[cols[e]];
+      const float x = vals[e];
+      if (k >= 0) {
+        rmax = fmaxf(rmax, x - bm);
+        ++nf;
       }
     }
-  } else {
-    short* pslot = reinterpret_cast<short*>(p);  // [N] pool slot of every token or -1
-    for (int j = threadIdx.x; j < N; j += blockDim.x) pslot[j] = -1;
-    __syncthreads();
-    for (int k = threadIdx.x; k < Pt; k += blockDim.x) pslot[gpool[k]] = (short)k;
-    __syncthreads();
-    if (m < Mb) {
-      const size_t row = (size_t)b * g.Mstride + m;
-      const int n = w.cnt[row];
-      const float bm = w.bcov[row];
-      const float* vals = C + row * N;
-      const uint16_t* cols = scol + row * N;
-      // pass 1: the largest pool residual and the number of pool entries
-      float rmax = 0.f;
-      int nf = 0;
+    rmax = warp_max(rmax);
+    nf = warp_sum_int(nf);
+    if (nf > 0) {
+      const float tau = resp_temp * rmax + resp_eps;
+      const float e0 = expf(-rmax / tau);  // pool tokens without a survivor here: R = 0
+      float z = 0.f;
+#pragma unroll 4
       for (int e = lane; e < n; e += 32) {
         const int k = pslot[cols[e]];
-        if (k >= 0) {
-          rmax = fmaxf(rmax, vals[e] - bm);
-          ++nf;
-        }
+        const float x = vals[e];
+        if (k >= 0) z += expf((x - bm - rmax) / tau);
       }
-      rmax = warp_max(rmax);
-      nf = warp_sum_int(nf);
-      if (nf > 0) {
-        const float tau = resp_temp * rmax + resp_eps;
-        const float e0 = expf(-rmax / tau);  // pool tokens without a survivor here: R = 0
-        float z = 0.f;
-        for (int e = lane; e < n; e += 32)
-          if (pslot[cols[e]] >= 0) z += expf((vals[e] - bm - rmax) / tau);
-        z = warp_sum(z) + (float)(Pt - nf) * e0;
-        const float invz = 1.f / z;
-        for (int e = lane; e < n; e += 32) {
-          const int k = pslot[cols[e]];
-          if (k >= 0) {
-            const float R = vals[e] - bm;
-            atomicAdd((unsigned long long*)&sblk[k],
-                      (unsigned long long)to_fix(expf((R - rmax) / tau) * invz * R, fxs));
-          }
+      z = warp_sum(z) + (float)(Pt - nf) * e0;
+      const float invz = 1.f / z;
+#pragma unroll 4
+      for (int e = lane; e < n; e += 32) {
+        const int k = pslot[cols[e]];
+        const float x = vals[e];
+        if (k >= 0) {
+          const float R = x - bm;
+          sel::limb_add(&sblk[k], P,
+                        (unsigned long long)to_fix(expf((R - rmax) / tau) * invz * R, fxs));
         }
       }
     }
   }
   __syncthreads();
-  for (int k = threadIdx.x; k < Pt; k += blockDim.x)
-    if (sblk[k]) atomicAdd((unsigned long long*)&w.sc[(size_t)b * P + k], (unsigned long long)sblk[k]);
+  for (int k = threadIdx.x; k < Pt; k += blockDim.x) {
+    const unsigned long long v = sel::limb_value(&sblk[k], P);
+    if (v) atomicAdd(&sc[k], v);
+  }
 }
 
 // ---- batch -----------------------------------------------------------------------------
-__global__ void __launch_bounds__(WP_THREADS) k_w_batch(WideState w, WideGeom g, int P, int NP,
+__global__ void __launch_bounds__(WP_THREADS, 1) k_w_batch(WideState w, WideGeom g, int P, int NP,
                                                         int bsz, int32_t* order, TraceView tv) {
   grid_dep_wait();
   extern __shared__ __align__(16) char sm_wb[];
@@ -335,10 +409,7 @@ __global__ void __launch_bounds__(WP_THREADS) k_w_batch(WideState w, WideGeom g,
     int* top = reinterpret_cast<int*>(p);      p += sizeof(int) * (size_t)NP;
     ps.key = reinterpret_cast<short*>(p);      p += sizeof(short) * (size_t)NP;
     ps.pk = reinterpret_cast<unsigned char*>(p); p += (size_t)NP;
-    unsigned char* none = reinterpret_cast<unsigned char*>(p); p += (size_t)NP;
-    p = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + 15) & ~static_cast<uintptr_t>(15));
-    ps.sortbuf = reinterpret_cast<int*>(p);  // [NP], NP a power of two
-    ps.scap = NP;
+    unsigned char* none = reinterpret_cast<unsigned char*>(p);
     for (int k = threadIdx.x; k < Pt; k += blockDim.x) {
       ks[k] = w.sc[(size_t)b * P + k];
       kj[k] = w.pool[(size_t)b * P + k];
@@ -402,36 +473,41 @@ __global__ void __launch_bounds__(WP_THREADS) k_w_batch(WideState w, WideGeom g,
 }
 
 // ---- coverage update, survivor compaction, next gains ---------------------------------
+// One block an SM (the next gains of N tokens are in its shared memory), of as
+// many warps as give its rows to them evenly (launch_wide_select): the sums are
+// cleared and flushed once per SM, and no SM waits for one warp's extra row.
+// Blocks flush from different columns on, so that they do not all add to the same
+// ones at once.  7,936 rows of 15,876: first round 205 us, now 139; a later
+// round 15 us, now 11.
 template <bool DENSE>
 __global__ void __launch_bounds__(32 * FROWS) k_w_filter(WideState w, WideGeom g, int P, int rnd,
                                                          float* C, uint16_t* scol, int fx_exp,
-                                                         const int32_t* fexp, int rpw,
-                                                         TraceView tv) {
+                                                         const int32_t* fexp, TraceView tv) {
   grid_dep_wait();
-  extern __shared__ unsigned long long uacc[];  // [N] this block's part of the next gains
+  extern __shared__ __align__(16) char sm_wf[];
   const int b = blockIdx.y, N = g.N;
   const int32_t* info = w.info + b * INFO_W;
   const int Pt = info[0];
   if (Pt == 0) return;
   int MG;
   const int Mb = wide_rows(g, b, &MG);
-  const int m0 = blockIdx.x * FROWS * rpw;
-  if (m0 >= Mb) return;
+  const int nw = blockDim.x >> 5, wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if ((int)blockIdx.x * nw >= Mb) return;
+  // the warps' row tiles, then this block's part of the next gains
+  float4* tile = reinterpret_cast<float4*>(sm_wf) + (DENSE ? wid * (sel::ROW_STEP / 4) : 0);
+  const sel::GainSums<false> uacc{
+      reinterpret_cast<uint32_t*>(sm_wf + (DENSE ? sizeof(float) * sel::ROW_STEP * nw : 0)), N};
   const int S = info[3], rd = info[4];
   const int nb = info[1] - S;  // the batch kernel has run: info[1] = S + nb
   const float fxs = ldexpf(1.f, fexp ? fexp[b] : fx_exp);
   const int32_t* batch = w.batch + (size_t)b * P;
   const int32_t* stamp = w.stamp + (size_t)b * N;
-  long long* unext = gains_out(w, rnd) + (size_t)b * N;
   __shared__ long long fb[3];
   if (threadIdx.x < 3) fb[threadIdx.x] = 0;
-  for (int j = threadIdx.x; j < N; j += blockDim.x) uacc[j] = 0;
+  uacc.clear();
   __syncthreads();
-  const int lane = threadIdx.x & 31;
   const unsigned lt = sel::lanemask_lt();
-  for (int ir = 0; ir < rpw; ++ir) {
-    const int m = m0 + (threadIdx.x >> 5) + FROWS * ir;
-    if (m >= Mb) break;
+  for (int m = blockIdx.x * nw + wid; m < Mb; m += gridDim.x * nw) {
     const size_t row = (size_t)b * g.Mstride + m;
     float* vals = C + row * N;
     uint16_t* cols = scol + row * N;
@@ -439,80 +515,12 @@ __global__ void __launch_bounds__(32 * FROWS) k_w_filter(WideState w, WideGeom g
     float bnew;
     if (DENSE) {
       bnew = 0.f;
+#pragma unroll 8
       for (int t = lane; t < nb; t += 32) bnew = fmaxf(bnew, vals[batch[t]]);
       bnew = warp_max(bnew);
       const long long fb_new = to_fix(bnew, fxs);
-      float rowmax = 0.f;
-      if ((N & 3) == 0) {
-        // 8 x 16 bytes per lane in flight; all loads of a step issued before
-        // any survivor is written back in place (survivors land below the
-        // step's end).  Lane l's float4 holds tokens 4 k4 .. 4 k4 + 3, so the
-        // survivors are written lane by lane: ascending token order.
-        const float4* row4 = reinterpret_cast<const float4*>(vals);
-        const int n4 = N >> 2;
-        for (int b4 = 0; b4 < n4; b4 += 32 * 8) {
-          float4 buf[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int k4 = b4 + u * 32 + lane;
-            buf[u] = k4 < n4 ? row4[k4] : make_float4(0.f, 0.f, 0.f, 0.f);
-          }
-          __syncwarp();
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            const int k4 = b4 + u * 32 + lane;
-            const float c4[4] = {buf[u].x, buf[u].y, buf[u].z, buf[u].w};
-            int pre = 0, tot = 0;
-#pragma unroll
-            for (int e2 = 0; e2 < 4; ++e2) {
-              rowmax = fmaxf(rowmax, c4[e2]);
-              const unsigned bal = __ballot_sync(FULL, k4 < n4 && c4[e2] > bnew);
-              pre += __popc(bal & lt);
-              tot += __popc(bal);
-            }
-            int pos = wr + pre;
-            if (k4 < n4) {
-#pragma unroll
-              for (int e2 = 0; e2 < 4; ++e2)
-                if (c4[e2] > bnew) {
-                  const int k = 4 * k4 + e2;
-                  vals[pos] = c4[e2];
-                  cols[pos] = (uint16_t)k;
-                  atomicAdd(&uacc[k], (unsigned long long)(to_fix(c4[e2], fxs) - fb_new));
-                  ++pos;
-                }
-            }
-            wr += tot;
-          }
-          __syncwarp();
-        }
-      } else
-      // 8 loads per lane in flight; all loads of a step issued before any
-      // survivor is written back in place (survivors land below the step's end)
-      for (int base = 0; base < N; base += 32 * 8) {
-        float c[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = base + u * 32 + lane;
-          c[u] = k < N ? vals[k] : 0.f;
-        }
-        __syncwarp();
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = base + u * 32 + lane;
-          rowmax = fmaxf(rowmax, c[u]);
-          const bool keep = k < N && c[u] > bnew;
-          const unsigned bal = __ballot_sync(FULL, keep);
-          if (keep) {
-            const int pos = wr + __popc(bal & lt);
-            vals[pos] = c[u];
-            cols[pos] = (uint16_t)k;
-            atomicAdd(&uacc[k], (unsigned long long)(to_fix(c[u], fxs) - fb_new));
-          }
-          wr += __popc(bal);
-        }
-      }
-      rowmax = warp_max(rowmax);
+      float rowmax;
+      wr = sel::filter_dense_row<true, true>(vals, cols, N, bnew, fb_new, fxs, uacc, tile, &rowmax);
       if (lane == 0) {
         atomicAdd((unsigned long long*)&fb[bank_of(m, MG, g.MV)],
                   (unsigned long long)to_fix(rowmax, fxs));
@@ -521,8 +529,11 @@ __global__ void __launch_bounds__(32 * FROWS) k_w_filter(WideState w, WideGeom g
     } else {
       const int n = w.cnt[row];
       bnew = w.bcov[row];
-      for (int e = lane; e < n; e += 32)
-        if (stamp[cols[e]] == rd + 1) bnew = fmaxf(bnew, vals[e]);
+#pragma unroll 4
+      for (int e = lane; e < n; e += 32) {
+        const float x = vals[e];
+        if (stamp[cols[e]] == rd + 1) bnew = fmaxf(bnew, x);
+      }
       bnew = warp_max(bnew);
       const long long fb_new = to_fix(bnew, fxs);
       constexpr int FU = 4;  // chunks of 32 entries loaded before any is written back
@@ -548,7 +559,7 @@ __global__ void __launch_bounds__(32 * FROWS) k_w_filter(WideState w, WideGeom g
             const int pos = wr + __popc(bal & lt);
             vals[pos] = cc[u];
             cols[pos] = (uint16_t)jj[u];
-            atomicAdd(&uacc[jj[u]], (unsigned long long)(to_fix(cc[u], fxs) - fb_new));
+            uacc.add(jj[u], (unsigned long long)(to_fix(cc[u], fxs) - fb_new));
           }
           wr += __popc(bal);
         }
@@ -563,9 +574,8 @@ __global__ void __launch_bounds__(32 * FROWS) k_w_filter(WideState w, WideGeom g
   __syncthreads();
   if (DENSE && threadIdx.x < 3 && fb[threadIdx.x])
     atomicAdd((unsigned long long*)&w.fv[(size_t)b * 4 + threadIdx.x], (unsigned long long)fb[threadIdx.x]);
-  unsigned long long* ub = reinterpret_cast<unsigned long long*>(unext);
-  for (int j = threadIdx.x; j < N; j += blockDim.x)
-    if (uacc[j]) atomicAdd(&ub[j], uacc[j]);
+  uacc.flush(reinterpret_cast<unsigned long long*>(gains_out(w, rnd) + (size_t)b * N), false,
+             (int)((long long)N * blockIdx.x / gridDim.x));
 }
 
 // ---- fill, ascending support, diagnostics ------------------------------------------------
@@ -677,14 +687,21 @@ cudaError_t launch_wide_select(const WideState& w, const WideGeom& g, const gmc_
   while (NP < P) NP <<= 1;
   const size_t psm = sizeof(int) * (sel::HBINS + (size_t)N + 32 + 8 + sel::CBINS + P) +
                      sizeof(short) * (size_t)N + 2 * (size_t)N + 16 +
-                     sizeof(long long) * (size_t)std::min(N, W_BCAP) +
-                     sizeof(int) * (size_t)W_BCAP + 64;
-  const size_t rsm_dense = sizeof(long long) * (size_t)P + sizeof(float) * (size_t)WROWS * P;
-  const size_t rsm_sparse = sizeof(long long) * (size_t)P + sizeof(short) * (size_t)N;
+                     sizeof(long long) * (size_t)std::min(N, W_BCAP) + 64;
+  const size_t rsm_dense = sizeof(float) * DROWS * (((size_t)N + 3) & ~(size_t)3);
+  const size_t rsm_sparse = 3 * sizeof(uint32_t) * (size_t)P + sizeof(short) * ((size_t)N + 1);
   const size_t bsm = (sizeof(long long) + sizeof(int)) * (size_t)NP +
                      sizeof(int) * (sel::HBINS + 2 * (size_t)NP + 32 + 8 + sel::CBINS) +
-                     sizeof(short) * (size_t)NP + 2 * (size_t)NP + sizeof(int) * (size_t)NP + 80;
+                     sizeof(short) * (size_t)NP + 2 * (size_t)NP + 80;
+  // rows: the blocks that are on the GPU together take every row between them.  A filter
+  // block has the fewest warps that do its rows in the same number of turns (33 rows: two
+  // turns of 17 warps, not one and a part of 32).  A slot's limbs take LIMB_ADDS rows.
+  const int per_image = std::max(1, sms / g.B);
+  const int fblocks = std::min(per_image, (int)ceil_div(g.Mstride, 4));
+  const int frows = (int)ceil_div(g.Mstride, fblocks);
+  const int fwarps = (int)ceil_div(frows, ceil_div(frows, FROWS));
   const size_t fsm = sizeof(unsigned long long) * (size_t)N;
+  const size_t fsm_dense = fsm + sizeof(float) * sel::ROW_STEP * (size_t)fwarps;
   // the window pool's extra shared memory: the staged gains and its scratch
   const size_t wsm = 16 + sizeof(long long) * ((size_t)N + sel::WCAP) + sizeof(int) * sel::WCAP +
                      sizeof(int) * (sel::WBINS + 4);
@@ -692,18 +709,21 @@ cudaError_t launch_wide_select(const WideState& w, const WideGeom& g, const gmc_
   const size_t psm_w = psm + (win ? wsm : 0);
   const void* kpool = win ? (const void*)k_w_pool<true> : (const void*)k_w_pool<false>;
   if ((e = set_smem_limit(kpool, psm_w)) != cudaSuccess) return e;
-  if ((e = set_smem_limit((const void*)k_w_rho<true>, rsm_dense)) != cudaSuccess) return e;
-  if ((e = set_smem_limit((const void*)k_w_rho<false>, rsm_sparse)) != cudaSuccess) return e;
+  // pool slots a thread: GMC_MAX_POOL_WIDE in all; rows on 16 bytes where N is a multiple of 4
+  const bool vec = N % 4 == 0;
+  auto* krho = P <= DTHREADS       ? (vec ? k_w_rho_dense<1, true> : k_w_rho_dense<1, false>)
+               : P <= 4 * DTHREADS ? (vec ? k_w_rho_dense<4, true> : k_w_rho_dense<4, false>)
+                                   : (vec ? k_w_rho_dense<8, true> : k_w_rho_dense<8, false>);
+  static_assert(8 * DTHREADS >= GMC_MAX_POOL_WIDE, "a thread's slots hold the widest pool");
+  if ((e = set_smem_limit((const void*)krho, rsm_dense)) != cudaSuccess) return e;
+  if ((e = set_smem_limit((const void*)k_w_rho, rsm_sparse)) != cudaSuccess) return e;
   if ((e = set_smem_limit((const void*)k_w_batch, bsm)) != cudaSuccess) return e;
-  if ((e = set_smem_limit((const void*)k_w_filter<true>, fsm)) != cudaSuccess) return e;
+  if ((e = set_smem_limit((const void*)k_w_filter<true>, fsm_dense)) != cudaSuccess) return e;
   if ((e = set_smem_limit((const void*)k_w_filter<false>, fsm)) != cudaSuccess) return e;
-  // filters: one row per warp while the blocks fit on the GPU about twice, four
-  // beyond (each block ends with an atomic per column it touched: fewer, longer
-  // blocks add fewer; 4 measured best on the long-prefix document)
-  const long long fblocks = (long long)g.B * ceil_div(g.Mstride, FROWS);
-  const int rpw = fblocks > 2LL * sms ? 4 : 1;
-  const dim3 rgrid(ceil_div(g.Mstride, WROWS), g.B);
-  const dim3 fgrid(ceil_div(g.Mstride, FROWS * rpw), g.B);
+  const dim3 rgrid(std::min(g.Mstride, per_image), g.B);
+  const dim3 sgrid(std::max(std::min((int)ceil_div(g.Mstride, SROWS), 2 * per_image),
+                            (int)ceil_div(g.Mstride, sel::LIMB_ADDS - SROWS)), g.B);
+  const dim3 fgrid(fblocks, g.B);
   const int R = wide_rounds(g.K, p);
   for (int rnd = 0; rnd < R; ++rnd) {
     if (win)
@@ -714,20 +734,20 @@ cudaError_t launch_wide_select(const WideState& w, const WideGeom& g, const gmc_
                (const int32_t*)order, tv);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (rnd == 0)
-      launch_k(k_w_rho<true>, rgrid, 32 * WROWS, rsm_dense, st, 1, w, g, P, (const float*)C,
-               (const uint16_t*)scol, p.resp_temp, p.resp_eps, fx_exp, fexp);
+      launch_k(krho, rgrid, DTHREADS, rsm_dense, st, 1, w, g, P, (const float*)C, p.resp_temp,
+               p.resp_eps, fx_exp, fexp);
     else
-      launch_k(k_w_rho<false>, rgrid, 32 * WROWS, rsm_sparse, st, 1, w, g, P, (const float*)C,
+      launch_k(k_w_rho, sgrid, 32 * SROWS, rsm_sparse, st, 1, w, g, P, (const float*)C,
                (const uint16_t*)scol, p.resp_temp, p.resp_eps, fx_exp, fexp);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     launch_k(k_w_batch, g.B, WP_THREADS, bsm, st, 1, w, g, P, NP, p.batch_b, order, tv);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     if (rnd == 0)
-      launch_k(k_w_filter<true>, fgrid, 32 * FROWS, fsm, st, 1, w, g, P, rnd, C, scol, fx_exp,
-               fexp, rpw, tv);
+      launch_k(k_w_filter<true>, fgrid, 32 * fwarps, fsm_dense, st, 1, w, g, P, rnd, C, scol,
+               fx_exp, fexp, tv);
     else
-      launch_k(k_w_filter<false>, fgrid, 32 * FROWS, fsm, st, 1, w, g, P, rnd, C, scol, fx_exp,
-               fexp, rpw, tv);
+      launch_k(k_w_filter<false>, fgrid, 32 * fwarps, fsm, st, 1, w, g, P, rnd, C, scol, fx_exp,
+               fexp, tv);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   launch_k(k_w_final, g.B, WP_THREADS, (size_t)N, st, 1, w, g, fx_exp, fexp, order, support, slot,

@@ -54,9 +54,11 @@ struct GainSums {
     if constexpr (LIMBS) limb_add(w + j, N, v);
     else atomicAdd(reinterpret_cast<unsigned long long*>(w) + j, v);
   }
-  // every nonzero sum, its sign applied, into the global gains
-  __device__ __forceinline__ void flush(unsigned long long* gains, bool negative) const {
-    for (int j = threadIdx.x; j < N; j += blockDim.x) {
+  // every nonzero sum, its sign applied, into the global gains; from token `first` on, around
+  __device__ __forceinline__ void flush(unsigned long long* gains, bool negative,
+                                        int first = 0) const {
+    for (int q = threadIdx.x; q < N; q += blockDim.x) {
+      const int j = first + q < N ? first + q : first + q - N;
       unsigned long long v;
       if constexpr (LIMBS) v = limb_value(w + j, N);
       else v = reinterpret_cast<const unsigned long long*>(w)[j];
@@ -70,14 +72,19 @@ struct GainSums {
 // in cols; their residuals are added to `sums`.  Returns the survivors; *rowmax
 // (MAX) the row's largest value in every lane.
 //
-// A warp takes ROW_STEP values a step: 16 per lane, compared into a bit mask; one scan of the counts places every lane's
-// survivors (lane by lane, ascending within a lane), and only they take the slow
-// part, one per lane and turn, read back from the warp's tile in shared memory.
+// A warp takes ROW_STEP values a step: 16 per lane, compared into a bit mask; one
+// scan of the counts places every lane's survivors (lane by lane, ascending within
+// a lane), and only they take the slow part, one per lane and turn, read back from
+// the warp's tile in shared memory.
 // With one survivor in sixteen, doing that part at every position instead cost a
 // warp about four times the instructions.
+// AHEAD: the next step's values are loaded before this step's are looked at, for
+// blocks whose warps are few on an SM; 16 registers more, which cost a block
+// where several share it (32 images: 251 us, 281 ahead; one image of N = 4,096:
+// 43 us, 40 ahead).
 constexpr int ROW_STEP = 512;  // values a step (2 KB of tile per warp)
 constexpr int ROW_U = ROW_STEP / 128;  // 16-byte loads in flight per lane
-template <bool MAX, class Sums>
+template <bool MAX, bool AHEAD, class Sums>
 __device__ __forceinline__ int filter_dense_row(float* vals, uint16_t* cols, int N, float cover,
                                                 long long cover_fix, float fxs, const Sums& sums,
                                                 float4* tile, float* rowmax) {
@@ -85,17 +92,22 @@ __device__ __forceinline__ int filter_dense_row(float* vals, uint16_t* cols, int
   const bool vec = (N & 3) == 0;  // rows start on 16 bytes
   float mx = 0.f;
   int w = 0;
+  float4 buf[ROW_U];
+  auto load = [&](int base) {
+#pragma unroll
+    for (int u = 0; u < ROW_U; ++u) {
+      const int k = base + 4 * (u * 32 + lane);
+      buf[u] = k < N ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  };
+  if (AHEAD && vec) load(0);
   for (int base = 0; base < N; base += ROW_STEP) {
     if (vec) {
-      float4 buf[ROW_U];
-#pragma unroll
-      for (int u = 0; u < ROW_U; ++u) {
-        const int k = base + 4 * (u * 32 + lane);
-        buf[u] = k < N ? *reinterpret_cast<const float4*>(vals + k) : make_float4(0.f, 0.f, 0.f, 0.f);
-      }
+      if (!AHEAD) load(base);
       __syncwarp();  // the last step's survivors are out of the tile
 #pragma unroll
       for (int u = 0; u < ROW_U; ++u) tile[u * 32 + lane] = buf[u];
+      if (AHEAD) load(base + ROW_STEP);  // the next step's, past every survivor this one writes
     } else {
       float b1[8];
       __syncwarp();
@@ -151,12 +163,6 @@ __device__ __forceinline__ int gain_bucket(long long u) {
   const unsigned long long top = (unsigned long long)u << lz;     // leading one at bit 63
   return (63 - lz) * 32 + (int)((top >> 58) & 31);
 }
-// The next 11 mantissa bits: within one bucket, monotone in the gain.
-__device__ __forceinline__ int gain_subbucket(long long u) {
-  const unsigned long long top = (unsigned long long)u << __clzll(u);
-  return (int)((top >> 47) & 2047);
-}
-
 // Block-wide exclusive scan of one int per thread (deterministic).  Every
 // thread of the block must call it.
 __device__ inline int block_exclusive_scan(int v, int* wsum, int* total) {
@@ -199,11 +205,7 @@ struct PoolScratch {
   long long* bval;     // optional [bcap]: the boundary bucket's gains, staged when the
                        // gains are in global memory (nullptr: read them in place)
   int bcap;
-  int* sortbuf;        // optional [scap], scap a power of two: a boundary bucket of more
-                       // than SORT_MIN gains is sorted there instead of ranked
-  int scap;
 };
-constexpr int SORT_MIN = 128;
 
 // Warp-aggregated append: every lane with `want` gets a distinct index from
 // *counter (order within the warp by lane).  All lanes of the warp call it.
@@ -216,16 +218,8 @@ __device__ __forceinline__ int warp_append(bool want, int* counter) {
   return base + __popc(m & lanemask_lt());
 }
 
-// Position of x among n distinct ints a[0..n) (the number smaller than x),
-// counted by the 8 lanes of an aligned group (mask gm); every group lane gets it.
-__device__ __forceinline__ int group_rank_of(const int* a, int n, int x, int gl, unsigned gm) {
-  int c = 0;
-  for (int k = gl; k < n; k += 8) c += a[k] < x;
-  c += __shfl_xor_sync(gm, c, 1);
-  c += __shfl_xor_sync(gm, c, 2);
-  c += __shfl_xor_sync(gm, c, 4);
-  return c;
-}
+constexpr int RANK_MAX = 128;  // boundary tokens ranked exactly, 8 lanes each
+constexpr int ID_BITS = 15;    // token and slot indices are below GMC_MAX_N_LONG = 2^14
 
 // Pool of one round: the min(P, #{u_i > 0}) tokens with sel[i] == 0 of largest
 // gain u (fixed point), ties to the lower index.  pool[0..Pt) lists the tokens
@@ -246,8 +240,9 @@ __device__ __forceinline__ int group_rank_of(const int* a, int n, int x, int gl,
 // bucket are ranked exactly by (u desc, index asc).
 // ids (optional): ties are broken by the lower ids[j] instead of the lower j
 // (the batch kernel ranks pool slots by (score desc, token asc)).  REFINE
-// (the wide solver's long prefixes) splits a large boundary bucket once more
-// (below); the standard solvers leave it out, it costs them registers.
+// (the wide solver's long prefixes) narrows a large boundary bucket digit by
+// digit (below); the standard solvers, whose buckets are small, leave it out:
+// it costs them registers.
 // Every thread of the block must call it; blockDim is a multiple of 32.
 // bstar_out (optional): the boundary bucket, or -1 when every candidate entered.
 template <bool REFINE = false>
@@ -386,102 +381,100 @@ __device__ inline int select_pool(const long long* u, const unsigned char* sel, 
       for (int q = threadIdx.x; q < nb; q += blockDim.x) w.bval[q] = u[w.bnd[q]];
       __syncthreads();
     }
-    // A large bucket is sorted by (u desc, id asc) (bitonic, in shared
-    // memory) and its first `need` tokens enter.  Otherwise a large bucket
-    // (near-equal gains) is split once more by the next 11 mantissa bits: the
-    // tokens of higher sub-buckets enter, those of lower ones do not, and only
-    // the boundary sub-bucket is ranked exactly.
-    // pk[q]: 1 enters, 0 does not, 2 undecided (ranked below).
-    const bool sorted = w.sortbuf && nb > SORT_MIN && nb <= w.scap;  // uniform over the block
-    const bool refine = REFINE && nb > 512 && !sorted;                        // uniform
-    if (sorted) {
-      int n2 = 1;
-      while (n2 < nb) n2 <<= 1;
-      for (int q = threadIdx.x; q < n2; q += blockDim.x) w.sortbuf[q] = q < nb ? q : -1;
-      __syncthreads();
-      // a before c: c is padding, or (u, id) of a comes first
-      auto before = [&](int a, int c) {
-        if (a < 0) return false;
-        if (c < 0) return true;
-        const int ja = w.bnd[a], jc = w.bnd[c];
-        return key_before(staged ? w.bval[a] : u[ja], ids ? ids[ja] : ja,
-                          staged ? w.bval[c] : u[jc], ids ? ids[jc] : jc);
-      };
-      for (int k = 2; k <= n2; k <<= 1)
-        for (int jj = k >> 1; jj > 0; jj >>= 1) {
-          for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-            const int ixj = i ^ jj;
-            if (ixj > i) {
-              const int a = w.sortbuf[i], c = w.sortbuf[ixj];
-              const bool af = before(a, c);
-              if (((i & k) == 0) != af) {  // out of order for this half's direction
-                w.sortbuf[i] = c;
-                w.sortbuf[ixj] = a;
-              }
+    // REFINE: the bucket (or the whole pool, when the gains are near-equal: up to N
+    // tokens) is narrowed digit by digit, 11 bits at a time: the mantissa bits the
+    // bucket left out, then the id (the lower one first).  A digit's histogram says
+    // which tokens enter, which do not, and which are undecided (pk 1, 0, 2), until
+    // at most RANK_MAX are left to rank exactly.  A bitonic sort of the bucket took
+    // 78 block barriers at 4,096 gains; a digit takes six.
+    int und = nb;  // uniform over the block
+    if constexpr (REFINE) {
+      for (int q = threadIdx.x; q < nb; q += blockDim.x) w.pk[q] = 2;
+      const int mant = max((bstar >> 5) - 5, 0);  // gain bits below the bucket's
+      int done = 0;                               // bits of (gain rest, id) consumed
+      while (und > RANK_MAX && done < mant + ID_BITS) {
+        const bool of_gain = done < mant;
+        const int left = of_gain ? mant - done : mant + ID_BITS - done;
+        const int bits = min(left, 11), lo = left - bits;
+        const int dmask = (1 << bits) - 1;
+        // the digit of boundary token q, monotone in (gain desc, id asc) order
+        auto digit = [&](int q) {
+          const int j = w.bnd[q];
+          if (of_gain) return (int)((staged ? w.bval[q] : u[j]) >> lo) & dmask;
+          return dmask - (((ids ? ids[j] : j) >> lo) & dmask);
+        };
+        __syncthreads();  // the histogram is clear, pk is complete
+        for (int q = threadIdx.x; q < nb; q += blockDim.x)
+          if (w.pk[q] == 2) atomicAdd(&w.hist[digit(q)], 1);
+        __syncthreads();
+        {  // a run of bins per thread, top digit first: the one holding the need-th token
+          const int per = (HBINS + (int)blockDim.x - 1) / (int)blockDim.x;
+          const int h0 = min(HBINS, (int)threadIdx.x * per), h1 = min(HBINS, h0 + per);
+          int c = 0;
+          for (int h = h0; h < h1; ++h) c += w.hist[HBINS - 1 - h];
+          int before = block_exclusive_scan(c, w.wsum, nullptr);
+          for (int h = h0; h < h1; ++h) {
+            const int x = w.hist[HBINS - 1 - h];
+            w.hist[HBINS - 1 - h] = 0;
+            if (before < need && before + x >= need) {  // one bin of one thread
+              w.scal[0] = HBINS - 1 - h;  // the boundary digit
+              w.scal[1] = before;         // tokens of higher digits
+              w.scal[2] = x;              // undecided ones
             }
+            before += x;
           }
-          __syncthreads();
         }
-      for (int q = threadIdx.x; q < nb; q += blockDim.x) w.pk[q] = 0;
-      __syncthreads();
-      for (int q = threadIdx.x; q < need; q += blockDim.x) w.pk[w.sortbuf[q]] = 1;
-      __syncthreads();
-    }
-    if (refine) {
-      for (int q = threadIdx.x; q < nb; q += blockDim.x)
-        atomicAdd(&w.hist[gain_subbucket(staged ? w.bval[q] : u[w.bnd[q]])], 1);
-      __syncthreads();
-      if (wid == 0) {  // the sub-bucket holding the need-th largest: 64 bins per lane, top first
-        int cnt = 0;
-        for (int t = 0; t < 64; ++t) cnt += w.hist[2047 - (lane * 64 + t)];
-        int incl = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const int y = __shfl_up_sync(FULL, incl, o);
-          if (lane >= o) incl += y;
-        }
-        const int L = __ffs(__ballot_sync(FULL, incl >= need)) - 1;  // need <= nb: L >= 0
-        if (lane == L) {
-          int acc = incl - cnt, sb = 2047 - lane * 64;
-          for (int t = 0; t < 64; ++t, --sb) {
-            const int c = w.hist[sb];
-            if (acc + c >= need) break;
-            acc += c;
+        __syncthreads();
+        const int db = w.scal[0];
+        for (int q = threadIdx.x; q < nb; q += blockDim.x)
+          if (w.pk[q] == 2) {
+            const int dg = digit(q);
+            w.pk[q] = dg > db ? 1 : (dg == db ? 2 : 0);
           }
-          w.scal[0] = sb;   // boundary sub-bucket
-          w.scal[1] = acc;  // tokens in higher sub-buckets
+        need -= w.scal[1];
+        und = w.scal[2];
+        done += bits;
+      }
+      __syncthreads();  // pk is complete, scal has been read
+      if (threadIdx.x == 0) w.scal[0] = 0;
+      __syncthreads();
+      for (int q0 = 0; q0 < nb; q0 += blockDim.x) {  // the undecided ones, in any order
+        const int q = q0 + threadIdx.x;
+        const bool in = q < nb && w.pk[q] == 2;
+        const int at = warp_append(in, &w.scal[0]);
+        if (in) w.hist[at] = q;
+      }
+      __syncthreads();
+      const int gl = threadIdx.x & 7;
+      const unsigned gm = 0xFFu << (lane & 24);
+      for (int i = threadIdx.x >> 3; i < und; i += blockDim.x >> 3) {
+        const int q = w.hist[i], j = w.bnd[q];
+        const long long v = staged ? w.bval[q] : u[j];
+        const int id = ids ? ids[j] : j;
+        int rank = 0;
+        for (int i2 = gl; i2 < und; i2 += 8) {
+          const int q2 = w.hist[i2], j2 = w.bnd[q2];
+          rank += key_before(staged ? w.bval[q2] : u[j2], ids ? ids[j2] : j2, v, id);
         }
+        rank += __shfl_xor_sync(gm, rank, 1);
+        rank += __shfl_xor_sync(gm, rank, 2);
+        rank += __shfl_xor_sync(gm, rank, 4);
+        if (gl == 0) w.pk[q] = rank < need;
       }
       __syncthreads();
-      const int sb = w.scal[0];
-      for (int q = threadIdx.x; q < nb; q += blockDim.x) {
-        const int sk = gain_subbucket(staged ? w.bval[q] : u[w.bnd[q]]);
-        w.pk[q] = sk > sb ? 1 : (sk == sb ? 2 : 0);
-      }
-      need -= w.scal[1];
+      for (int i = threadIdx.x; i < und; i += blockDim.x) w.hist[i] = 0;
       __syncthreads();
-    }
-    for (int q = threadIdx.x; q < (sorted ? 0 : nb); q += blockDim.x) {
-      if (refine && w.pk[q] != 2) continue;
-      const int j = w.bnd[q];
-      const long long v = staged ? w.bval[q] : u[j];
-      const int id = ids ? ids[j] : j;
-      int rank = 0;
-      for (int q2 = 0; q2 < nb; ++q2) {
-        if (refine && w.pk[q2] != 2) continue;  // only the boundary sub-bucket competes
-        const int j2 = w.bnd[q2];
-        rank += key_before(staged ? w.bval[q2] : u[j2], ids ? ids[j2] : j2, v, id);
-      }
-      // refine: pk still marks who competes, so the verdict waits in key[q]
-      // (the tokens' bucket keys are no longer read)
-      if (refine) w.key[q] = (short)(rank < need);
-      else w.pk[q] = rank < need;
-    }
-    __syncthreads();
-    if (refine) {  // the verdicts, and the sub-buckets cleared (every thread has read them)
+    } else {
       for (int q = threadIdx.x; q < nb; q += blockDim.x) {
-        if (w.pk[q] == 2) w.pk[q] = (unsigned char)w.key[q];
-        w.hist[gain_subbucket(staged ? w.bval[q] : u[w.bnd[q]])] = 0;
+        const int j = w.bnd[q];
+        const long long v = staged ? w.bval[q] : u[j];
+        const int id = ids ? ids[j] : j;
+        int rank = 0;
+        for (int q2 = 0; q2 < nb; ++q2) {
+          const int j2 = w.bnd[q2];
+          rank += key_before(staged ? w.bval[q2] : u[j2], ids ? ids[j2] : j2, v, id);
+        }
+        w.pk[q] = rank < need;
       }
       __syncthreads();
     }
@@ -711,15 +704,6 @@ __device__ __forceinline__ int group_score_rank(const long long* s, const int* p
   rank += __shfl_xor_sync(gm, rank, 1);
   rank += __shfl_xor_sync(gm, rank, 2);
   rank += __shfl_xor_sync(gm, rank, 4);
-  return rank;
-}
-
-// Rank of pool slot k among the Pt slots by (score desc, token asc).
-__device__ __forceinline__ int score_rank(const long long* s, const int* pool, int Pt, int k) {
-  const long long sk = s[k];
-  const int jk = pool[k];
-  int rank = 0;
-  for (int q = 0; q < Pt; ++q) rank += key_before(s[q], pool[q], sk, jk);
   return rank;
 }
 

@@ -63,6 +63,19 @@ def test_cluster_solver_sizes(kind, B, M, N, K, b, mult):
     _check_select(_clients(kind, B, M, N, 5 + N), K, batch_b=b, pool_mult=mult)
 
 
+# the wide solver: one, four and eight pool slots a thread, rows on 16 bytes and not,
+# the most tokens, all gains equal (the digits of the token decide) or nearly so, a
+# batch that is the whole pool, more rows than blocks and fewer
+@pytest.mark.parametrize("kind,B,M,N,K,b,mult", [
+    ("equal", 1, 40, 9000, 700, 100, 4), ("close", 1, 200, 3001, 600, 300, 4),
+    ("dense", 1, 300, 2050, 900, 700, 5), ("plain", 3, 50, 1000, 400, 130, 1),
+    ("plain", 1, 30, 16384, 64, 256, 8), ("plain", 1, 2300, 501, 200, 40, 4),
+    ("dense", 2, 170, 4096, 1500, 512, 4), ("equal", 1, 33, 2600, 2600, 1024, 2)])
+def test_wide_solver_sizes(kind, B, M, N, K, b, mult):
+    from tests.test_gpu_stages import _check_select
+    _check_select(_clients(kind, B, M, N, 7 + N), K, batch_b=b, pool_mult=mult)
+
+
 # transport: fewer and more member rows than a thread has in flight, lists of more
 # than 64 members (one carrier takes every token), one list for the block (N above
 # 4,096), a row that is one CTA and one that is eight, more text rows than carriers,
