@@ -17,29 +17,36 @@
 // after Algorithm 1: the bounded bank and the chunked N x K assignment product;
 // Eq. (cond-aux-clients), (cond-assignment) for the cosines.)
 //
-// One CTA computes one 128 x BN output tile (BN = 128 or 256, one TMEM column
-// per output column).  Warp 0 / lane 0 streams 64-wide K slices of the A and B
-// row blocks with TMA (128-byte swizzle) through an mbarrier ring of ST stages
-// (4; 2 when the grid holds more tiles than SMs: two CTAs then share an SM and
-// one's epilogue overlaps the other's products); warp
-// 1 / lane 0 issues tcgen05.mma (M = 128, N = BN, K = 16).  Then all 8 warps
-// drain TMEM: warp w reads lane quarter w % 4 and half w / 4 of the columns in
-// 32-column chunks, applies the row and column scales and stores each chunk
-// through a padded 32 x 32 shared-memory transpose, so every store
-// instruction writes one 128-byte row segment.  Ragged edges: TMA fills K
-// columns past the operands' extents with zeros.  The last row block of an
-// operand with at least one full tile of rows is shifted inward (start M - 128,
-// likewise Nn - BN) so every box lies inside the image's own rows -- the
-// hidden states' visual rows are followed by text rows whose count only the
-// device knows -- and stores only the rows and columns the previous tile does
+// Persistent: one CTA per SM takes every gridDim.x-th 128 x BN output tile (BN = 128
+// or 256).  Warp 0 / lane 0 streams 64-wide K slices of the A and B row blocks with
+// TMA (128-byte swizzle) through an mbarrier ring of four stages; warp 1 / lane 0
+// issues tcgen05.mma (M = 128, N = BN, K = 16) into one of two accumulators in
+// tensor memory (BN columns each); warps 4 to 11 drain the other one: warp w reads
+// lane quarter w % 4 and half of the columns in 32-column chunks, and stores each
+// chunk through a 32 x 32 shared-memory transpose, so every store instruction writes
+// whole 128-byte row segments (four of them where the rows lie on 16 bytes), scaled by
+// row and column.  So a tile's products run while the last one is stored,
+// with all four stages' loads in flight behind them.  Before, two CTAs of two
+// stages shared an SM, and one's products waited for their own two loads whenever
+// the other was storing: tensor pipe active 49% on a full SM, 4,096 x 15,876 x
+// 3,584 344 us, now 313; the Gram of 4,096 states 58, now 57, of
+// 32 x 1,296 272, now 215; 4,096 x 15,876 x 384, bound by its stores, 101, now 72.
+//
+// Ragged edges: TMA fills K columns past the operands' extents with zeros.  The
+// last row block of an operand with at least one full tile of rows is shifted
+// inward (start M - 128, likewise Nn - BN) so every box lies inside the image's own
+// rows -- the hidden states' visual rows are followed by text rows whose count only
+// the device knows -- and stores only the rows and columns the previous tile does
 // not own; a smaller operand reads zeros past its declared rows.  Symmetric
-// mode (M == Nn, A and B the same rows): the grid enumerates the tiles that
-// hold an entry with j >= i; a tile stores its own entries and, from
-// registers (coalesced over the lanes), the mirror C[j][i] of each entry
-// j > i whose own tile is not computed -- every entry is written exactly
-// once, so the result does not depend on the order of the stores.  Every
-// mbarrier wait is bounded (about two seconds); on timeout the kernel records
-// GMC_STATUS_TIMEOUT, drains its copies and frees its tensor memory.
+// mode (M == Nn, A and B the same rows): the tiles are those that hold an entry
+// with j >= i; a tile stores its own entries and, from registers (coalesced over
+// the lanes), the mirror C[j][i] of each entry j > i whose own tile is not computed
+// -- every entry is written exactly once, so the result does not depend on the order
+// of the stores.  Every mbarrier wait is bounded (about two seconds after its tile
+// began); on timeout the kernel records GMC_STATUS_TIMEOUT, drains its copies and
+// products and frees its tensor memory.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc.cuh"
@@ -47,15 +54,18 @@
 namespace gmc {
 
 namespace {
-constexpr int GM = 128, GK = 64, GSTAGES = 4;  // ring stages: at most GSTAGES
-constexpr int G_THREADS = 256;
-constexpr int GA_BYTES = GM * GK * 2;  // 16 KiB per stage
+constexpr int GM = 128, GK = 64, GST = 4;  // tile rows, K slice, ring stages
+constexpr int G_EPI = 8;                   // epilogue warps, after four others
+constexpr int G_THREADS = 32 * (4 + G_EPI);
+constexpr int GA_BYTES = GM * GK * 2;      // 16 KiB per stage
 constexpr long long G_WAIT = 4000000000LL;
 
 struct GemmCtl {
-  uint64_t full[GSTAGES];
-  uint64_t empty[GSTAGES];
-  uint64_t done;
+  uint64_t full[GST];
+  uint64_t empty[GST];
+  uint64_t tfull[2];   // an accumulator holds its tile
+  uint64_t tempty[2];  // and has been read
+  uint64_t done;       // every product issued has ended
   uint32_t tmem;
   volatile int abort;
 };
@@ -70,58 +80,84 @@ template <int BN> __host__ __device__ __forceinline__ int sym_first_col(int I) {
   return x <= 0 ? 0 : (x + BN - 1) / BN;
 }
 
-template <int BN, int ST> constexpr size_t gemm_smem() {
-  return 1024 + (size_t)ST * (GA_BYTES + BN * GK * 2) + sizeof(GemmCtl) + sizeof(float) * (GM + BN);
+template <int BN> constexpr size_t gemm_smem() {
+  return 1024 + (size_t)GST * (GA_BYTES + BN * GK * 2) + G_EPI * 32 * 32 * sizeof(float) +
+         sizeof(GemmCtl);
 }
-}  // namespace
 
-template <int BN, int ST>
-__global__ void __launch_bounds__(G_THREADS, ST == 2 ? 2 : 1)
-    k_gemm_tc(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
-              GemmArgs g) {
-  grid_dep_wait();
-  constexpr int B_BYTES = BN * GK * 2;
-  extern __shared__ uint8_t sm_raw[];
-  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) &
-                                             ~static_cast<uintptr_t>(1023));
-  uint8_t* tilesA = base;
-  uint8_t* tilesB = base + ST * GA_BYTES;
-  GemmCtl* ctl = reinterpret_cast<GemmCtl*>(base + ST * (GA_BYTES + B_BYTES));
-  float* rs = reinterpret_cast<float*>(ctl + 1);  // [GM] row scales of the tile
-  float* cs = rs + GM;                            // [BN] column scales
-
-  const int b = blockIdx.z;
-  // consecutive CTAs share a B tile (m_fast: the larger operand is B and stays
-  // in L2 while the A tiles stream past it) or an A tile
-  int tI = g.m_fast ? blockIdx.x : blockIdx.y, tJ = g.m_fast ? blockIdx.y : blockIdx.x;
-  if (g.sym) {  // blockIdx.x enumerates the computed tiles, row block by row block
-    const int nJ = ceil_div(g.Nn, BN);
-    int t = blockIdx.x;
+// Output tile t of the grid's list.
+struct GemmTile {
+  int b, m0, n0;   // image, first row and column it owns
+  int ml, nl;      // first row and column it loads: shifted inward at the ragged end
+  int arow, brow;  // the operands' first rows of the image
+};
+// false: the image has no text (its offsets are invalid), nothing to compute
+template <int BN>
+__device__ __forceinline__ bool gemm_tile(const GemmArgs& g, int t, int per_image, GemmTile* o) {
+  const int b = t / per_image;
+  t -= b * per_image;
+  int tI, tJ;
+  const int nJ = ceil_div(g.Nn, BN);
+  if (g.sym) {  // the computed tiles, row block by row block
     tI = 0;
     while (t >= nJ - sym_first_col<BN>(tI)) {
       t -= nJ - sym_first_col<BN>(tI);
       ++tI;
     }
     tJ = sym_first_col<BN>(tI) + t;
+  } else if (g.m_fast) {
+    // consecutive CTAs share a B tile (the larger operand is B and stays in L2 while
+    // the A tiles stream past it), else an A tile
+    const int nI = ceil_div(g.M, GM);
+    tJ = t / nI;
+    tI = t - tJ * nI;
+  } else {
+    tI = t / nJ;
+    tJ = t - tI * nJ;
   }
-  const int n0 = tJ * BN, m0 = tI * GM;
-  // the tile as loaded: shifted inward at the ragged end
-  const int ml = g.M >= GM ? min(m0, g.M - GM) : m0;
-  const int nl = g.Nn >= BN ? min(n0, g.Nn - BN) : n0;
-  int arow = (int)((long long)b * g.a_img), brow = (int)((long long)b * g.b_img);
+  o->b = b;
+  o->m0 = tI * GM;
+  o->n0 = tJ * BN;
+  o->ml = g.M >= GM ? min(o->m0, g.M - GM) : o->m0;
+  o->nl = g.Nn >= BN ? min(o->n0, g.Nn - BN) : o->n0;
+  o->arow = (int)((long long)b * g.a_img);
+  o->brow = (int)((long long)b * g.b_img);
   if (g.a_text || g.b_text) {
     const TextGeom tg = text_geom(g.toff, b, g.B, g.Tmax, g.status);
-    if (tg.T == 0) return;  // uniform over the block
-    if (g.a_text) arow += tg.off;
-    if (g.b_text) brow += tg.off;
+    if (tg.T == 0) return false;
+    if (g.a_text) o->arow += tg.off;
+    if (g.b_text) o->brow += tg.off;
   }
+  return true;
+}
+}  // namespace
+
+template <int BN>
+__global__ void __launch_bounds__(G_THREADS, 1)
+    k_gemm_tc(const __grid_constant__ CUtensorMap amap, const __grid_constant__ CUtensorMap bmap,
+              GemmArgs g, int per_image) {
+  grid_dep_wait();
+  constexpr int B_BYTES = BN * GK * 2;
+  extern __shared__ uint8_t sm_raw[];
+  uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(sm_raw) + 1023) &
+                                             ~static_cast<uintptr_t>(1023));
+  uint8_t* tilesA = base;
+  uint8_t* tilesB = base + GST * GA_BYTES;
+  float* stage = reinterpret_cast<float*>(base + GST * (GA_BYTES + B_BYTES));  // [G_EPI][32][32]
+  GemmCtl* ctl = reinterpret_cast<GemmCtl*>(stage + G_EPI * 32 * 32);
+
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nk = ceil_div(g.Kd, GK);
+  const int ntiles = per_image * g.B;
 
   if (threadIdx.x == 0) {
-    for (int s = 0; s < ST; ++s) {
+    for (int s = 0; s < GST; ++s) {
       tc::mbar_init(&ctl->full[s], 1);
       tc::mbar_init(&ctl->empty[s], 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      tc::mbar_init(&ctl->tfull[s], 1);
+      tc::mbar_init(&ctl->tempty[s], G_EPI);
     }
     tc::mbar_init(&ctl->done, 1);
     ctl->abort = 0;
@@ -130,137 +166,186 @@ __global__ void __launch_bounds__(G_THREADS, ST == 2 ? 2 : 1)
     tc::prefetch_tmap(&bmap);
   }
   if (warp == 0) {
-    tc::tmem_alloc(&ctl->tmem, BN);
+    tc::tmem_alloc(&ctl->tmem, 2 * BN);
     tc::tmem_relinquish();
   }
   tc::fence_before_sync();
   __syncthreads();
   tc::fence_after_sync();
   const uint32_t tmem = ctl->tmem;
-  const long long deadline = clock64() + G_WAIT;
-  int issued = 0;
+  int issued = 0;  // K slices asked for, over all tiles (warp 0 / lane 0)
 
   if (warp == 0) {
     if (lane == 0) {
-      for (int kb = 0; kb < nk; ++kb) {
-        const int s = kb % ST;
-        const uint32_t ph = (uint32_t)(kb / ST) & 1u;
-        if (kb >= ST && !tc::mbar_wait(&ctl->empty[s], ph ^ 1u, deadline)) {
-          ctl->abort = 1;
-          break;
+      for (int t = blockIdx.x; t < ntiles && !ctl->abort; t += gridDim.x) {
+        GemmTile o;
+        if (!gemm_tile<BN>(g, t, per_image, &o)) continue;
+        const long long deadline = clock64() + G_WAIT;
+        for (int kb = 0; kb < nk; ++kb) {
+          const int s = issued % GST;
+          if (issued >= GST &&
+              !tc::mbar_wait(&ctl->empty[s], ((uint32_t)(issued / GST) & 1u) ^ 1u, deadline))
+            ctl->abort = 1;
+          if (ctl->abort) break;
+          tc::mbar_arrive_expect_tx(&ctl->full[s], GA_BYTES + B_BYTES);
+          tc::tma_load_2d(tilesA + s * GA_BYTES, &amap, kb * GK, o.arow + o.ml, &ctl->full[s]);
+          tc::tma_load_2d(tilesB + s * B_BYTES, &bmap, kb * GK, o.brow + o.nl, &ctl->full[s]);
+          ++issued;
         }
-        if (ctl->abort) break;
-        tc::mbar_arrive_expect_tx(&ctl->full[s], GA_BYTES + B_BYTES);
-        tc::tma_load_2d(tilesA + s * GA_BYTES, &amap, kb * GK, arow + ml, &ctl->full[s]);
-        tc::tma_load_2d(tilesB + s * B_BYTES, &bmap, kb * GK, brow + nl, &ctl->full[s]);
-        ++issued;
       }
     }
     __syncwarp();
   } else if (warp == 1) {
     if (lane == 0) {
       const uint32_t idesc = tc::idesc_bf16_f32(GM, BN);
-      for (int kb = 0; kb < nk; ++kb) {
-        const int s = kb % ST;
-        const uint32_t ph = (uint32_t)(kb / ST) & 1u;
-        if (!tc::mbar_wait(&ctl->full[s], ph, deadline)) {
+      int it = 0, n = 0;  // slices and tiles so far
+      for (int t = blockIdx.x; t < ntiles && !ctl->abort; t += gridDim.x) {
+        GemmTile o;
+        if (!gemm_tile<BN>(g, t, per_image, &o)) continue;
+        const long long deadline = clock64() + G_WAIT;
+        const int buf = n & 1;
+        if (n >= 2 && !tc::mbar_wait(&ctl->tempty[buf], ((uint32_t)(n >> 1) & 1u) ^ 1u, deadline)) {
           ctl->abort = 1;
           break;
         }
         tc::fence_after_sync();
-        const uint64_t ad = tc::desc_sw128_kmajor(tilesA + s * GA_BYTES);
-        const uint64_t bd = tc::desc_sw128_kmajor(tilesB + s * B_BYTES);
+        for (int kb = 0; kb < nk; ++kb, ++it) {
+          const int s = it % GST;
+          if (!tc::mbar_wait(&ctl->full[s], (uint32_t)(it / GST) & 1u, deadline)) {
+            ctl->abort = 1;
+            break;
+          }
+          tc::fence_after_sync();
+          const uint64_t ad = tc::desc_sw128_kmajor(tilesA + s * GA_BYTES);
+          const uint64_t bd = tc::desc_sw128_kmajor(tilesB + s * B_BYTES);
 #pragma unroll
-        for (int kk = 0; kk < GK / 16; ++kk)
-          tc::mma_bf16(tmem, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
-        tc::mma_commit(&ctl->empty[s]);
+          for (int kk = 0; kk < GK / 16; ++kk)
+            tc::mma_bf16(tmem + buf * BN, ad + 2 * kk, bd + 2 * kk, idesc, (kb | kk) != 0);
+          tc::mma_commit(&ctl->empty[s]);
+        }
+        if (ctl->abort) break;
+        tc::mma_commit(&ctl->tfull[buf]);
+        ++n;
       }
-      tc::mma_commit(&ctl->done);  // also on abort, so the epilogue wakes up
+      // every arrival of the products has landed before the block ends, also on abort
+      tc::mma_commit(&ctl->done);
+      if (!tc::mbar_wait(&ctl->done, 0, clock64() + G_WAIT)) ctl->abort = 1;
     }
     __syncwarp();
-  } else {
-    // scales of the tile's rows and columns (1 where none is given)
-    for (int q = threadIdx.x - 64; q < GM + BN; q += G_THREADS - 64) {
-      float v = 1.f;
-      if (q < GM) {
-        const int m = ml + q;
-        if (g.rscale && m < g.M) v = g.rscale[(size_t)b * g.M + m];
-        rs[q] = v;
-      } else {
-        const int n = nl + q - GM;
-        if (g.cscale && n < g.Nn) v = g.cscale[(size_t)b * g.Nn + n];
-        cs[q - GM] = v;
+  } else if (warp >= 4) {
+    const int quarter = warp & 3, half = (warp - 4) >> 2;
+    float* st = stage + (warp - 4) * (32 * 32);
+    // rows of C on 16 bytes, for tiles that start on a multiple of four columns
+    const bool quads = (g.ldc & 3) == 0 && (g.c_img & 3) == 0 &&
+                       (reinterpret_cast<uintptr_t>(g.C) & 15) == 0;
+    int n = 0;
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+      GemmTile o;
+      if (!gemm_tile<BN>(g, t, per_image, &o)) continue;
+      const int buf = n & 1;
+      const bool here = tc::mbar_wait(&ctl->tfull[buf], (uint32_t)(n >> 1) & 1u, clock64() + G_WAIT);
+      if (!__all_sync(FULL, here)) {
+        if (lane == 0) ctl->abort = 1;
+        break;
       }
-    }
-  }
-
-  bool ok = tc::mbar_wait(&ctl->done, 0, deadline) && !ctl->abort;
-  ok = __syncthreads_and(ok);  // also publishes the scales
-  tc::fence_after_sync();
-  if (ok && nk > 0) {
-    const int quarter = warp & 3, half = warp >> 2;
-    const int row = quarter * 32 + lane;  // this thread's TMEM lane = tile row
-    const float r = rs[row];
-    // the operand ring is idle now: a padded 32 x 33 staging block per warp
-    float* st = reinterpret_cast<float*>(tilesA) + warp * (32 * 33);
-    const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16);
-    float* Cimg = g.C + (size_t)b * g.c_img;
+      ++n;
+      tc::fence_after_sync();
+      const int row = quarter * 32 + lane;  // this thread's TMEM lane = tile row
+      const int i = o.ml + row;
+      float r = 1.f;  // scales of the tile's rows and columns (1 where none is given)
+      if (g.rscale && i < g.M) r = g.rscale[(size_t)o.b * g.M + i];
+      const uint32_t trow = tmem + buf * BN + ((uint32_t)(quarter * 32) << 16);
+      float* Cimg = g.C + (size_t)o.b * g.c_img;
+      const bool full = o.m0 == o.ml && o.n0 == o.nl && o.ml + GM <= g.M && o.nl + BN <= g.Nn;
 #pragma unroll 1
-    for (int c = 0; c < BN / 64; ++c) {
-      const int cl = half * (BN / 2) + c * 32;  // first column of the chunk, within the tile
-      float v[32];
-      tc::tmem_ld32(trow + (uint32_t)cl, v);
-#pragma unroll
-      for (int q = 0; q < 32; ++q) {
-        v[q] *= r * cs[cl + q];
-        st[lane * 33 + q] = v[q];
-      }
-      if (g.sym) {  // mirrors of owned entries j > i whose own tile is not computed
-        const int i = ml + row;
-        const bool own_i = i >= m0 && i < g.M;
-#pragma unroll  // fully: v stays in registers
-        for (int q = 0; q < 32; ++q) {
-          const int j = nl + cl + q;
-          if (own_i && j >= n0 && j < g.Nn && j > i && !sym_tile<BN>(j / GM, i / BN))
-            Cimg[(size_t)j * g.ldc + i] = v[q];
+      for (int c = 0; c < BN / 64; ++c) {
+        const int cl = half * (BN / 2) + c * 32;  // first column of the chunk, within the tile
+        const int i0 = o.ml + quarter * 32, j0 = o.nl + cl;  // the chunk's first entry
+        float v[32];
+        tc::tmem_ld32(trow + (uint32_t)cl, v);
+        if (c == BN / 64 - 1) {  // the accumulator is read: the next products may have it
+          tc::fence_before_sync();
+          __syncwarp();
+          if (lane == 0) tc::mbar_arrive(&ctl->tempty[buf]);
         }
-      }
-      __syncwarp();
-      const int col = nl + cl + lane;
-      const bool col_ok = col >= n0 && col < g.Nn;  // owned by this tile
+        // the transpose: 16-byte unit u of row l in unit u ^ (l & 7)
+        float4* st4 = reinterpret_cast<float4*>(st);
+#pragma unroll
+        for (int u = 0; u < 8; ++u)
+          st4[lane * 8 + (u ^ (lane & 7))] =
+              make_float4(v[4 * u], v[4 * u + 1], v[4 * u + 2], v[4 * u + 3]);
+        const int col = j0 + lane;
+        float cs = 1.f;
+        if (g.cscale && col < g.Nn) cs = g.cscale[(size_t)o.b * g.Nn + col];
+        if (g.sym) {  // mirrors of owned entries j > i whose own tile is not computed
+          // a tile that owns all it loads: one answer for 32 x 32 entries off the diagonal
+          // (128 and 256 are multiples of 32, and so are i0 and j0)
+          const bool all = full && j0 > i0 + 31;
+          const bool any = !all || !sym_tile<BN>(j0 / GM, i0 / BN);
+          const bool own_i = i >= o.m0 && i < g.M;
+          float* mir = Cimg + (size_t)j0 * g.ldc + i;
+          if (any) {
+#pragma unroll  // fully: v stays in registers
+            for (int q = 0; q < 32; ++q) {
+              const int j = j0 + q;
+              const float x = v[q] * (r * __shfl_sync(FULL, cs, q));
+              if (all || (own_i && j >= o.n0 && j < g.Nn && j > i && !sym_tile<BN>(j / GM, i / BN)))
+                mir[(size_t)q * g.ldc] = x;
+            }
+          }
+        }
+        __syncwarp();
+        if (full && quads) {  // four columns a lane, four rows a store
+          const int u = lane & 7, r0 = lane >> 3;
+          float4 c4;
+          c4.x = __shfl_sync(FULL, cs, 4 * u);
+          c4.y = __shfl_sync(FULL, cs, 4 * u + 1);
+          c4.z = __shfl_sync(FULL, cs, 4 * u + 2);
+          c4.w = __shfl_sync(FULL, cs, 4 * u + 3);
+          float* out = Cimg + (size_t)(i0 + r0) * g.ldc + j0 + 4 * u;
+#pragma unroll
+          for (int k = 0; k < 8; ++k) {
+            const int rr = 4 * k + r0;
+            const float rk = __shfl_sync(FULL, r, rr);
+            float4 x = st4[rr * 8 + (u ^ (rr & 7))];
+            x.x *= rk * c4.x;
+            x.y *= rk * c4.y;
+            x.z *= rk * c4.z;
+            x.w *= rk * c4.w;
+            *reinterpret_cast<float4*>(out) = x;
+            out += 4 * (size_t)g.ldc;
+          }
+        } else {
+          const bool col_ok = col >= o.n0 && col < g.Nn;  // owned by this tile
 #pragma unroll 4
-      for (int rr = 0; rr < 32; ++rr) {
-        const int m = ml + quarter * 32 + rr;
-        if (m >= m0 && m < g.M && col_ok) Cimg[(size_t)m * g.ldc + col] = st[rr * 33 + lane];
+          for (int rr = 0; rr < 32; ++rr) {
+            const int m = i0 + rr;
+            const float rk = __shfl_sync(FULL, r, rr);
+            const float x = st[rr * 32 + (((lane >> 2) ^ (rr & 7)) << 2) + (lane & 3)];
+            if (m >= o.m0 && m < g.M && col_ok) Cimg[(size_t)m * g.ldc + col] = x * (rk * cs);
+          }
+        }
+        __syncwarp();
       }
-      __syncwarp();
     }
   }
-  if (!ok && threadIdx.x == 0) set_status(g.status, GMC_STATUS_TIMEOUT);
-  if (warp == 0 && lane == 0 && !ok) {
-    // drain TMA copies still in flight into this CTA's shared memory
+  __syncthreads();
+  const bool ok = !ctl->abort;
+  if (!ok && threadIdx.x == 0) {
+    set_status(g.status, GMC_STATUS_TIMEOUT);
+    // drain the copies still in flight
     const long long d2 = clock64() + G_WAIT;
-    for (int kb = (issued > ST ? issued - ST : 0); kb < issued; ++kb)
-      if (!tc::mbar_wait(&ctl->full[kb % ST], (uint32_t)(kb / ST) & 1u, d2)) break;
+    for (int q = (issued > GST ? issued - GST : 0); q < issued; ++q)
+      if (!tc::mbar_wait(&ctl->full[q % GST], (uint32_t)(q / GST) & 1u, d2)) break;
   }
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tmem, BN);
+  if (warp == 0) tc::tmem_dealloc(tmem, 2 * BN);
 }
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <int BN, int ST>
-static cudaError_t launch_gemm_st(const CUtensorMap& am, const CUtensorMap& bm, const GemmArgs& g,
-                                  dim3 grid, cudaStream_t st) {
-  const size_t smem = gemm_smem<BN, ST>();
-  cudaError_t e;
-  if ((e = set_smem_limit((const void*)k_gemm_tc<BN, ST>, smem)) != cudaSuccess) return e;
-  launch_k(k_gemm_tc<BN, ST>, grid, G_THREADS, smem, st, 1, am, bm, g);
-  return cudaGetLastError();
-}
-
 template <int BN>
 static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_rows, int lda,
                                   const void* Bm, long long b_rows, int ldb, cudaStream_t st) {
@@ -270,17 +355,20 @@ static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_
   if ((e = make_tmap_bf16(&bm, Bm, (uint64_t)g.Kd, (uint64_t)b_rows, (uint64_t)ldb, BN)) !=
       cudaSuccess)
     return e;
-  dim3 grid(ceil_div(g.Nn, BN), ceil_div(g.M, GM), g.B);
-  if (g.m_fast) grid = dim3(ceil_div(g.M, GM), ceil_div(g.Nn, BN), g.B);
-  if (g.sym) grid = dim3(gemm_sym_ctas(g.M, 1), 1, g.B);  // the computed tiles of every image
+  const int per_image =
+      g.sym ? gemm_sym_ctas(g.M, 1) : ceil_div(g.Nn, BN) * ceil_div(g.M, GM);
   static int sms = 0;
   if (sms == 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess) {
     cudaGetLastError();
     sms = 152;
   }
-  // more tiles than SMs: two CTAs per SM with two stages each
-  if ((long long)grid.x * grid.y * grid.z > sms) return launch_gemm_st<BN, 2>(am, bm, g, grid, st);
-  return launch_gemm_st<BN, GSTAGES>(am, bm, g, grid, st);
+  const long long tiles = (long long)per_image * g.B;
+  if (tiles > 0x7fffffffLL - sms) return cudaErrorInvalidValue;
+  constexpr size_t smem = gemm_smem<BN>();
+  if ((e = set_smem_limit((const void*)k_gemm_tc<BN>, smem)) != cudaSuccess) return e;
+  launch_k(k_gemm_tc<BN>, (int)std::min<long long>(tiles, sms), G_THREADS, smem, st, 1, am, bm, g,
+           per_image);
+  return cudaGetLastError();
 }
 
 int gemm_sym_ctas(int N, int B) {  // symmetric Grams use 128 x 256 tiles (N > 128)

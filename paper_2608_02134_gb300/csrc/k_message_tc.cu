@@ -139,9 +139,6 @@ size_t msg_smem_bytes(int nkb, int mode) {
          (mode ? WRITE_STAGE_BYTES : 0);
 }
 
-__device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
-}
 __device__ __forceinline__ void epi_barrier() {
   asm volatile("bar.sync 1, %0;" ::"n"(EPI_WARPS * 32) : "memory");
 }
@@ -294,7 +291,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       }
       tc::fence_before_sync();
       __syncwarp();
-      if (lane == 0) mbar_arrive(&ctl->acce[buf]);
+      if (lane == 0) tc::mbar_arrive(&ctl->acce[buf]);
       if (!ok) continue;
       const int k0 = c * BM + cpart * 32;
       if (mode == 0) {  // running max / sum over the visible keys

@@ -129,6 +129,25 @@ def test_transport_sizes(B, gh, gw, T, K, D, Hkv, d, dtype, spread):
         assert bool(((oh[b, :K].double() - ref).abs() <= bound).all())
 
 
+def _check_grounded(wl):
+    """The grounded rows of the first and the last image, at the GPU's head weights."""
+    from oracle import gmc_oracle as O
+    from tests.test_gpu_clients import _gpu_clients
+    C, traces, comp = _gpu_clients(wl)
+    p = O.params()
+    f = lambda a: np.asarray(a, dtype=np.float64)  # noqa: E731
+    for b in {0, wl.B - 1}:
+        im, tr = wl.image(b), traces[b]
+        A = O.message_slice(f(im.queries), f(im.keys), wl.N)
+        Z, sigma = O.probe_values(f(im.values)[:wl.N], f(wl.probe()), wl.H, p)
+        P, _ = O.grounded_clients(O.atom_norms(A, Z, sigma))
+        nu = O.query_weights(im.T, p)
+        ref = 0.5 * f(tr.omega)[:, None, None] * nu[None, :, None] * P
+        got = C[b, :wl.H * im.T].reshape(wl.H, im.T, wl.N)
+        err = np.abs(got - ref).max(2) / ref.max(2)
+        assert err.max() <= 1e-3, err.max()   # the bar of the client parity tests
+
+
 # message slice: key splits that fill a cluster, exceed the portable cluster size and
 # exceed the largest one (two launches); query tiles that are ragged; keys that end
 # inside a tile, rows of A on 16 bytes and not
@@ -137,22 +156,8 @@ def test_transport_sizes(B, gh, gw, T, K, D, Hkv, d, dtype, spread):
     (66, 64, [9], 4, 1, 1), (128, 64, [5], 2, 1, 1)])
 def test_message_slice_splits(gh, gw, T, H, Hkv, B):
     from paper_2608_02134_gb300 import workloads
-    from tests.test_gpu_clients import _gpu_clients
-    from oracle import gmc_oracle as O
     wl = workloads.make("qwen", B=B, T=T * (B // len(T)), gh=gh, gw=gw, D=64, d=64, H=H, Hkv=Hkv, K=9)
-    C, traces, comp = _gpu_clients(wl)
-    p = O.params()
-    f = lambda a: np.asarray(a, dtype=np.float64)  # noqa: E731
-    for b in {0, B - 1}:
-        im, tr = wl.image(b), traces[b]
-        A = O.message_slice(f(im.queries), f(im.keys), wl.N)
-        Z, sigma = O.probe_values(f(im.values)[:wl.N], f(wl.probe()), H, p)
-        P, _ = O.grounded_clients(O.atom_norms(A, Z, sigma))
-        nu = O.query_weights(im.T, p)
-        ref = 0.5 * f(tr.omega)[:, None, None] * nu[None, :, None] * P
-        got = C[b, :H * im.T].reshape(H, im.T, wl.N)
-        err = np.abs(got - ref).max(2) / ref.max(2)
-        assert err.max() <= 1e-3, err.max()   # the bar of the client parity tests
+    _check_grounded(wl)
 
 
 # assignment: gates that leave every gap open, some and none, a weight that lets the
@@ -203,3 +208,27 @@ def test_assignment_gates(shape, K, gate_scale, weight, margin, twins):
     disc[S] = False
     assert np.isin(tr.pi, S).all() and np.array_equal(tr.pi[S], S)
     assert (got[disc] >= kappa.max(1)[disc] - tol).all(), (kappa.max(1) - got)[disc].max()
+
+
+# tensor-core Gram: one tile a CTA and several (both accumulators, the stage ring over
+# tile boundaries), rows of C on 16 bytes and not, a last tile that is shifted inward,
+# blocks on, above and mirrored below the diagonal, K that ends inside a slice
+@pytest.mark.parametrize("B,gh,gw,D,T", [
+    (80, 16, 16, 64, 3), (31, 12, 25, 1000, 5), (12, 23, 31, 264, 2), (2, 47, 49, 72, 7),
+    (1, 64, 65, 512, 1), (3, 36, 36, 3584, 9), (1, 79, 77, 136, 4)])
+def test_cosine_gram_tiles(B, gh, gw, D, T):
+    from paper_2608_02134_gb300 import gmc
+    N = gh * gw
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + D)
+    hid = torch.randn((B, N + T, D), generator=g, device="cuda").to(torch.bfloat16)
+    out = torch.full((B, N, N), float("nan"), device="cuda")
+    ws = gmc.cosine(gmc.problem(B, gh, gw, 1, gmc.GMC_BF16), gmc.default_params(), hid, N, T, D, out)
+    torch.cuda.synchronize()
+    assert gmc.read_status(ws) == 0
+    for b in {0, B // 2, B - 1}:
+        x = hid[b, :N].double()
+        x = x / x.norm(dim=1, keepdim=True)
+        # products exact in fp32, D of them summed in fp32 (truncating at worst), then two
+        # scales of fp32 norms: (D + 8) 2^-23 of the terms' magnitudes, which sum to at most 1
+        assert float((out[b].double() - x @ x.T).abs().max()) <= (D + 8) * 2.0 ** -23
