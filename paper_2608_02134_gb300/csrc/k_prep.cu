@@ -49,9 +49,14 @@ __global__ void k_rownorm(const Tin* __restrict__ hidden, const int32_t* toff, i
 // Z_h[i] = V_{kv(h)}[i] W_h (Eq. (1): (V_h O_h) P with W_h = O_h P), ||Z_h[i]||^2,
 // per-block partial sums of ||Z_h||_F^2, and
 // sigma_h = sqrt(lambda_mass) * max(||Z_h||_F / sqrt(N r), eps_mass) (Eq. (1)).
-// A block covers PR_TOK tokens of one KV group: the values and the group's
-// W_h are staged in shared memory, one thread per (token, head) computes the
-// four probe coordinates.  The last block of an image to finish (a ticket per
+// A block covers PR_TOK tokens of one KV group: the values and the group's W_h are
+// staged in shared memory, and a warp takes a head, a lane a token of it: W_h is then
+// one broadcast load for the warp, the values are read 16 bytes a lane, and the
+// coordinates are written in whole lines.  With a (token, head) pair a lane the
+// loads of W_h took four shared-memory wavefronts each and the block was bound by
+// them (32 images of N = 1,296, 28 heads of 128: 110 us, now 78; N = 15,876: 51,
+// now 35; one image of N = 1,296, where the chain of latencies sets the time:
+// 11.7, now 9.0).  The last block of an image to finish (a ticket per
 // image, zeroed with the status word) sums the partials in a fixed order.
 // With Qp (the tensor-core message slice follows), the blocks of KV group g
 // also write the group's packed text queries first: Qp [B][Hkv][RQ][d], row
@@ -70,8 +75,25 @@ __global__ void __launch_bounds__(256) k_probe(
   __shared__ int last;
   const int b = blockIdx.z, g = blockIdx.y, pb = blockIdx.x;
   const TextGeom tg = text_geom(toff, b, B, Tmax, status);
+  const int grp = H / Hkv, HD = Hkv * d, i0 = pb * PR_TOK;
+  constexpr int VE = 16 / sizeof(Tin);  // elements per 16-byte unit
+  const int pitch = d / VE + 1 - (d / VE & 1);  // units a value row: odd, so lanes meet no bank twice
+  float4* Ws = sm_probe4;                               // [grp][d]
+  uint4* Vs = reinterpret_cast<uint4*>(Ws + grp * d);   // [PR_TOK][pitch]
+  if (tg.T > 0) {  // uniform over the image: every copy in flight before the queries are packed
+    const SeqIdx sq(b, N, K, tg.off, tg.T);
+    const int nu = d / VE;
+    for (int idx = threadIdx.x; idx < PR_TOK * nu; idx += blockDim.x) {
+      const int ii = idx / nu, u = idx - ii * nu, i = i0 + ii;
+      cp_async16(&Vs[ii * pitch + u], keys + sq.value_row(min(i, N - 1), HD) + (size_t)g * d + u * VE,
+                 i < N);
+    }
+    const float4* W4 = reinterpret_cast<const float4*>(W) + (size_t)g * grp * d;
+    for (int idx = threadIdx.x; idx < grp * d; idx += blockDim.x) cp_async16(&Ws[idx], &W4[idx]);
+    cp_async_commit();
+  }
   if (Qp) {
-    const int grp = H / Hkv, nv = d / 8;  // 16-byte pieces per row
+    const int nv = d / 8;  // 16-byte pieces per row
     for (int idx = threadIdx.x;; idx += blockDim.x) {
       const int row = pb + (idx / nv) * nP, q = idx % nv;
       if (row >= RQ) break;  // row grows with idx
@@ -85,90 +107,51 @@ __global__ void __launch_bounds__(256) k_probe(
     }
   }
   if (tg.T == 0) return;  // uniform over the image
-  const SeqIdx sq(b, N, K, tg.off, tg.T);
-  const int grp = H / Hkv, HD = Hkv * d, i0 = pb * PR_TOK;
-  float4* Ws = sm_probe4;                                    // [grp][d + 1]
-  float* Vs = reinterpret_cast<float*>(Ws + grp * (d + 1));  // [PR_TOK][d + 1] (padded rows)
-  float* zs = Vs + PR_TOK * (d + 1);                         // [PR_TOK][grp]
-  const float4* W4 = reinterpret_cast<const float4*>(W) + (size_t)g * grp * d;
-  // W_h rows by cp.async, the values through registers four loads at a time:
-  // every copy of the block is in flight before the first one lands
-  for (int idx = threadIdx.x; idx < grp * d; idx += blockDim.x)
-    cp_async16(&Ws[(idx / d) * (d + 1) + idx % d], &W4[idx]);
-  cp_async_commit();
-  constexpr int VE = 16 / sizeof(Tin);  // elements per 16-byte load
-  const int nld = PR_TOK * d / VE;
-  for (int idx0 = 0; idx0 < nld; idx0 += 4 * (int)blockDim.x) {  // uniform over the block
-    uint4 raw[4];
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int idx = idx0 + u * (int)blockDim.x + (int)threadIdx.x;
-      const int ii = idx / (d / VE), k = (idx % (d / VE)) * VE, i = i0 + ii;
-      raw[u] = make_uint4(0, 0, 0, 0);
-      if (idx < nld && i < N)
-        raw[u] = *reinterpret_cast<const uint4*>(keys + sq.value_row(i, HD) + (size_t)g * d + k);
-    }
-#pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int idx = idx0 + u * (int)blockDim.x + (int)threadIdx.x;
-      if (idx >= nld) continue;
-      const int ii = idx / (d / VE), k = (idx % (d / VE)) * VE;
-      const Tin* e = reinterpret_cast<const Tin*>(&raw[u]);
-#pragma unroll
-      for (int q = 0; q < VE; ++q) Vs[ii * (d + 1) + k + q] = to_f32(e[q]);
-    }
-  }
   cp_async_wait<0>();
   __syncthreads();
-  for (int task = threadIdx.x; task < PR_TOK * grp; task += blockDim.x) {
-    const int ii = task / grp, jh = task % grp, i = i0 + ii;
-    const float* v = Vs + ii * (d + 1);
-    const float4* w = Ws + jh * (d + 1);
-    // four coordinates loaded ahead of their FMAs; even and odd k accumulate
-    // apart and are added once at the end (d is a multiple of 4)
+  const int lane = threadIdx.x & 31, i = i0 + lane;
+  static_assert(PR_TOK == 32, "a lane per token");
+  for (int jh = threadIdx.x >> 5; jh < grp; jh += (int)blockDim.x >> 5) {
+    const uint4* v = Vs + lane * pitch;
+    const float4* w = Ws + jh * d;
+    // even and odd k accumulate apart and are added once at the end (VE is even)
     float a0 = 0.f, a1 = 0.f, a2 = 0.f, a3 = 0.f, b0 = 0.f, b1 = 0.f, b2 = 0.f, b3 = 0.f;
 #pragma unroll 2
-    for (int k = 0; k < d; k += 4) {
-      float x[4];
-      float4 c[4];
+    for (int u = 0; u < d / VE; ++u) {
+      const uint4 raw = v[u];
+      const Tin* x = reinterpret_cast<const Tin*>(&raw);
 #pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        x[u] = v[k + u];
-        c[u] = w[k + u];
-      }
-#pragma unroll
-      for (int u = 0; u < 4; u += 2) {
-        a0 = fmaf(x[u], c[u].x, a0);
-        a1 = fmaf(x[u], c[u].y, a1);
-        a2 = fmaf(x[u], c[u].z, a2);
-        a3 = fmaf(x[u], c[u].w, a3);
-        b0 = fmaf(x[u + 1], c[u + 1].x, b0);
-        b1 = fmaf(x[u + 1], c[u + 1].y, b1);
-        b2 = fmaf(x[u + 1], c[u + 1].z, b2);
-        b3 = fmaf(x[u + 1], c[u + 1].w, b3);
+      for (int q = 0; q < VE; q += 2) {
+        const float x0 = to_f32(x[q]), x1 = to_f32(x[q + 1]);
+        const float4 c0 = w[u * VE + q], c1 = w[u * VE + q + 1];
+        a0 = fmaf(x0, c0.x, a0);
+        a1 = fmaf(x0, c0.y, a1);
+        a2 = fmaf(x0, c0.z, a2);
+        a3 = fmaf(x0, c0.w, a3);
+        b0 = fmaf(x1, c1.x, b0);
+        b1 = fmaf(x1, c1.y, b1);
+        b2 = fmaf(x1, c1.z, b2);
+        b3 = fmaf(x1, c1.w, b3);
       }
     }
     const float z0 = a0 + b0, z1 = a1 + b1, z2 = a2 + b2, z3 = a3 + b3;
-    const float n2 = z0 * z0 + z1 * z1 + z2 * z2 + z3 * z3;
+    float n2 = z0 * z0 + z1 * z1 + z2 * z2 + z3 * z3;
     if (i < N) {
       const size_t o = ((size_t)b * H + g * grp + jh) * N + i;
       reinterpret_cast<float4*>(Z)[o] = make_float4(z0, z1, z2, z3);
       zn2[o] = n2;
+    } else {
+      n2 = 0.f;
     }
-    zs[ii * grp + jh] = i < N ? n2 : 0.f;
-  }
-  __syncthreads();
-  // per head of the group: eight threads sum every eighth token, a fixed
-  // shuffle tree adds the eight
-  for (int jh0 = 0; jh0 < grp; jh0 += (int)blockDim.x / 8) {  // uniform over the block
-    const int jh = jh0 + (int)threadIdx.x / 8, pt = threadIdx.x & 7;
-    float sacc = 0.f;
-    if (jh < grp)
-      for (int ii = pt; ii < PR_TOK; ii += 8) sacc += zs[ii * grp + jh];
+    // the head's partial: lanes 0 to 7 sum every eighth token, a fixed shuffle tree
+    // adds the eight
+    float sacc = n2 + __shfl_down_sync(FULL, n2, 8);
+    sacc += __shfl_down_sync(FULL, n2, 16);
+    sacc += __shfl_down_sync(FULL, n2, 24);
     sacc += __shfl_xor_sync(FULL, sacc, 4);
     sacc += __shfl_xor_sync(FULL, sacc, 2);
     sacc += __shfl_xor_sync(FULL, sacc, 1);
-    if (jh < grp && pt == 0) sigpart[((size_t)b * nP + pb) * H + g * grp + jh] = sacc;
+    if (lane == 0) sigpart[((size_t)b * nP + pb) * H + g * grp + jh] = sacc;
   }
   __threadfence();
   __syncthreads();
@@ -268,8 +251,8 @@ cudaError_t launch_probe(const Dims& dm, const void* keys, const float* W, const
   const __nv_bfloat16* q16 = static_cast<const __nv_bfloat16*>(queries);
   const int grp = dm.H / dm.Hkv;
   dim3 grid(s.nP, dm.Hkv, dm.B);
-  const size_t smem = sizeof(float4) * grp * (dm.d + 1) +
-                      sizeof(float) * ((size_t)PR_TOK * (dm.d + 1) + (size_t)PR_TOK * grp);
+  const int units = dm.d * (dm.dtype == GMC_BF16 ? 2 : 4) / 16;  // of a value row
+  const size_t smem = 16 * ((size_t)grp * dm.d + (size_t)PR_TOK * (units + 1 - (units & 1)));
   cudaError_t e;
   if (dm.dtype == GMC_BF16) {
     if ((e = set_smem_limit((const void*)k_probe<__nv_bfloat16>, smem)) != cudaSuccess) return e;

@@ -160,6 +160,18 @@ def test_message_slice_splits(gh, gw, T, H, Hkv, B):
     _check_grounded(wl)
 
 
+# probe: one head a KV group, more heads than warps, value rows of an odd and an even
+# number of 16-byte units, a last block that is not full, both types
+@pytest.mark.parametrize("name,gh,gw,T,H,Hkv,d,B", [
+    ("qwen", 5, 13, [3], 4, 4, 8, 1), ("qwen", 9, 9, [17, 2], 18, 1, 72, 2),
+    ("tiny", 7, 11, [6], 12, 1, 20, 1), ("tiny", 4, 8, [9], 3, 3, 64, 1),
+    ("qwen", 11, 12, [40], 28, 4, 128, 3)])
+def test_probe_sizes(name, gh, gw, T, H, Hkv, d, B):
+    from paper_2608_02134_gb300 import workloads
+    _check_grounded(workloads.make(name, B=B, T=T * (B // len(T)), gh=gh, gw=gw, D=64, d=d, H=H,
+                                   Hkv=Hkv, K=9))
+
+
 # assignment: gates that leave every gap open, some and none, a weight that lets the
 # spatial term outweigh any gap and one of zero, one carrier, duplicated tokens (gap
 # zero), several images: the carrier of every discarded token has the largest kappa
