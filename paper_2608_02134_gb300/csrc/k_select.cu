@@ -575,7 +575,7 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
     for (int q = q0; q < q1; ++q) mine += s.rptr[q];
     int tot = 0;
     int at = block_exclusive_scan(mine, s.wsum, &tot);
-    if (tot > lay.cap) return;  // uniform over the block
+    if (tot > lay.cap) return;  // uniform over the block; below 2^16: positions are 16 bits
     for (int q = q0; q < q1; ++q) {
       const int n = s.rptr[q];
       s.rptr[q] = (uint16_t)at;
@@ -584,15 +584,24 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
     if (threadIdx.x == 0) s.rptr[nrows] = (uint16_t)tot;
     for (int j = threadIdx.x; j <= N; j += SEL_THREADS) s.cs[j] = 0;
     __syncthreads();
-    // every entry by one thread, MU loads in flight (rows are very uneven); its row by
-    // a binary search of the rows' offsets; tokens counted in cs[j + 1]
-    auto row_of = [&](int p) {
+    // every entry by one thread, MU loads in flight (rows are very uneven); tokens
+    // counted in cs[j + 1].  Its row: the row of its 32 entries' first one, from a table
+    // (a binary search of the rows' offsets for each, kept in the histogram's bins), then a
+    // step or two; a search for every entry was most of the time before the first round (22
+    // us at N = 1,296, now 13).
+    for (int c = threadIdx.x; 32 * c < tot; c += SEL_THREADS) {
       int lo2 = 0, hi2 = nrows;  // rptr[lo2] <= p < rptr[hi2]
       while (hi2 - lo2 > 1) {
         const int mid = (lo2 + hi2) >> 1;
-        if (s.rptr[mid] <= p) lo2 = mid; else hi2 = mid;
+        if (s.rptr[mid] <= 32 * c) lo2 = mid; else hi2 = mid;
       }
-      return lo2;
+      s.hist[c] = lo2;
+    }
+    __syncthreads();
+    auto row_of = [&](int p) {
+      int q = s.hist[p >> 5];
+      while (s.rptr[q + 1] <= p) ++q;
+      return q;
     };
     constexpr int MU = 8;
     for (int b0 = threadIdx.x; b0 < tot; b0 += MU * SEL_THREADS) {
@@ -638,6 +647,7 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
       s.cpos[d] = (uint16_t)p;
     }
     __syncthreads();  // cs[j] is now the first entry of token j, cs[N] the total
+    for (int c = threadIdx.x; 32 * c < tot; c += SEL_THREADS) s.hist[c] = 0;
     if (threadIdx.x == 0) s.scal[SC_GLOBAL] = 0;
     __syncthreads();
   };
@@ -676,14 +686,61 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
     __syncthreads();
     int n = *cnt;
     const int guessed = n;
+    int listed = n;
+    if (n < P && lo > 1) {  // too few: once more from half the gain or a quarter of it
+      __syncthreads();
+      if (threadIdx.x == 0) *cnt = 0;
+      s.ck[threadIdx.x] = 0;  // LCAP == SEL_THREADS
+      lo = max(1ull, 4 * n < P ? lo >> 2 : lo >> 1);
+      __syncthreads();
+      list_candidates(gain_addr, ga, s, N, lo, cnt);
+      __syncthreads();
+      listed = n = *cnt;
+    }
     if (n > LCAP || (n < P && lo > 1)) {  // the guess missed (uniform over the cluster)
       __syncthreads();
       if (threadIdx.x == 0) *cnt = 0;
       s.ck[threadIdx.x] = 0;  // LCAP == SEL_THREADS
       __syncthreads();
-      n = pool_search(gain_addr, ga, s, N, P, cnt, &lo);
+      listed = n = pool_search(gain_addr, ga, s, N, P, cnt, &lo);
     }
     const int Pt = min(n, P);
+    // Ranking costs the square of the list: a long one is cut first, to those at or
+    // above a key found by halving the keys' range (a barrier a step) that leaves P to
+    // RANK_MAX of them (more where keys are equal).  405 candidates: 5 us, now 0.9.
+    constexpr int RANK_MAX = SEL_THREADS / 4;  // ranked in one turn
+    if (n > max(RANK_MAX, P)) {
+      const uint32_t key = s.ck[threadIdx.x];  // LCAP == SEL_THREADS; past the list: 0
+      const int jq = s.cj[threadIdx.x];
+      const uint32_t top = __reduce_max_sync(FULL, key);
+      if (lane == 0) s.wsum[wid] = (int)top;
+      __syncthreads();
+      uint32_t above = __reduce_max_sync(FULL, (uint32_t)s.wsum[lane & (SEL_WARPS - 1)]) + 1;
+      uint32_t from = gain_key(lo);
+      while (n > max(RANK_MAX, P) && above - from > 1) {  // n keys >= from, fewer than P >= above
+        const uint32_t mid = from + ((above - from) >> 1);
+        const int c = __syncthreads_count(key >= mid);
+        if (c >= P) {
+          from = mid;
+          n = c;
+        } else {
+          above = mid;
+        }
+      }
+      const bool in = (int)threadIdx.x < listed && key >= from;
+      const unsigned bal = __ballot_sync(FULL, in);
+      __syncthreads();  // every key and token is in a register, wsum has been read
+      s.ck[threadIdx.x] = 0;
+      if (lane == 0) s.wsum[wid] = __popc(bal);
+      __syncthreads();
+      const int before = __reduce_add_sync(FULL, lane < wid ? s.wsum[lane] : 0);
+      if (in) {
+        const int at = before + __popc(bal & lanemask_lt());
+        s.ck[at] = key;
+        s.cj[at] = jq;
+      }
+      __syncthreads();
+    }
     // rank every candidate by its key among them (4 lanes each, four keys a load);
     // slot = rank
     {
@@ -769,15 +826,15 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
     }
     // Threshold of the next pool, by the last thread while others work: the gain g at
     // rank P, lowered by the smoothed fall of g per round and by a factor that the
-    // lists' lengths steer to about 3 P / 2 candidates.
+    // lists' lengths steer to 3 P / 2 to 3 P candidates.
     auto next_threshold = [&]() {
       unsigned long long next = 1;
       if (Pt == P) {
         const float g = key_gain((uint32_t)s.scal[SC_KEY]);
         if (glast > 0.f) fall = 0.5f * (fall + fminf(1.f, fmaxf(0.4f, __fdividef(g, glast))));
         glast = g;
-        room *= guessed > 5 * P ? 1.25f : guessed > 3 * P ? 1.12f : guessed > 7 * P / 4 ? 1.05f
-                : guessed < P ? 0.85f : guessed < 5 * P / 4 ? 0.95f : 1.f;
+        room *= guessed > 6 * P ? 1.25f : guessed > 4 * P ? 1.12f : guessed > 3 * P ? 1.05f
+                : guessed < P ? 0.85f : guessed < 3 * P / 2 ? 0.95f : 1.f;
         room = fminf(0.97f, fmaxf(0.3f, room));
         next = (unsigned long long)__float2ull_rz(g * fall * room);
         if (next == 0) next = 1;
