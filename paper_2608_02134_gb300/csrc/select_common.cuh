@@ -196,7 +196,7 @@ __device__ inline int block_exclusive_scan(int v, int* wsum, int* total) {
 constexpr int CBINS = 64;       // coarse bins: the binary exponent of a gain
 struct PoolScratch {
   int* hist;           // [HBINS] fine bins, all zero on entry and on return
-  int* coarse;         // [CBINS] coarse bins, all zero on entry and on return
+  int* coarse;         // [CBINS] coarse bins
   int* bnd;            // [N]  tokens of the boundary bin, ascending
   short* key;          // [N]  bucket of every token (-1: not a candidate)
   unsigned char* pk;   // [N]  boundary tokens that enter the pool
@@ -229,8 +229,7 @@ constexpr int ID_BITS = 15;    // token and slot indices are below GMC_MAX_N_LON
 // in every block that calls this with the same data.  Returns Pt.
 //
 // Every gain gets an 11-bit bucket (exponent, 5 mantissa bits; monotone in u).
-// One pass counts the buckets and their exponents (64 coarse bins, counted
-// once per warp and exponent); every warp then finds the boundary bucket
+// One pass counts the buckets, their sums per exponent are 64 coarse bins; every warp then finds the boundary bucket
 // holding the P-th largest gain from the coarse bins and the 32 fine bins of
 // one exponent.  Warp w owns 32-token chunks [w * nc, (w + 1) * nc) (lane =
 // token within a chunk, so every shared access is conflict-free); ballots
@@ -276,11 +275,12 @@ __device__ inline int select_pool(const long long* u, const unsigned char* sel, 
         }
         w.key[j] = (short)kb;
       }
-      // exponents: one atomic per warp and distinct exponent
-      const int e = kb >= 0 ? kb >> 5 : -1;
-      const unsigned same = __match_any_sync(FULL, e);
-      if (e >= 0 && (same & lt) == 0) atomicAdd(&w.coarse[e], __popc(same));
     }
+  }
+  __syncthreads();
+  for (int e = wid; e < CBINS; e += nw) {  // an exponent's 32 buckets
+    const int c = __reduce_add_sync(FULL, w.hist[e * 32 + lane]);
+    if (lane == 0) w.coarse[e] = c;
   }
   __syncthreads();
   // 2. boundary bucket, found by every warp alike: coarse bins from the top,
@@ -339,10 +339,7 @@ __device__ inline int select_pool(const long long* u, const unsigned char* sel, 
   for (int c = 0; c < nc; ++c) {
     const int j = (wid * nc + c) * 32 + lane;
     const int kb = j < N ? w.key[j] : -1;
-    if (kb >= 0) {
-      w.hist[kb] = 0;
-      w.coarse[kb >> 5] = 0;
-    }
+    if (kb >= 0) w.hist[kb] = 0;
   }
   int pre, nb;
   {
