@@ -78,13 +78,12 @@ cudaError_t launch_gram_simt(const Dims& dm, const void* hidden, Scratch& s, cud
 }
 
 cudaError_t launch_gram(const Dims& dm, const void* hidden, Scratch& s, cudaStream_t st) {
-  // bf16 states with at least one full 128-row tile: tcgen05.  The split-contraction
-  // Gram of k_gram_tc.cu gives a 128-row block pair to two CTAs and keeps more SMs busy
-  // on a small image (N = 1,296: 24 us with the norms, the general kernel 45), but from
-  // its third wave of CTAs on the general kernel in symmetric mode (k_gemm_tc.cu) is
-  // ahead: N = 2,025 (two waves) 39 and 49 us, N = 2,304 (2.5) 53 and 41, N = 2,592 65
-  // and 47, three images of 1,296 55 and 47.  fp32 states (exact fp32 products) and
-  // tiny grids: the CUDA-core kernel above.
+  // bf16 states with at least one full 128-row tile: tcgen05.  Problems whose
+  // 128 x 256 tiles on or above the diagonal fill the GPU at least once (the
+  // document page, serving batches) run the general kernel in symmetric mode
+  // (k_gemm_tc.cu); a single smaller image runs the split-contraction Gram of
+  // k_gram_tc.cu, which keeps more SMs busy at that size.  fp32 states (exact
+  // fp32 products) and tiny grids: the CUDA-core kernel above.
   if (!gram_tc_supported(dm)) return launch_gram_simt(dm, hidden, s, st);
   static int sms = 0;
   if (sms == 0) {
@@ -95,8 +94,7 @@ cudaError_t launch_gram(const Dims& dm, const void* hidden, Scratch& s, cudaStre
       sms = 152;
     }
   }
-  const long long blocks = ceil_div(dm.N, 128);  // of rows; the split Gram's CTAs:
-  if (dm.N >= 256 && blocks * (blocks + 1) * dm.B > 2LL * sms) {
+  if (dm.N >= 256 && gemm_sym_ctas(dm.N, dm.B) >= sms) {
     GemmArgs g{};
     g.B = dm.B; g.M = dm.N; g.Nn = dm.N; g.Kd = dm.D;
     g.a_img = dm.N; g.b_img = dm.N; g.a_text = 1; g.b_text = 1;
