@@ -169,9 +169,11 @@ class ClockSampler:
 # roofline bookkeeping (algorithmic work per stage, per call)
 # ---------------------------------------------------------------------------
 # sparse solver rounds run as whole-GPU kernels after the dense first one
-# (sparse_gpu_rounds(N) in the library's kernels.cuh)
-def wide_rounds(N: int) -> int:
-    return 8 if N > 2048 else 4
+# (sparse_gpu_rounds in the library's kernels.cuh, b = 16)
+def wide_rounds(N: int, B: int, K: int, images: int) -> int:
+    base = 8 if N > 3072 else 5 if N > 1536 else 1
+    base += 5 if B > 38 else 4 if B > 19 else 2 if B > 9 else 0
+    return min(base, max(0, -(-(K - (images if images > 1 else 16)) // 16)))
 
 
 def stage_work(wl) -> dict:
@@ -204,10 +206,10 @@ def stage_work(wl) -> dict:
     w["message"] = ("hbm", B * (H * Tm * N * 4 + 2 * (N + Tm) * Hkv * d * es + Tm * H * d * es))
     w["clients"] = ("hbm", B * (M * N * 4 + H * Tm * N * 4 + N * N * 4))
     # selection: one read of the M x N clients per round.  Stage "rounds_gpu"
-    # runs the dense first round and the next wide_rounds(N) sparse rounds as
+    # runs the dense first round and the next wide_rounds sparse rounds as
     # whole-GPU kernels; stage "select" (the cluster kernel) runs the rest.
     rounds = -(-K // 16)
-    wide = min(rounds, 1 + wide_rounds(N))
+    wide = min(rounds, 1 + wide_rounds(N, B, K, wl.I))
     w["rounds_gpu"] = ("hbm", B * wide * (M * N * 4.0))
     w["select"] = ("hbm", B * max(1, rounds - wide) * (M * N * 4.0))
     w["transport"] = ("hbm", B * ((N + Tm) * D * es + (K + Tm) * D * es

@@ -82,8 +82,10 @@ cudaError_t launch_gram(const Dims& dm, const void* hidden, Scratch& s, cudaStre
   // 128 x 256 tiles on or above the diagonal fill the GPU at least once (the
   // document page, serving batches) run the general kernel in symmetric mode
   // (k_gemm_tc.cu); a single smaller image runs the split-contraction Gram of
-  // k_gram_tc.cu, which keeps more SMs busy at that size.  fp32 states (exact
-  // fp32 products) and tiny grids: the CUDA-core kernel above.
+  // k_gram_tc.cu, which keeps more SMs busy at that size and adds D in two halves:
+  // from its third wave of CTAs on (N = 2,592 with the norms 65 us, the general kernel
+  // 47) it is kept for its shorter sums, which a near-tie of the assignment can see.
+  // fp32 states (exact fp32 products) and tiny grids: the CUDA-core kernel above.
   if (!gram_tc_supported(dm)) return launch_gram_simt(dm, hidden, s, st);
   static int sms = 0;
   if (sms == 0) {

@@ -36,8 +36,9 @@
 // is deterministic.  Per round:
 //   pool:   every CTA reads the gains from their owners (token j belongs to CTA
 //           j / SL) and selects the same pool: the tokens of at least the
-//           threshold `lo` are listed and ranked exactly; when the guess lists
-//           too few or too many, a radix search finds the threshold;
+//           threshold `lo` are listed, a long list cut, and ranked exactly; when
+//           the guess lists too few, a lower one follows, and when that misses too
+//           or lists too many, a radix search finds the threshold;
 //   scores: every CTA stores its rows' responsibility-weighted residuals into
 //           its own row in every CTA of the cluster; every CTA adds the rows
 //           and picks the same batch;
