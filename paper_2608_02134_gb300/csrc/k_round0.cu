@@ -29,6 +29,11 @@
 namespace gmc {
 
 namespace {
+// Threads of a sparse round's pool block: a turn takes four tokens a thread.  1,024
+// from N = 2,048 on (a second turn costs more than the wider barriers).
+constexpr int POOL_THREADS = 1024;
+int pool_threads(int N) { return N > 2048 ? POOL_THREADS : POOL_THREADS / 2; }
+
 // The responsibility and filter kernels have ROWS warps a block (a template
 // parameter: 16 for one image, 8 for a batch) and take `rpw` consecutive rows per
 // warp.  Every block pays for tables of N tokens, and the filters end with a global
@@ -318,24 +323,31 @@ __global__ void __launch_bounds__(32 * ROWS) k_r0_filter(
 
 // ---- sparse rounds on the whole GPU -------------------------------------------
 
-__global__ void __launch_bounds__(512) k_rg_pool(const long long* __restrict__ ucur,
-                                                   long long* unext, int B, int N, int K, int P,
-                                                   const int32_t* toff, int Tmax,
-                                                   const int32_t* __restrict__ order,
-                                                   int32_t* pool0, int32_t* info, long long* sc,
-                                                   TraceView tv) {
+// One block per image: a chain of memory round trips and barriers.  The gains are read
+// once, into shared memory and into the buffer the filter adds its changes to, and
+// nothing says which tokens are selected: their entries are all dead, so their gains are
+// exactly zero and they are no candidates.  Two reads of the gains and one of the
+// selected tokens took N = 1,296 7.0 us, 2,592 8.2, 4,096 9.4; now 6.7, 6.6 and 7.3.
+__global__ void __launch_bounds__(POOL_THREADS, 1) k_rg_pool(const long long* __restrict__ ucur,
+                                                          long long* unext, int B, int N, int K,
+                                                          int P, const int32_t* toff, int Tmax,
+                                                          int32_t* pool0, int32_t* info,
+                                                          long long* sc, TraceView tv) {
   grid_dep_wait();
   extern __shared__ __align__(16) char sm_rgp[];
   const int b = blockIdx.x;
+  const int S = info[b * INFO_W + 1], rd = info[b * INFO_W + 2];
+  int hint = info[b * INFO_W + 5];
   for (int k = threadIdx.x; k < P; k += blockDim.x) sc[(size_t)b * P + k] = 0;
   // the next gains start from these: the filter adds only the changes of the
   // rows whose coverage grows
-  for (int j = threadIdx.x; j < N; j += blockDim.x) unext[(size_t)b * N + j] = ucur[(size_t)b * N + j];
-  const int S = info[b * INFO_W + 1], rd = info[b * INFO_W + 2];
+  const long long* ub = ucur + (size_t)b * N;
+  long long* un = unext + (size_t)b * N;
   // nothing to do here once the budget is met or when the first round found
   // no gain: the cluster kernel handles those cases
   const bool skip = (toff && text_geom(toff, b, B, Tmax, nullptr).T == 0) || rd == 0 || S >= K;
   if (skip) {
+    for (int j = threadIdx.x; j < N; j += blockDim.x) un[j] = ub[j];
     if (threadIdx.x == 0) info[b * INFO_W] = 0;
     return;
   }
@@ -354,24 +366,20 @@ __global__ void __launch_bounds__(512) k_rg_pool(const long long* __restrict__ u
   int* pool = reinterpret_cast<int*>(p);    p += sizeof(int) * P;
   w.key = reinterpret_cast<short*>(p);     p += sizeof(short) * (size_t)N;
   w.pk = reinterpret_cast<unsigned char*>(p); p += (size_t)N;
-  unsigned char* self = reinterpret_cast<unsigned char*>(p);
+  unsigned char* none = reinterpret_cast<unsigned char*>(p);
   // the gains in shared memory (select_pool reads them often): copied here
   // without a boundary hint, else by the window pool's first pass
-  int hint = info[b * INFO_W + 5];
-  const long long* ub = ucur + (size_t)b * N;
   for (int j = threadIdx.x; j < N; j += blockDim.x) {
-    self[j] = 0;
-    if (hint < 0) ug[j] = ub[j];
+    none[j] = 0;
+    if (hint < 0) un[j] = ug[j] = ub[j];
   }
   for (int h = threadIdx.x; h < sel::HBINS; h += blockDim.x) w.hist[h] = 0;
   if (threadIdx.x < sel::CBINS) w.coarse[threadIdx.x] = 0;
   for (int q = threadIdx.x; q < sel::WBINS + 4; q += blockDim.x) ws.win[q] = 0;
   __syncthreads();
-  for (int q = threadIdx.x; q < S; q += blockDim.x) self[order[(size_t)b * K + q]] = 1;
-  __syncthreads();
-  int Pt = sel::select_pool_window([&](int j) { return ub[j]; }, ug, self, N, P, ws, pool,
+  int Pt = sel::select_pool_window([&](int j) { return un[j] = ub[j]; }, ug, none, N, P, ws, pool,
                                    nullptr, &hint);
-  if (Pt < 0) Pt = sel::select_pool(ug, self, N, P, w, pool, nullptr, nullptr, &hint);
+  if (Pt < 0) Pt = sel::select_pool(ug, none, N, P, w, pool, nullptr, nullptr, &hint);
   if (tv.base)
     for (int j = threadIdx.x; j < N; j += blockDim.x) tv.gains(b, rd, N)[j] = ug[j];
   for (int k = threadIdx.x; k < P; k += blockDim.x) pool0[(size_t)b * P + k] = k < Pt ? pool[k] : -1;
@@ -676,8 +684,8 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   for (int rr = 1; rr <= rounds; ++rr) {
     long long* ucur = rr % 2 == 1 ? r0.u1 : r0.u2;
     long long* unext = rr % 2 == 1 ? r0.u2 : r0.u1;
-    launch_k(k_rg_pool, B, 512, psm, st, 1, (const long long*)ucur, unext, B, N, K, P,
-             uniform ? nullptr : toff, T, (const int32_t*)order, r0.pool, r0.info, r0.s0, tv);
+    launch_k(k_rg_pool, B, pool_threads(N), psm, st, 1, (const long long*)ucur, unext, B, N, K, P,
+             uniform ? nullptr : toff, T, r0.pool, r0.info, r0.s0, tv);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     launch_k(k_rg_rho<ROWS>, grid, 32 * ROWS, rsm, st, 1, (const float*)C, (const uint16_t*)scol,
              (const float*)r0.bcov, (const int32_t*)r0.cnt, B, N, M, H, L2, toff, T, uniform,
