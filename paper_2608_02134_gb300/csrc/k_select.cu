@@ -588,8 +588,8 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
     // every entry by one thread, MU loads in flight (rows are very uneven); tokens
     // counted in cs[j + 1].  Its row: the row of its 32 entries' first one, from a table
     // (a binary search of the rows' offsets for each, kept in the histogram's bins), then a
-    // step or two; a search for every entry was most of the time before the first round (22
-    // us at N = 1,296, now 13).
+    // step or two; a search for every entry was most of the time before the first round (21
+    // us at N = 1,296, now 12).
     for (int c = threadIdx.x; 32 * c < tot; c += SEL_THREADS) {
       int lo2 = 0, hi2 = nrows;  // rptr[lo2] <= p < rptr[hi2]
       while (hi2 - lo2 > 1) {
