@@ -15,7 +15,7 @@
 // instead of scanning the whole assignment.
 //
 // Layout.  A block takes AT = 32 consecutive tokens, one per lane, and its
-// ASSIGN_WARPS warps split the support (warp w: entries w, w + 8, ...).  The
+// ASSIGN_WARPS warps split the support (warp w: entries w, w + 16, ...).  The
 // cosines of support entry k with the block's tokens are one contiguous
 // 128-byte segment: row S_k of the symmetric N x N cosine matrix, or row k of
 // the K x N support cosines of long prefixes (cs mode).  So both passes read
