@@ -125,6 +125,15 @@ __global__ void __launch_bounds__(WP_THREADS, 1) k_w_pool(WideState w, WideGeom 
   }
   sel::PoolScratch ps;
   char* p = sm_wp;
+  sel::WindowScratch ws{};
+  long long* ug = nullptr;  // win: the gains, staged for the pool's passes
+  if (win) {  // first, where its 16-byte loads are aligned whatever N is
+    ws.win = reinterpret_cast<int*>(p);       p += sizeof(int) * (sel::WBINS + 4);
+    ws.cu = reinterpret_cast<long long*>(p);  p += sizeof(long long) * sel::WCAP;
+    ws.cj = reinterpret_cast<int*>(p);        p += sizeof(int) * sel::WCAP;
+    ug = reinterpret_cast<long long*>(p);     p += sizeof(long long) * (size_t)N;
+    for (int q = threadIdx.x; q < sel::WBINS + 4; q += blockDim.x) ws.win[q] = 0;
+  }
   ps.hist = reinterpret_cast<int*>(p);       p += sizeof(int) * sel::HBINS;
   ps.bnd = reinterpret_cast<int*>(p);        p += sizeof(int) * (size_t)N;
   ps.wsum = reinterpret_cast<int*>(p);       p += sizeof(int) * 32;
@@ -137,17 +146,6 @@ __global__ void __launch_bounds__(WP_THREADS, 1) k_w_pool(WideState w, WideGeom 
   p = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + 15) & ~static_cast<uintptr_t>(15));
   ps.bval = reinterpret_cast<long long*>(p);  // the boundary bucket's gains
   ps.bcap = min(N, W_BCAP);
-  p += sizeof(long long) * (size_t)ps.bcap;
-  sel::WindowScratch ws{};
-  long long* ug = nullptr;  // win: the gains, staged for the pool's passes
-  if (win) {
-    p = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(p) + 15) & ~static_cast<uintptr_t>(15));
-    ug = reinterpret_cast<long long*>(p);     p += sizeof(long long) * (size_t)N;
-    ws.cu = reinterpret_cast<long long*>(p);  p += sizeof(long long) * sel::WCAP;
-    ws.cj = reinterpret_cast<int*>(p);        p += sizeof(int) * sel::WCAP;
-    ws.win = reinterpret_cast<int*>(p);
-    for (int q = threadIdx.x; q < sel::WBINS + 4; q += blockDim.x) ws.win[q] = 0;
-  }
   for (int j = threadIdx.x; j < N; j += blockDim.x) {
     none[j] = 0;
     if (tv.base) tv.gains(b, rd, N)[j] = ucur[j];
@@ -705,7 +703,7 @@ cudaError_t launch_wide_select(const WideState& w, const WideGeom& g, const gmc_
   const size_t fsm = sizeof(unsigned long long) * (size_t)N;
   const size_t fsm_dense = fsm + sizeof(float) * sel::ROW_STEP * (size_t)fwarps;
   // the window pool's extra shared memory: the staged gains and its scratch
-  const size_t wsm = 16 + sizeof(long long) * ((size_t)N + sel::WCAP) + sizeof(int) * sel::WCAP +
+  const size_t wsm = sizeof(long long) * ((size_t)N + sel::WCAP) + sizeof(int) * sel::WCAP +
                      sizeof(int) * (sel::WBINS + 4);
   const int win = P <= sel::WCAP / 2 && psm + wsm <= 227 * 1024 ? 1 : 0;
   const size_t psm_w = psm + (win ? wsm : 0);

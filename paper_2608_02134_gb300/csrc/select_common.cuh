@@ -533,8 +533,8 @@ constexpr int WTOP = 8;     // window buckets above the hint
 constexpr int WCAP = 256;   // candidates ranked exactly
 constexpr int WU = 4;       // tokens a thread handles per pass step
 struct WindowScratch {
-  int* win;        // [WBINS + 4] window bins (top bucket first) and 4 counters;
-                   // all zero on entry and on return
+  int* win;        // [WBINS + 4] window bins (top bucket first) and 4 counters, on 16
+                   // bytes (read four bins a load); all zero on entry and on return
   long long* cu;   // [WCAP] candidates' gains
   int* cj;         // [WCAP] candidates' tokens
 };

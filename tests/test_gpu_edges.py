@@ -76,6 +76,21 @@ def test_wide_solver_sizes(kind, B, M, N, K, b, mult):
     _check_select(_clients(kind, B, M, N, 7 + N), K, batch_b=b, pool_mult=mult)
 
 
+# the wide solver's window pool (at most 128 slots, beyond the cluster solver's
+# bytes) at odd token counts, where the staged gains end on 8 bytes and not on 16,
+# over enough rounds that the window is read: pools of 64 and 128, one
+# image and two
+@pytest.mark.parametrize("B,M,N,K,b", [(1, 4300, 8191, 200, 32), (1, 7700, 8191, 70, 16),
+                                       (2, 4300, 8189, 100, 32)])
+def test_window_pool_at_odd_token_counts(B, M, N, K, b):
+    from paper_2608_02134_gb300 import gmc
+    from tests.test_gpu_stages import _check_select
+    n0 = gmc.launch_count()
+    _check_select(_clients("plain", B, M, N, 3 + N), K, batch_b=b)
+    # the whole-GPU solver ran (four launches a round)
+    assert gmc.launch_count() - n0 == 3 + 4 * (-(-K // b)) + 1 + 1
+
+
 # transport: fewer and more member rows than a thread has in flight, lists of more
 # than 64 members (one carrier takes every token), one list for the block (N above
 # 4,096), a row that is one CTA and one that is eight, more text rows than carriers,
