@@ -45,6 +45,13 @@ struct LaneSum {
   }
 };
 
+// a + x, *e its rounding error (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float x, float* e) {
+  const float t = a + x, z = t - a;
+  *e = (a - (t - z)) + (x - z);
+  return t;
+}
+
 // A 16-byte shared load that is issued where it stands: the weights of a pair
 // re-read their probe values instead of holding 2 HB of them in registers
 // beside the sums.
@@ -74,6 +81,15 @@ __host__ __device__ constexpr int hs_stride(int H, int HB, int TT) {
 // offsets from one address and feed HB^2 FMAs.  Then every lane applies its
 // token's weights Z_h . Z_g + sigma_h sigma_g and the lanes are added.  With fewer
 // pairs than HS_WARPS the queries are dealt to `ts` slices of warps.
+//
+// Precision.  The squares W2 of a token are a lane's sum over the queries: every FOLD
+// stages (32 queries of a lane, 16 with TT > 1) it goes into a total whose rounding
+// errors are kept (Knuth's two-sum), in the lane's own words of shared memory.  Against
+// 64 bits, root mean square over the tokens at T = 64, 128, 256, TT = 1: 6.8e-8, 5.3e-8,
+// 4.3e-8 (one chain over all queries: 1.2e-7, 1.7e-7, 2.3e-7); it costs 2% of the kernel
+// there.  A pair's Gram entry keeps its one chain: its errors average out over
+// the tokens, and rounding the sum to fp32 is what is left (1.1e-8 to 2e-8 of the norms'
+// product at T = 64 to 256, with chains of 32 as well).
 // TT: 1 reads whole 128-byte lines; 2 and 4 make more, smaller blocks for a
 // single small image (head_tokens).  Bound by the shared-memory and FMA issue
 // of 14 loads against 49 FMAs and the two stages' barriers.  The 4 x 4 tiles
@@ -87,11 +103,13 @@ __global__ void __launch_bounds__(32 * HS_WARPS, HB == 8 ? 1 : 2)
                  const float* __restrict__ sigma, const int32_t* toff, int B, int N, int Tmax,
                  int H, float wq, float* hgpart, int nHG, float* W2, int ts, uint32_t* status) {
   grid_dep_wait();
-  constexpr int TOK = 32 / TT, NV = HB * HB, TC = HS_TC * TT;
+  constexpr int TOK = 32 / TT, NV = HB * HB, TC = HS_TC * TT, FOLD = TT == 1 ? 4 : 2;
   extern __shared__ __align__(16) float sm_hs[];  // [2][TC][stride], then Z [nb HB][TOK]
   __shared__ float sgm[GMC_MAX_HEADS + 8];       // sigma_h of the image
   __shared__ float part[HS_WARPS][NV];        // slices' sums of a pair (ts > 1)
-  __shared__ float w2s[HS_WARPS][HB][TOK];    // slices' query-weighted squares (ts > 1)
+  // query-weighted squares: a lane's total and its rounding errors, then (ts > 1)
+  // the slices' sums
+  __shared__ float w2s[HS_WARPS][HB][32], w2e[HS_WARPS][HB][32];
   const int b = blockIdx.y;
   const TextGeom tg = text_geom(toff, b, B, Tmax, status);
   if (tg.T == 0) return;
@@ -190,6 +208,15 @@ __global__ void __launch_bounds__(32 * HS_WARPS, HB == 8 ? 1 : 2)
               for (int v = 0; v < HB; ++v) acc[u * HB + v] = fmaf(x[u], x[v], acc[u * HB + v]);
             }
           }
+          if (st % FOLD == FOLD - 1 && st + 1 < nst) {
+#pragma unroll
+            for (int u = 0; u < HB; ++u) {
+              float e = 0.f;
+              w2s[w][u][lane] = st < FOLD ? w2[u] : two_sum(w2s[w][u][lane], w2[u], &e);
+              w2e[w][u][lane] = st < FOLD ? 0.f : w2e[w][u][lane] + e;
+              w2[u] = 0.f;
+            }
+          }
         } else {
 #pragma unroll 1
           for (int t0 = slice * TT; t0 < tend; t0 += ts * TT, row += ts * TT * stride) {
@@ -212,6 +239,11 @@ __global__ void __launch_bounds__(32 * HS_WARPS, HB == 8 ? 1 : 2)
     if (diag) {  // sum_t nu_t A[h,t,i]^2 of the block's heads
 #pragma unroll
       for (int u = 0; u < HB; ++u) {
+        if (nst > FOLD) {
+          float e;
+          const float t = two_sum(w2s[w][u][lane], w2[u], &e);
+          w2[u] = t + (w2e[w][u][lane] + e);
+        }
 #pragma unroll
         for (int o = TOK; o < 32; o <<= 1) w2[u] += __shfl_xor_sync(FULL, w2[u], o);
         if (ts > 1) {
@@ -452,31 +484,39 @@ __device__ void cluster_heads(const float* hgb, int b, int T, int N, int H, int 
   }
 }
 
-// A sum held as hi + lo, every addition's rounding error kept in lo (Knuth's
-// two-sum): about 48 bits, on the fp32 pipe.  fp64 additions run at a small
-// fraction of its rate on this GPU: with them the reduction below took 15.3
-// instead of 10.3 us at the 162 partials of N = 1,296, H = 28.
-struct Sum2 {
-  float hi = 0.f, lo = 0.f;
+// A sum of fp32 terms in three words: every addition's rounding error is kept in mid
+// (Knuth's two-sum), and that sum's errors in lo: about 72 bits, all on the fp32 pipe.
+// fp64 additions run at a small fraction of its rate on this GPU: the reduction below
+// took 33 us longer with them in a batch of 32 images, 2 us at one (two words,
+// about 48 bits: 1 us less than three).
+struct Sum3 {
+  float hi = 0.f, mid = 0.f, lo = 0.f;
   __device__ __forceinline__ void add(float x) {
-    const float t = hi + x, z = t - hi;
-    lo += (hi - (t - z)) + (x - z);
-    hi = t;
+    float e;
+    hi = two_sum(hi, x, &e);
+    mid = two_sum(mid, e, &e);
+    lo += e;
   }
-  __device__ __forceinline__ void add(const Sum2& o) {
+  __device__ __forceinline__ void add(const Sum3& o) {
+    float e;
     add(o.hi);
-    lo += o.lo;
+    mid = two_sum(mid, o.mid, &e);
+    lo += e + o.lo;
   }
   // the sum over the lanes that differ in the bits below `n` (a fixed tree)
   __device__ __forceinline__ void reduce(int n) {
     for (int o = n / 2; o > 0; o >>= 1) {
-      Sum2 y;
+      Sum3 y;
       y.hi = __shfl_xor_sync(FULL, hi, o);
+      y.mid = __shfl_xor_sync(FULL, mid, o);
       y.lo = __shfl_xor_sync(FULL, lo, o);
       add(y);
     }
   }
-  __device__ __forceinline__ float value() const { return hi + lo; }
+  // rounded to fp32 once; a sum past its range is infinite, and so are its errors not numbers
+  __device__ __forceinline__ float value() const {
+    return isfinite(hi) ? (float)((double)hi + ((double)mid + (double)lo)) : hi;
+  }
 };
 
 // The pattern Gram of image blockIdx.y: the token blocks' partials added up.
@@ -495,7 +535,7 @@ __global__ void __launch_bounds__(32 * HR_WARPS)
                 int cluster, const ViewGrams vg, int nrb, uint32_t* status) {
   grid_dep_wait();
   extern __shared__ float sm_hc[];
-  __shared__ Sum2 psum[HR_WARPS][33];
+  __shared__ Sum3 psum[HR_WARPS][33];
   __shared__ int last;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, b = blockIdx.y;
   const int HH = H * H, HE = HH + H;
@@ -505,7 +545,7 @@ __global__ void __launch_bounds__(32 * HR_WARPS)
   if ((int)blockIdx.x < ngb) {
     const int p = blockIdx.x * 32 + lane;
     const float* src = hgpart + (size_t)b * nHG * HH + p;
-    Sum2 s;
+    Sum3 s;
     if (p < HH) {
       constexpr int U = 12;
       for (int k0 = w; k0 < nHG; k0 += U * HR_WARPS) {
@@ -523,13 +563,13 @@ __global__ void __launch_bounds__(32 * HR_WARPS)
     __syncthreads();
     // half-warp: one entry, lane = source warp
     const int pe = 2 * w + (lane >> 4), p2 = blockIdx.x * 32 + pe;
-    Sum2 t = psum[lane & 15][pe];
+    Sum3 t = psum[lane & 15][pe];
     t.reduce(HR_WARPS);
     if ((lane & 15) == 0 && p2 < HH) HG[(size_t)b * HE + p2] = t.value();
   } else {
     const int h = (blockIdx.x - ngb) * HR_WARPS + w;
     if (h < H) {
-      Sum2 s;
+      Sum3 s;
       const float* r = rs + ((size_t)b * H + h) * nRS * Tmax;
       const int n = nRS * tg.T;  // (part, query) pairs, eight per lane in flight
       for (int k0 = lane; k0 < n; k0 += 32 * 8) {

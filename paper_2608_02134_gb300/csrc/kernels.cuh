@@ -90,8 +90,9 @@ struct Scratch {
   uint32_t* tick3;   // [B]            last-block tickets of the head-Gram reduction (same)
   float* gatev;      // [B][4]         Delta_bar, s_x, mean message energy
   float* sigma;      // [B][H]         mass coordinate sigma_h
-  float* hgpart;     // [B][nHG][H*H]  block partials of the head-pattern Gram
-  float* HG;         // [B][H*H + H]   head-pattern Gram, then sum_t rs[h,t] per head
+  float* hgpart;     // [B][nHG][H*H]  block partials (fp32 sums) of the head-pattern Gram
+  float* HG;         // [B][H*H + H]   head-pattern Gram, then sum_t rs[h,t] per head, each
+                     //                summed in 72 bits and rounded once
   float* W2;         // [B][H][N]      sum_t nu_t A[h,t,i]^2
   float* omega;      // [B][H]
   float* ebar;       // [B][N]  message energy e_i (the assignment divides by its mean)

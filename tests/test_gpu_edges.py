@@ -29,6 +29,48 @@ def test_head_statistics_sizes(H, Hkv, T, gh, gw, B):
     _compare(wl, range(B))
 
 
+# the query-weighted squares over many queries (whole lines of tokens, one lane a
+# token): every head sees the same nearly even attention, so that neither the heads
+# nor a few large terms hide how the sum over the queries was rounded.  Root mean
+# square error over the tokens: the attention's, the probe's and the heads' fp32 leave
+# 8.5e-8 and 6.1e-8; with one fp32 chain over the queries it is 1.5e-7 and 9.5e-8
+@pytest.mark.parametrize("B,T,bar", [(8, 256, 1.1e-7), (8, 100, 7.5e-8)])
+def test_message_energy_over_many_queries(B, T, bar):
+    from paper_2608_02134_gb300 import gmc
+    from tests import parity
+    gh, gw, H, Hkv, d, D, K = 36, 36, 28, 4, 64, 64, 16
+    N = gh * gw
+    g = torch.Generator(device="cuda")
+    g.manual_seed(T)
+    rnd = lambda *s: torch.randn(s, generator=g, device="cuda")  # noqa: E731
+    hid = rnd(B, N + T, D).bfloat16()
+    key = rnd(B, 1, N + T, 1, d).expand(-1, -1, -1, Hkv, -1)
+    kv = torch.cat([key, rnd(B, 1, N + T, Hkv, d)], 1).bfloat16().contiguous()
+    q = (0.5 * rnd(B, T, 1, d)).expand(-1, -1, H, -1).bfloat16().contiguous()
+    pos = torch.zeros(B * 3 * (N + T), dtype=torch.int32, device="cuda")
+    W = rnd(H, d, 4) / d ** 0.5
+    comp = gmc.Compressor(B, gh, gw, T, H, Hkv, d, D, K, gmc.GMC_BF16, trace=True)
+    out = comp.run(hid.view(-1, D), kv.view(-1), q.view(-1), pos, W)
+    torch.cuda.synchronize()
+    assert comp.status() == 0
+    tr = parity.parse_trace(out.trace.cpu().numpy(), out.layout, B, K, H, N,
+                            comp.params.max_head_clusters)
+    nu = torch.ones(T, dtype=torch.float64, device="cuda")
+    nu[-1] = comp.params.terminal_q_weight
+    nu /= nu.sum()
+    for b in {0, B - 1}:
+        S = q[b, :, 0].double() @ kv[b, 0, :, 0].double().T / d ** 0.5
+        S[:, N:] = S[:, N:].masked_fill(torch.ones(T, T, device="cuda").triu(1).bool(), -torch.inf)
+        W2 = (nu[:, None] * torch.softmax(S, 1)[:, :N].square()).sum(0)
+        V = kv[b, 1, :N].double().repeat_interleave(H // Hkv, 1)
+        Z2 = torch.einsum("nhd,hdr->nhr", V, W.double()).square().sum(2)
+        om = torch.tensor(tr[b].omega, dtype=torch.float64, device="cuda")
+        e = ((Z2 + Z2.mean(0) / 4) @ om * W2).sqrt()
+        got = torch.tensor(tr[b].ebar, dtype=torch.float64, device="cuda")
+        rel = (got / (e / e.mean()) - 1).square().mean().sqrt()
+        assert float(rel) <= bar, float(rel)
+
+
 def _clients(kind, B, M, N, seed):
     r = np.random.default_rng(seed)
     if kind == "equal":      # every token its own row of one value: all gains tie in every round
