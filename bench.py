@@ -168,16 +168,9 @@ class ClockSampler:
 # ---------------------------------------------------------------------------
 # roofline bookkeeping (algorithmic work per stage, per call)
 # ---------------------------------------------------------------------------
-# sparse solver rounds run as whole-GPU kernels after the dense first one
-# (sparse_gpu_rounds in the library's kernels.cuh, b = 16)
-def wide_rounds(N: int, B: int, K: int, images: int) -> int:
-    base = 8 if N > 3072 else 5 if N > 1536 else 1
-    base += 5 if B > 38 else 4 if B > 19 else 2 if B > 9 else 0
-    return min(base, max(0, -(-(K - (images if images > 1 else 16)) // 16)))
-
-
-def stage_work(wl) -> dict:
-    """Algorithmic bytes / flops each stage must move or compute for one call."""
+def stage_work(wl, sparse: int) -> dict:
+    """Algorithmic bytes / flops each stage must move or compute for one call, `sparse` of
+    whose rounds after the dense first one run as whole-GPU kernels."""
     B, N, H, Hkv, d, D, K = wl.B, wl.N, wl.H, wl.Hkv, wl.d, wl.D, wl.K
     es = 2 if wl.dtype == "bf16" else 4
     Tm = sum(wl.T) / B
@@ -206,10 +199,10 @@ def stage_work(wl) -> dict:
     w["message"] = ("hbm", B * (H * Tm * N * 4 + 2 * (N + Tm) * Hkv * d * es + Tm * H * d * es))
     w["clients"] = ("hbm", B * (M * N * 4 + H * Tm * N * 4 + N * N * 4))
     # selection: one read of the M x N clients per round.  Stage "rounds_gpu"
-    # runs the dense first round and the next wide_rounds sparse rounds as
-    # whole-GPU kernels; stage "select" (the cluster kernel) runs the rest.
+    # runs the dense first round and the next `sparse` rounds as whole-GPU
+    # kernels; stage "select" (the cluster kernel) runs the rest.
     rounds = -(-K // 16)
-    wide = min(rounds, 1 + wide_rounds(N, B, K, wl.I))
+    wide = min(rounds, 1 + sparse)
     w["rounds_gpu"] = ("hbm", B * wide * (M * N * 4.0))
     w["select"] = ("hbm", B * max(1, rounds - wide) * (M * N * 4.0))
     w["transport"] = ("hbm", B * ((N + Tm) * D * es + (K + Tm) * D * es
@@ -339,6 +332,18 @@ def run_gmc(args):
         for k, v in gmc.profile_read().items():
             prof[k] = prof.get(k, 0.0) + v / nprof
     gmc.profile_enable(False)
+    # sparse rounds on the whole GPU (three launches each): what a call launches beyond one
+    # whose budget the dense first round fills
+    sparse = 0
+    if "rounds_gpu" in prof:
+        one = gmc.Compressor(wl.B, wl.gh, wl.gw, wl.T_max, wl.H, wl.Hkv, wl.d, wl.D,
+                             comp.params.batch_b, dt,
+                             text_lengths=wl.T if wl.ragged else None, device=dev)
+        n0 = gmc.launch_count()
+        one.run(inp["hidden"], inp["keys"], inp["queries"], inp["pos_ids"], inp["vo_probe"])
+        torch.cuda.synchronize(dev)
+        sparse = (launches // args.steps - (gmc.launch_count() - n0)) // 3
+        del one
 
     # ---- end to end through pinned host memory --------------------------------
     out_host = {"idx": torch.empty(comp.out_idx.shape, dtype=comp.out_idx.dtype).pin_memory(),
@@ -384,7 +389,7 @@ def run_gmc(args):
 
     # ---- roofline of the dominant stage ----------------------------------------
     pk = peaks()
-    work = stage_work(wl)
+    work = stage_work(wl, sparse)
     dom = max(prof, key=prof.get) if prof else None
 
     def roofline(stage):

@@ -678,7 +678,7 @@ static int compress_impl(const gmc_problem* prob, const gmc_params* params,
       g_launches += 1;
     }
   } else {
-    GMC_STAGE("rounds_gpu", 3 + 3 * sparse_gpu_rounds(N, dm.B, Ke, p.batch_b, dm.I),
+    GMC_STAGE("rounds_gpu", 3 + 3 * sparse_gpu_rounds(dm.B, N, dm.M, HV, T, LS, p, Ke, dm.I),
               launch_round0(r0, dm.B, N, Ke, dm.M, dm.toff, HV, T, LS, p, fx, nullptr, s.C,
                             s.scol, s.u0, s.order, s.status, tv, st, dm.I));
     GMC_STAGE("select", 1,
@@ -943,7 +943,7 @@ int gmc_select(const float* clients, int B, int M, int N, int K, const gmc_param
                         s.order, s.status, tv, st));
   GMC_TRY(launch_select(r0, B, N, K, M, nullptr, 0, 1, 0, p, 0, s.fexp, s.C, s.scol, s.u0,
                         s.order, s.support, s.slot, out_idx, s.status, tv, st));
-  g_launches += 7 + 3 * sparse_gpu_rounds(N, B, K, p.batch_b, 1);
+  g_launches += 7 + 3 * sparse_gpu_rounds(B, N, M, 0, 1, 0, p, K, 1);
   return GMC_OK;
 }
 

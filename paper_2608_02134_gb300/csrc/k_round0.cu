@@ -680,7 +680,7 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   if ((e = set_smem_limit((const void*)k_rg_rho<ROWS>, rsm)) != cudaSuccess) return e;
   const size_t gsm = sel::gain_sums_bytes(N) + (size_t)N;
   if ((e = set_smem_limit((const void*)k_rg_filter<ROWS>, gsm)) != cudaSuccess) return e;
-  const int rounds = sparse_gpu_rounds(N, B, K, p.batch_b, I);
+  const int rounds = sparse_gpu_rounds(B, N, M, H, T, L2, p, K, I);
   for (int rr = 1; rr <= rounds; ++rr) {
     long long* ucur = rr % 2 == 1 ? r0.u1 : r0.u2;
     long long* unext = rr % 2 == 1 ? r0.u2 : r0.u1;
@@ -706,7 +706,7 @@ cudaError_t launch_round0(R0State& r0, int B, int N, int K, int M, const int32_t
                           int32_t* order, uint32_t* status, const TraceView& tv,
                           cudaStream_t st, int I) {
   const int P = p.pool_mult * p.batch_b;
-  r0.ugain = sparse_gpu_rounds(N, B, K, p.batch_b, I) % 2 == 0 ? r0.u1 : r0.u2;
+  r0.ugain = sparse_gpu_rounds(B, N, M, H, T, L2, p, K, I) % 2 == 0 ? r0.u1 : r0.u2;
   cudaError_t e;
   const size_t smem =
       sizeof(long long) * (size_t)N + sizeof(int) * (sel::HBINS + N + 32 + 8 + sel::CBINS + P) +

@@ -55,6 +55,7 @@
 // the pool by a histogram, took 11.8 us at N = 1,296 and 20 us at N = 4,096,
 // where its lists did not fit.
 #include <cooperative_groups.h>
+#include <algorithm>
 
 #include "common.cuh"
 #include "kernels.cuh"
@@ -1455,6 +1456,34 @@ static int first_cluster_size(int B) {
   int CS = 1;
   while (CS * 2 <= SEL_MAX_CS && (long long)B * CS * 2 <= g_num_sms) CS *= 2;
   return CS;
+}
+
+// Until the survivor lists fit the cluster's shared memory a round costs 50 us and more
+// in a cluster (they stay in global memory), 21 to 40 us on the whole GPU; after that 8
+// to 11 us in a cluster.  How many rounds that takes follows from the load, the entries
+// of a CTA's dense rows over what its shared memory holds of them, and from the tokens a
+// round selects.  A grounded row counts a third in the load (attention is concentrated:
+// few entries survive a round), a spatial one five times (its distances fall off slowly);
+// gmc_select's rows have no kind.  Calls in us by sparse rounds on the GPU at b = 16:
+//   N = 1,296, T = 64, K = 453   1: 379, 2: 368, 3: 362, 6: 379   (the rule: 1)
+//   N = 1,296, T = 256, K = 77   1: 483, 2: 320, 3: 322, 6: 319   (2)
+//   N = 2,304, T = 32, H = 4     2: 563, 3: 426, 4: 427, 8: 438   (3)
+//   N = 3,025, T = 64            2: 599, 4: 489, 5: 493, 6: 501   (5)
+//   N = 4,096, T = 128           4: 915, 6: 817, 8: 745, 10: 767  (8)
+//   N = 6,400, T = 128           8: 1,606, 10: 1,525, 12: 1,439, 16: 1,469  (12)
+// Over 134 shapes (N 144 to 7,568, T 8 to 256, one to 64 images, b 8 to 32) the rule is
+// 1.4% above the best count in the mean, 8% at most; steps in N alone 6.2%, 58%.
+int sparse_gpu_rounds(int B, int N, int M, int H, int T, int L2, const gmc_params& p, int K,
+                      int images) {
+  if (num_sms() != cudaSuccess) cudaGetLastError();
+  const int CS = first_cluster_size(B), SL = ((N + CS - 1) / CS + 31) & ~31;
+  const int cap = sel_layout(N, p.pool_mult * p.batch_b, CS, SL, (M + CS - 1) / CS).cap;
+  const double ground = (double)H * T, rows = ground / 3 + (M - ground - L2) + 5.0 * L2;
+  const double load = rows * N / CS / (cap > 0 ? cap : 1);
+  const double rounds = std::max(1.0, (0.92 * sqrt(load) - 1.5) * sqrt(16.0 / p.batch_b));
+  const int left = K - (images > 1 ? images : p.batch_b);  // no more than the budget has left
+  const int most = left > 0 ? (left + p.batch_b - 1) / p.batch_b : 0;
+  return (int)std::min(rounds, (double)most);
 }
 
 // Bytes per CTA that bound the problems given to the cluster solver: what an

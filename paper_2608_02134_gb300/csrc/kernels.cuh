@@ -154,26 +154,17 @@ cudaError_t launch_gram(const Dims&, const void* hidden, Scratch&, cudaStream_t)
 cudaError_t launch_build_clients(const Dims&, const gmc_params&, int fx_exp, Scratch&,
                                  const ViewRows& views, const float* app,
                                  cudaStream_t, int part = 0);
-// State left by the first (dense) selection round, run over the whole GPU.
-// Sparse rounds of the solver run on the whole GPU, after the dense first one
-// and before the cluster kernel takes over: until the survivor lists fit the
-// cluster's shared memory, and no more than the budget has rounds left.  Larger
-// images keep more survivors, and a batch leaves fewer CTAs per image.  A round
-// costs about 21 us on the whole GPU and 9-18 us in a cluster that holds its
-// lists, but 50 us and more in one that does not (they stay in global memory).
-// Measured calls by sparse rounds on the GPU: N = 1,296: 0 525 us, 1 320, 2 327,
-// 4 328; N = 2,592: 2 937, 3 956, 4 716, 5 686, 8 709; N = 4,096: 6 924, 8 889, 10
-// 907; 32 images of N = 1,296: 1 4.31 ms, 2 4.15, 4 3.99, 6 3.98.
-inline int sparse_gpu_rounds(int N, int B, int K, int batch_b, int images) {
-  const int base = (N > 3072 ? 8 : (N > 1536 ? 5 : 1)) + (B > 38 ? 5 : (B > 19 ? 4 : (B > 9 ? 2 : 0)));
-  const int left = K - (images > 1 ? images : batch_b);
-  const int most = left > 0 ? (left + batch_b - 1) / batch_b : 0;
-  return base < most ? base : most;
-}
+// Sparse rounds of the solver that run on the whole GPU, after the dense first one and
+// before the cluster kernel takes over (k_select.cu), for images of M client rows at the
+// widest: H * T grounded rows, L2 spatial ones, the rest appearance rows (H = L2 = 0:
+// a caller's clients).
+int sparse_gpu_rounds(int B, int N, int M, int H, int T, int L2, const gmc_params&, int K,
+                      int images);
 
 // per-image words of R0State::info
 constexpr int INFO_W = 8;
 
+// State left by the rounds run over the whole GPU.
 struct R0State {
   int32_t* pool;   // [B][P]  pool of the current whole-GPU round (-1 padded)
   int32_t* info;   // [B][INFO_W]  pool size of the current round, tokens selected so far,
@@ -201,10 +192,9 @@ cudaError_t launch_select(const R0State&, int B, int N, int K, int M, const int3
 // gmc_select: copies the caller's clients into s.C, then the per-image total,
 // fixed-point exponent (s.fexp) and column sums (s.u0)
 cudaError_t launch_select_prep(const float* clients, int B, int M, int N, Scratch& s, cudaStream_t);
-// Whether the cluster solver's per-CTA state (a copy of every token's gain,
-// bucket and pool slot, and its share of the client rows) fits one CTA's
-// shared memory for this problem on this device; where it does not, every
-// round runs on the whole GPU (launch_wide_select).
+// Whether the cluster solver takes this problem on this device (a bound on the tokens,
+// the pool and a CTA's share of the client rows, k_select.cu); where it does not,
+// every round runs on the whole GPU (launch_wide_select).
 bool select_fits(int B, int N, int M, int P);
 // Batched certificate c_B of the trace from the recorded rounds (one block per image).
 cudaError_t launch_certificate(int B, int N, int K, const TraceView&, cudaStream_t);

@@ -105,6 +105,21 @@ def test_cluster_solver_sizes(kind, B, M, N, K, b, mult):
     _check_select(_clients(kind, B, M, N, 5 + N), K, batch_b=b, pool_mult=mult)
 
 
+# the hand-over to the cluster solver follows what its shared memory holds of the lists:
+# at one token count more client rows take more rounds on the whole GPU (launches of a
+# call: copy and sum, exponent, column sums, three of the dense round, three a sparse
+# round, the cluster's), and never more than the budget has left
+@pytest.mark.parametrize("B,M,N,K,sparse", [
+    (1, 2000, 1296, 200, 1), (1, 8720, 1296, 200, 4), (1, 8720, 1296, 33, 2), (1, 8720, 1296, 16, 0),
+    (4, 600, 900, 60, 1)])
+def test_sparse_rounds_follow_the_client_rows(B, M, N, K, sparse):
+    from paper_2608_02134_gb300 import gmc
+    from tests.test_gpu_stages import _check_select
+    n0 = gmc.launch_count()
+    _check_select(_clients("plain", B, M, N, 11 + M), K)
+    assert gmc.launch_count() - n0 == 7 + 3 * sparse
+
+
 # the wide solver: one, four and eight pool slots a thread, rows on 16 bytes and not,
 # the most tokens, all gains equal (the digits of the token decide) or nearly so, a
 # batch that is the whole pool, more rows than blocks and fewer
