@@ -690,7 +690,14 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
   dim3 grid(RQ / BM, dm.Hkv, dm.B * sp.n);
   const size_t fsmem = 1024 + fused_region_bytes(nkb) + sizeof(FusedCtl) +
                        sizeof(float) * (size_t)(dm.H / dm.Hkv) * (sp.kt_per * BM + 1);
-  if (sp.kt_per <= FUSED_MAX_TILES && sp.n <= FUSED_MAX_CLUSTER && fsmem <= 227 * 1024) {
+  bool fused = sp.kt_per <= FUSED_MAX_TILES && sp.n <= FUSED_MAX_CLUSTER && fsmem <= 227 * 1024;
+  if (fused && sp.n > FUSED_PORTABLE &&
+      cudaFuncSetAttribute((const void*)k_message_fused,
+                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
+    cudaGetLastError();  // no cluster of that size here: the two launches below
+    fused = false;
+  }
+  if (fused) {
     uint32_t cols = 32;
     while (cols < (uint32_t)(sp.kt_per * BM)) cols *= 2;
     if ((e = set_smem_limit((const void*)k_message_fused, fsmem)) != cudaSuccess) return e;
@@ -706,10 +713,6 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
     attr[0].val.clusterDim.z = sp.n;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    if (sp.n > FUSED_PORTABLE &&
-        (e = cudaFuncSetAttribute((const void*)k_message_fused,
-                                  cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
-      return e;
     int ncl = 0;
     if (cudaOccupancyMaxActiveClusters(&ncl, (void*)k_message_fused, &cfg) == cudaSuccess && ncl > 0) {
       attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // see grid_dep_wait
