@@ -24,6 +24,8 @@
 // softmax arithmetic.  Every wait is clock-bounded.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.cuh"
 #include "tc.cuh"
@@ -102,30 +104,52 @@ __host__ __device__ inline size_t fused_region_bytes(int nkb) {
 struct MsgSplit {
   int kt_per;  // key tiles per split at the widest image (an image's own: split_tiles)
   int n;       // splits
+  bool fused;  // the splits of a query tile as one cluster, one launch
 };
 
-// Key splits of a query tile.  Few query tiles: enough splits for one wave of
-// CTAs.  Many: one split would do, but the fused kernel writes A from logits
-// it keeps in TMEM, in whole 128-byte lines, where the two launches compute every
-// logit twice and store row by row; so the splits are at least as many as
-// hold an image's keys in TMEM (FUSED_MAX_TILES each) while a cluster can span
-// them, and at most a portable cluster where that is enough.  Measured, two
-// launches -> fused: 32 ragged images of N = 1,296 (13 key tiles, T <= 256)
-// 695 us -> 492, N = 4,096 at T = 128 (33 tiles, 9 splits) 69 us ->
-// 47.
+// Clusters of n CTAs, one CTA an SM, that the GPU holds at once (what the occupancy query
+// answers on a GB300: a cluster stays inside one of its groups of 16 to 20 SMs).  In a
+// long queue clusters of seven use the SMs of a group better than its two at a time: 18.
+constexpr int CLUSTERS[FUSED_MAX_CLUSTER + 1] = {0,  152, 76, 46, 36, 28, 23, 15, 15,
+                                                 15, 13,  8,  8,  7,  7,  7,  7};
+constexpr int QUEUED_SEVENS = 18;
+
+// Key splits of a query tile, and in one launch or two.
+//
+// Two launches compute every logit twice; any number of splits will do, so few query
+// tiles get enough of them for one wave of CTAs.  The fused kernel writes A from logits
+// it keeps in TMEM: a split takes at most FUSED_MAX_TILES key tiles, and the splits of a
+// query tile are one cluster (a portable one where that is enough), of which the GPU
+// holds few at once when they are large.  Times in us, by the key tiles kt of a split,
+// fitted to 172 shapes (N 576 to 7,056, T 8 to 256, 4 and 32 KV groups, one to 32 images):
+//   fused: 6 + 5.8 kt, and 3 + 3.8 kt more for each further wave of clusters;
+//   two launches: 13 + 6.2 kt for each wave of CTAs.
+// The faster one by these is 0.1% above the faster one measured in the mean, 4% at most;
+// fused wherever it fits: 3.8% and 36%.  Fused / two launches: N = 576, T = 64: 12.5 /
+// 19.4; N = 4,096, T = 256: 84 / 114, T = 128: 49 / 56, T = 64: 46 / 38, T = 8: 30 / 24;
+// N = 6,400, T = 64: 66 / 50; 16 images of N = 1,296, T = 256: 441 / 461.
 MsgSplit msg_split(int B, int Hkv, int RQ, int N, int T) {
-  const int nkt = (N + T + BM - 1) / BM;
-  const int base = (RQ / BM) * Hkv * B;
-  int target = SPLIT_TARGET_CTAS / base > 1 ? SPLIT_TARGET_CTAS / base : 1;
-  const int need = (nkt + FUSED_MAX_TILES - 1) / FUSED_MAX_TILES;
-  if (need <= FUSED_MAX_CLUSTER) {
-    if (target > FUSED_PORTABLE) target = FUSED_PORTABLE;
-    if (target < need) target = need;
-  }
-  MsgSplit sp;
-  sp.kt_per = (nkt + target - 1) / target;
-  sp.n = (nkt + sp.kt_per - 1) / sp.kt_per;
-  return sp;
+  const int nkt = ceil_div(N + T, BM);
+  const long long base = (long long)(RQ / BM) * Hkv * B;  // query tiles
+  const int target = SPLIT_TARGET_CTAS / base > 1 ? (int)(SPLIT_TARGET_CTAS / base) : 1;
+  auto split = [&](int splits) {
+    MsgSplit sp;
+    sp.kt_per = ceil_div(nkt, splits);
+    sp.n = ceil_div(nkt, sp.kt_per);
+    sp.fused = false;
+    return sp;
+  };
+  const MsgSplit two = split(target);
+  const int need = ceil_div(nkt, FUSED_MAX_TILES);
+  if (need > FUSED_MAX_CLUSTER) return two;
+  MsgSplit one = split(std::max(need, std::min(target, FUSED_PORTABLE)));
+  one.fused = true;
+  int held = CLUSTERS[one.n];
+  if (one.n == 7 && base > 2 * held) held = QUEUED_SEVENS;
+  const long long w1 = (base + held - 1) / held;
+  const long long w2 = (base * two.n + SPLIT_TARGET_CTAS - 1) / SPLIT_TARGET_CTAS;
+  const double t1 = 6 + 5.8 * one.kt_per + (w1 - 1) * (3 + 3.8 * one.kt_per);
+  return t1 <= w2 * (13 + 6.2 * two.kt_per) ? one : two;
 }
 
 // Key tiles per split of an image with nkt tiles: spread evenly, so that an
@@ -297,23 +321,22 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (mode == 0) {  // running max / sum over the visible keys
         float mt = -INFINITY;
 #pragma unroll
-        for (int q = 0; q < 32; ++q) {
-          v[q] *= scale;
+        for (int q = 0; q < 32; ++q)
           if (k0 + q < kvis) mt = fmaxf(mt, v[q]);
-        }
+        mt *= scale;
         if (mt > -INFINITY) {
           const float mn = fmaxf(m, mt);
           float acc = l * expf(m - mn);
 #pragma unroll
-          for (int q = 0; q < 32; ++q)
-            if (k0 + q < kvis) acc += expf(v[q] - mn);
+          for (int q = 0; q < 32; ++q)  // the logit's product is not rounded by itself
+            if (k0 + q < kvis) acc += expf(fmaf(v[q], scale, -mn));
           l = acc;
           m = mn;
         }
       } else if (k0 < N) {  // normalised visual columns; uniform over the warp
         const int nv = min(32, N - k0);
 #pragma unroll
-        for (int q = 0; q < 32; ++q) v[q] = expf(v[q] * scale - M) * invL;
+        for (int q = 0; q < 32; ++q) v[q] = expf(fmaf(v[q], scale, -M)) * invL;
         if (nv == 32 && (N & 3) == 0) {
 #pragma unroll
           for (int q = 0; q < 32; q += 4) {
@@ -690,7 +713,7 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
   dim3 grid(RQ / BM, dm.Hkv, dm.B * sp.n);
   const size_t fsmem = 1024 + fused_region_bytes(nkb) + sizeof(FusedCtl) +
                        sizeof(float) * (size_t)(dm.H / dm.Hkv) * (sp.kt_per * BM + 1);
-  bool fused = sp.kt_per <= FUSED_MAX_TILES && sp.n <= FUSED_MAX_CLUSTER && fsmem <= 227 * 1024;
+  bool fused = sp.fused && fsmem <= 227 * 1024;
   if (fused && sp.n > FUSED_PORTABLE &&
       cudaFuncSetAttribute((const void*)k_message_fused,
                            cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {

@@ -224,12 +224,27 @@ def _check_grounded(wl):
 # exceed the largest one (two launches); query tiles that are ragged; keys that end
 # inside a tile, rows of A on 16 bytes and not
 @pytest.mark.parametrize("gh,gw,T,H,Hkv,B", [
-    (16, 8, [40], 4, 2, 1), (23, 41, [70, 3, 33], 6, 2, 3), (36, 37, [21], 28, 28, 12),
+    (16, 8, [40], 4, 2, 1), (48, 54, [8], 4, 4, 1), (23, 41, [70, 3, 33], 6, 2, 3), (36, 37, [21], 28, 28, 12),
     (66, 64, [9], 4, 1, 1), (128, 64, [5], 2, 1, 1)])
 def test_message_slice_splits(gh, gw, T, H, Hkv, B):
     from paper_2608_02134_gb300 import workloads
     wl = workloads.make("qwen", B=B, T=T * (B // len(T)), gh=gh, gw=gw, D=64, d=64, H=H, Hkv=Hkv, K=9)
     _check_grounded(wl)
+
+
+# few query tiles of a large image run as two launches over many splits, more of them as
+# one launch of clusters (a call of gmc_clients counts one launch less): both, at one
+# grid each, against the oracle's rows
+@pytest.mark.parametrize("gh,gw,few,many", [(48, 54, 8, 192), (64, 64, 64, 128)])
+def test_message_slice_launches(gh, gw, few, many):
+    from paper_2608_02134_gb300 import gmc, workloads
+    count = []
+    for T in (few, many):
+        wl = workloads.make("qwen", B=1, T=T, gh=gh, gw=gw, D=64, d=64, H=28, Hkv=4, K=9)
+        n0 = gmc.launch_count()
+        _check_grounded(wl)
+        count.append(gmc.launch_count() - n0)
+    assert count[0] == count[1] + 1
 
 
 # probe: one head a KV group, more heads than warps, value rows of an odd and an even
