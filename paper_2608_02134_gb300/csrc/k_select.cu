@@ -277,7 +277,9 @@ __device__ __forceinline__ float div_by(float x, float d, float r) {
 
 // Lists the tokens of gain >= lo >= 1 (key in ck, token in cj, any order; at most
 // LCAP are kept) and counts them in *cnt (zero on entry).  A selected token's
-// entries are all dead, so its gain is exactly zero and it is never listed.
+// entries are all dead, so its gain is exactly zero and it is never listed.  Gains are
+// signed, as in the rounds before: sums of invalid clients (negative or infinite ones,
+// reported in the status) may have wrapped, and are then no candidates.
 // addr(j): where token j's gain is; ga: that of the thread's first GA tokens.
 // Every thread calls it; a barrier follows at the caller.
 constexpr int GA = 4;
@@ -303,8 +305,9 @@ __device__ __forceinline__ void list_candidates(Addr addr, const uint32_t* ga, c
     int tot = 0;
 #pragma unroll
     for (int t = 0; t < U; ++t) {
-      bal[t] = __ballot_sync(FULL, v[t] >= lo);
-      mine |= v[t] >= lo ? 1u << t : 0u;
+      const bool at = (long long)v[t] >= (long long)lo;
+      bal[t] = __ballot_sync(FULL, at);
+      mine |= at ? 1u << t : 0u;
       tot += __popc(bal[t]);
     }
     if (!tot) continue;  // warp-uniform
@@ -1087,7 +1090,7 @@ __global__ void __launch_bounds__(SEL_THREADS, 1) k_select(SelArgs a) {
         for (int c = 0; c < CS; ++c) v += s.spart[c * SP + k];
       }
       s.s_acc[k] = (long long)v;
-      s.sk[k] = v ? gain_key(v) : 0u;  // past Pt: zero
+      s.sk[k] = (long long)v > 0 ? gain_key(v) : 0u;  // past Pt: zero
     }
     __syncthreads();
     // 8 lanes rank each pool token by its score's key, four keys a load; tokens whose

@@ -40,6 +40,20 @@ def test_nonfinite_hidden_state_is_reported_with_check_mode():
     assert g2.status == 0
 
 
+def test_clients_below_zero_are_reported_and_leave_a_support():
+    """Negative clients are outside gmc_select's contract: the total is no scale for the
+    fixed-point gains and their sums wrap.  No token has a positive gain then, so the budget
+    is filled in index order; the status says why."""
+    from tests.test_gpu_stages import _select_gpu
+    N, K = 1100, 40
+    C = np.full((1, 60, N), 1e-13, np.float32)
+    C[0, 0], C[0, 1] = 100.0, -1000.0
+    idx, _, st = _select_gpu(C, K)
+    from paper_2608_02134_gb300 import gmc
+    assert st == gmc.STATUS_NONFINITE
+    assert idx[0].tolist() == list(range(K))
+
+
 def test_check_mode_off_leaves_clean_status():
     from paper_2608_02134_gb300 import gmc
     from tests import gpu_harness as GH
