@@ -17,8 +17,8 @@ namespace gmc {
 cudaError_t set_smem_limit(const void* func, size_t bytes) {
   static std::mutex mu;
   static std::unordered_map<const void*, size_t> done;
-  // the 48 KB default covers a kernel's static arrays too (20 KB at most here)
-  if (bytes <= 28 * 1024) return cudaSuccess;
+  // the 48 KB default covers a kernel's static arrays too (33 KB at most: k_transport<float>)
+  if (bytes <= 14 * 1024) return cudaSuccess;
   std::lock_guard<std::mutex> lk(mu);
   auto it = done.find(func);
   if (it != done.end() && it->second >= bytes) return cudaSuccess;
