@@ -358,9 +358,13 @@ static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_
   const int per_image =
       g.sym ? gemm_sym_ctas(g.M, 1) : ceil_div(g.Nn, BN) * ceil_div(g.M, GM);
   static int sms = 0;
-  if (sms == 0 && cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, 0) != cudaSuccess) {
-    cudaGetLastError();
-    sms = 152;
+  if (sms == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+      cudaGetLastError();
+      sms = 152;
+    }
   }
   const long long tiles = (long long)per_image * g.B;
   if (tiles > 0x7fffffffLL - sms) return cudaErrorInvalidValue;
