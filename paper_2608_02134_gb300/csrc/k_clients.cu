@@ -312,7 +312,7 @@ cudaError_t launch_build_clients(const Dims& dm, const gmc_params& p, int fx_exp
 // in one pass, then the fixed-point exponent and column sums.
 // ---------------------------------------------------------------------------
 // Copies image b's clients into the solver's buffer, sums them in fp64 and
-// clears the column sums.  Bound by memory (one read, one write): SEL_BLOCKS
+// clears the column sums.  Bound by memory (one read, one write): nblk (512)
 // blocks per image, each over a contiguous share, four 16-byte loads per thread in
 // flight where both sides start on 16 bytes.  It replaced a device copy, a sum
 // over 64 blocks with one load per thread in flight (58 us) and a one-thread

@@ -609,8 +609,7 @@ int head_block(int H) {
 // Tokens per head-statistics block.  32 (whole lines) once those blocks fill
 // the SMs twice over; below that smaller blocks keep more SMs busy: at one
 // image of N = 1,296 the 162 blocks of 8 tokens, at N = 4,096 the 256 of 16.
-int head_tokens(int B, int N, int H) {
-  (void)H;
+int head_tokens(int B, int N) {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;

@@ -30,7 +30,7 @@ namespace gmc {
 
 namespace {
 // Threads of a sparse round's pool block: a turn takes four tokens a thread.  1,024
-// from N = 2,048 on (a second turn costs more than the wider barriers).
+// above N = 2,048 (a second turn costs more than the wider barriers).
 constexpr int POOL_THREADS = 1024;
 int pool_threads(int N) { return N > 2048 ? POOL_THREADS : POOL_THREADS / 2; }
 
@@ -517,7 +517,7 @@ __global__ void __launch_bounds__(32 * ROWS, ROWS == 16 ? 3 : 4) k_rg_filter(
   __shared__ int batch[GMC_MAX_POOL];
   extern __shared__ __align__(16) char sm_rgf[];  // the falls of the gains, then the batch flags [N]
   const sel::GainSums<true> sums{reinterpret_cast<uint32_t*>(sm_rgf), N};
-  unsigned char* inb = reinterpret_cast<unsigned char*>(sm_rgf) + sel::gain_sums_bytes(N);
+  unsigned char* inb = reinterpret_cast<unsigned char*>(sm_rgf) + sel::gain_sums_bytes<true>(N);
   const int b = blockIdx.y;
   const int Pt = info[b * INFO_W];
   if (Pt == 0) return;
@@ -666,7 +666,7 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   launch_k(k_r0_rho<ROWS>, grid, 32 * ROWS, 0, st, 1, C, B, N, M, H, L2, toff, T, uniform, r0.pool,
            r0.info, P, p.resp_temp, p.resp_eps, fx_exp, fexp, I, rpw, r0.s0);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  const size_t fsm = sizeof(float) * ROWS * sel::ROW_STEP + sel::gain_sums_bytes(N);
+  const size_t fsm = sizeof(float) * ROWS * sel::ROW_STEP + sel::gain_sums_bytes<true>(N);
   if ((e = set_smem_limit((const void*)k_r0_filter<ROWS>, fsm)) != cudaSuccess) return e;
   launch_k(k_r0_filter<ROWS>, grid, 32 * ROWS, fsm, st, 1, C, scol, B, N, K, M, H, L2, toff,
            T, uniform, r0.pool, r0.info, r0.s0, P, p.batch_b, fx_exp, fexp, r0.u1, r0.bcov, r0.cnt,
@@ -678,7 +678,7 @@ static cudaError_t launch_rounds_rows(const R0State& r0, int B, int N, int K, in
   if ((e = set_smem_limit((const void*)k_rg_pool, psm)) != cudaSuccess) return e;
   const size_t rsm = sizeof(short) * (size_t)N;
   if ((e = set_smem_limit((const void*)k_rg_rho<ROWS>, rsm)) != cudaSuccess) return e;
-  const size_t gsm = sel::gain_sums_bytes(N) + (size_t)N;
+  const size_t gsm = sel::gain_sums_bytes<true>(N) + (size_t)N;
   if ((e = set_smem_limit((const void*)k_rg_filter<ROWS>, gsm)) != cudaSuccess) return e;
   const int rounds = sparse_gpu_rounds(B, N, M, H, T, L2, p, K, I);
   for (int rr = 1; rr <= rounds; ++rr) {
@@ -718,7 +718,8 @@ cudaError_t launch_round0(R0State& r0, int B, int N, int K, int M, const int32_t
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   // one image: 16 warps per block (fewer, larger blocks finish the rounds sooner); a
   // batch: 8
-  return (B == 1 ? launch_rounds_rows<16> : launch_rounds_rows<8>)(r0, B, N, K, M, toff, H, T, L2, p, fx_exp, fexp, C, scol, order, tv, st, I, smem);
+  return (B == 1 ? launch_rounds_rows<16> : launch_rounds_rows<8>)(
+      r0, B, N, K, M, toff, H, T, L2, p, fx_exp, fexp, C, scol, order, tv, st, I, smem);
 }
 
 }  // namespace gmc

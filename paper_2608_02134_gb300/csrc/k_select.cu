@@ -150,7 +150,8 @@ enum { FB_LO = 4 };  // 64-bit word of fb: the next pool's threshold
 
 // Byte offsets of the arrays in a CTA's shared memory.
 struct SelOff {
-  uint32_t gacc, sown, spart, s_acc, fb, ck, cj, selw, wpre, pool, wsum, scal, hist, bcov, rmaxb, zlo, zhi, bnb, rptr, chg, uloc, sk, cs, rval, rtok, crow, cpos, sw, inb, poolslot;
+  uint32_t gacc, sown, spart, s_acc, fb, ck, cj, selw, wpre, pool, wsum, scal, hist, bcov, rmaxb,
+      zlo, zhi, bnb, rptr, chg, uloc, sk, cs, rval, rtok, crow, cpos, sw, inb, poolslot;
 };
 struct Layout {
   SelOff o;

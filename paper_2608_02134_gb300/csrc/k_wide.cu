@@ -700,7 +700,7 @@ cudaError_t launch_wide_select(const WideState& w, const WideGeom& g, const gmc_
   const int fblocks = std::min(per_image, (int)ceil_div(g.Mstride, 4));
   const int frows = (int)ceil_div(g.Mstride, fblocks);
   const int fwarps = (int)ceil_div(frows, ceil_div(frows, FROWS));
-  const size_t fsm = sizeof(unsigned long long) * (size_t)N;
+  const size_t fsm = sel::gain_sums_bytes<false>(N);
   const size_t fsm_dense = fsm + sizeof(float) * sel::ROW_STEP * (size_t)fwarps;
   // the window pool's extra shared memory: the staged gains and its scratch
   const size_t wsm = sizeof(long long) * ((size_t)N + sel::WCAP) + sizeof(int) * sel::WCAP +

@@ -131,7 +131,7 @@ struct Scratch {
 };
 
 constexpr int ROWS_PER_BLOCK = 8;  // rownorm / probe / client builder blocks
-int head_tokens(int B, int N, int H);  // tokens per head-statistics block: 8, 16 or 32
+int head_tokens(int B, int N);  // tokens per head-statistics block: 8, 16 or 32
 constexpr int ASSIGN_WARPS = 16;   // warps per assignment block (32 tokens, one per lane)
 int assign_blocks(int N);          // assignment blocks per image
 constexpr int PROBE_TOK = 32;       // tokens per probe block

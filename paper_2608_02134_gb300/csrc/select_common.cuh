@@ -37,11 +37,12 @@ __device__ __forceinline__ unsigned long long limb_value(const uint32_t* w, int 
          ((unsigned long long)w[2 * stride] << (2 * LIMB));
 }
 
-// Sums of a block's changes of the gains, one per token: limbs, or 64-bit words
-// where the limbs of N tokens would not leave room for two blocks on an SM.
-constexpr int LIMB_MAX_N = 8192;
+// Sums of a block's changes of the gains, one per token: limbs in the rounds of the
+// standard path (N <= GMC_MAX_N: 96 KB at most), 64-bit words in the wide solver, whose
+// N tokens would take 192 KB of limbs.
+template <bool LIMBS>
 __host__ __device__ inline size_t gain_sums_bytes(int N) {
-  return (N <= LIMB_MAX_N ? 12 : 8) * (size_t)N;
+  return (LIMBS ? 3 * sizeof(uint32_t) : sizeof(unsigned long long)) * (size_t)N;
 }
 template <bool LIMBS>
 struct GainSums {
@@ -333,7 +334,7 @@ __device__ inline int select_pool(const long long* u, const unsigned char* sel, 
     cu += __popc(__ballot_sync(FULL, kb > bstar));
     ca += __popc(__ballot_sync(FULL, kb >= 0 && kb == bstar));
   }
-  if (lane == 0) w.wsum[wid] = (cu << 16) | ca;  // cu, ca < 2^15: N <= 8192
+  if (lane == 0) w.wsum[wid] = (cu << 16) | ca;  // cu, ca <= N <= 2^14
   __syncthreads();
   // every warp has read the histograms: clear the bins this thread counted
   for (int c = 0; c < nc; ++c) {
