@@ -79,7 +79,10 @@ constexpr int ENTRY_BYTES = 10;  // flat mode: value 4, token 2, row 2, place 2
 // Images of up to this many tokens sum a CTA's gain changes in its own shared
 // memory and send one remote addition per token, whole warps to one owner;
 // scattered remote additions cost about 4 cycles each.  Larger images send them
-// one by one: their sums would take the room of a fifth of the entries.
+// one by one: their sums would take the room of a fifth of the entries, and the
+// hand-over comes later.  Whole calls with the sums against without: N = 1,296
+// 280.7 us / 290.5, 2,025 432 / 430, 3,025 556 / 566, 3,844 (T = 128) 755 / 834,
+// 4,096 (T = 128) 744 / 719; above the line, 5,040 978 / 968, 6,400 1,619 / 1,423.
 constexpr int AGG_MAX_N = 4096;
 __host__ __device__ inline bool aggregates(int N, int R) {
   return N <= AGG_MAX_N && R <= sel::LIMB_ADDS;  // a row adds to a token at most once

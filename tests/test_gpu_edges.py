@@ -90,8 +90,9 @@ def _clients(kind, B, M, N, seed):
 
 
 # the cluster solver: more equal or nearly equal gains than a round lists exactly
-# (the radix search and its ties), lists in global memory, token counts that are no
-# multiple of 32, the widest pool, pools that are no power of two, one to sixteen
+# (the radix search and its ties), lists that are in global memory for its first rounds
+# (23,700 and 21,300 entries a CTA where 19,200 fit) above and below N = 4,096, token
+# counts that are no multiple of 32, the widest pool, pools that are no power of two, one to sixteen
 # CTAs an image, a budget of one round, rounds left over by a fill
 @pytest.mark.parametrize("kind,B,M,N,K,b,mult", [
     ("equal", 1, 1200, 1200, 100, 16, 4), ("close", 1, 1300, 1300, 90, 16, 4),
@@ -99,7 +100,8 @@ def _clients(kind, B, M, N, seed):
     ("plain", 1, 90, 1025, 300, 32, 4), ("plain", 2, 700, 500, 100, 3, 5),
     ("plain", 20, 300, 300, 60, 16, 4), ("plain", 90, 120, 200, 40, 16, 4),
     ("plain", 1, 400, 640, 16, 16, 4), ("plain", 1, 60, 7000, 200, 16, 4),
-    ("equal", 1, 40, 700, 64, 16, 4)])
+    ("equal", 1, 40, 700, 64, 16, 4), ("dense", 1, 3000, 4500, 60, 2, 4),
+    ("dense", 1, 2500, 4501, 40, 2, 4), ("dense", 1, 3000, 1100, 40, 1, 4)])
 def test_cluster_solver_sizes(kind, B, M, N, K, b, mult):
     from tests.test_gpu_stages import _check_select
     _check_select(_clients(kind, B, M, N, 5 + N), K, batch_b=b, pool_mult=mult)
