@@ -52,20 +52,22 @@ template <> struct Row8<float> {
   }
 };
 
+// Thread t's 8 elements into a slice of `cnt` threads' elements at p: its 16-byte units
+// are t and cnt + t, so that a warp's accesses are whole lines in fp32 too.
 template <typename Tin> struct Vec8;
 template <> struct Vec8<__nv_bfloat16> {
-  static __device__ __forceinline__ void store(__nv_bfloat16* p, const float* v) {
+  static __device__ __forceinline__ void store(__nv_bfloat16* p, int t, int, const float* v) {
     uint4 raw;
     __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&raw);
 #pragma unroll
     for (int q = 0; q < 4; ++q) h[q] = __floats2bfloat162_rn(v[2 * q], v[2 * q + 1]);
-    *reinterpret_cast<uint4*>(p) = raw;
+    reinterpret_cast<uint4*>(p)[t] = raw;
   }
 };
 template <> struct Vec8<float> {
-  static __device__ __forceinline__ void store(float* p, const float* v) {
-    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
-    *reinterpret_cast<float4*>(p + 4) = make_float4(v[4], v[5], v[6], v[7]);
+  static __device__ __forceinline__ void store(float* p, int t, int cnt, const float* v) {
+    reinterpret_cast<float4*>(p)[t] = make_float4(v[0], v[1], v[2], v[3]);
+    reinterpret_cast<float4*>(p)[cnt + t] = make_float4(v[4], v[5], v[6], v[7]);
   }
 };
 
@@ -100,7 +102,10 @@ inline int transport_split(int D) {
 // nothing.  Against rows in registers, a block scan of the membership and text
 // rows copied beside the carriers: 4 x (N = 2,295, K = 459, D = 3,584) from a
 // caller's assignment 95.0 -> 63.2 us a call, N = 1,296, K = 257 13.3 -> 10.3 us,
-// 32 such images 213 -> 202 us.
+// 32 such images 213 -> 202 us.  In fp32 a thread's two units lie a slice apart: side by
+// side, each copy of a warp touched half of every 32-byte sector and the sectors were
+// fetched twice (calls of N = 1,296, K = 257 23.8 us, now 20.8; 4,096, 400 48.3, now
+// 40.1; 6,400, 640 69.9, now 58.2).
 template <typename Tin, bool COOP>
 __global__ void __launch_bounds__(TR_THREADS) k_transport(
     const Tin* __restrict__ hidden, const Tin* __restrict__ keys, const int32_t* __restrict__ pos,
@@ -205,10 +210,12 @@ __global__ void __launch_bounds__(TR_THREADS) k_transport(
     __syncthreads();
     load_words();
   }
-  // this thread's chunk of the CTA's slice of D
-  const int nch = D / TR_VEC, cper = ceil_div(nch, S), ch = part * cper + tid;
-  const bool active = tid < cper && ch < nch;
-  const Tin* hb = hidden + sq.hidden_row(0, D) + (active ? ch * TR_VEC : 0);
+  // the CTA's slice of D: cnt threads take TR_VEC elements each (units tid and, in fp32,
+  // cnt + tid)
+  const int nch = D / TR_VEC, cper = ceil_div(nch, S), c0 = part * cper;
+  const int cnt = max(0, min(cper, nch - c0));
+  const bool active = tid < cnt;
+  const Tin* hb = hidden + sq.hidden_row(0, D) + c0 * TR_VEC;
   const float* mb = mass + (size_t)b * N;
   float acc[TR_VEC];
 #pragma unroll
@@ -257,9 +264,9 @@ __global__ void __launch_bounds__(TR_THREADS) k_transport(
 #pragma unroll
       for (int u = 0; u < TR_GRP; ++u)
         if (q0 + u < n && active) {
-          const uint4* row = reinterpret_cast<const uint4*>(hb + (size_t)lst[q0 + u] * D);
+          const uint4* row = reinterpret_cast<const uint4*>(hb + (size_t)lst[q0 + u] * D) + tid;
 #pragma unroll
-          for (int x = 0; x < U; ++x) cp_async16(&ring[(q0 + u) % TR_RING][x][tid], row + x);
+          for (int x = 0; x < U; ++x) cp_async16(&ring[(q0 + u) % TR_RING][x][tid], row + x * cnt);
         }
       cp_async_commit();
     };
@@ -319,7 +326,7 @@ __global__ void __launch_bounds__(TR_THREADS) k_transport(
       v[t] = acc[t] * scale;
       if (check && !isfinite(v[t])) set_status(status, GMC_STATUS_NONFINITE);
     }
-    Vec8<Tin>::store(out_hidden + sq.out_hidden_row(r, D) + ch * TR_VEC, v);
+    Vec8<Tin>::store(out_hidden + sq.out_hidden_row(r, D) + c0 * TR_VEC, tid, cnt, v);
   }
   if (t0 < nkv) {
     kd[t0] = kk;
