@@ -860,7 +860,7 @@ static size_t carve_select(int B, int M, int N, int K, Scratch* s, char* base,
                            R0State* r0s = nullptr, int wide_pool = 0, WideState* ws = nullptr) {
   Carver c{base};
   Scratch t{};
-  t.nSel = 512;  // blocks of the copy and total pass per image (about three per SM)
+  t.nSel = 304;  // most blocks of the copy and total pass per image (two per SM)
   t.status = c.take<uint32_t>(4);
   t.C = c.take<float>((size_t)B * M * N);
   t.scol = c.take<uint16_t>((size_t)B * M * N);

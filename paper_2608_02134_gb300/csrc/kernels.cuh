@@ -111,7 +111,7 @@ struct Scratch {
   int32_t* pi;       // [B][N]
   uint32_t* mbits;   // [B][K][ceil(N/32)] members of each carrier slot, bit i = token i
   float* mass;       // [B][N]
-  double* selpart;   // [B][nSel]      select-path total mass partials
+  double* selpart;   // [B][<= nSel]   select-path total mass partials
   int32_t* fexp;     // [B]            select-path fixed-point exponents
   __nv_bfloat16* Qp; // [B][Hkv][RQ][d] packed text queries of each KV group (tcgen05 path)
   int nP, nHG, nA, nSel, nE, nRS;
