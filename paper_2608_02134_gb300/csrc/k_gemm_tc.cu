@@ -18,7 +18,7 @@
 // Eq. (cond-aux-clients), (cond-assignment) for the cosines.)
 //
 // Persistent: one CTA per SM takes every gridDim.x-th 128 x BN output tile (BN = 128
-// or 256).  Warp 0 / lane 0 streams 64-wide K slices of the A and B row blocks with
+// or 256, launch_gemm_tc).  Warp 0 / lane 0 streams 64-wide K slices of the A and B row blocks with
 // TMA (128-byte swizzle) through an mbarrier ring of four stages; warp 1 / lane 0
 // issues tcgen05.mma (M = 128, N = BN, K = 16) into one of two accumulators in
 // tensor memory (BN columns each); warps 4 to 11 drain the other one: warp w reads
@@ -346,17 +346,8 @@ __global__ void __launch_bounds__(G_THREADS, 1)
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <int BN>
-static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_rows, int lda,
-                                  const void* Bm, long long b_rows, int ldb, cudaStream_t st) {
-  CUtensorMap am, bm;
-  cudaError_t e = make_tmap_bf16(&am, A, (uint64_t)g.Kd, (uint64_t)a_rows, (uint64_t)lda, GM);
-  if (e != cudaSuccess) return e;
-  if ((e = make_tmap_bf16(&bm, Bm, (uint64_t)g.Kd, (uint64_t)b_rows, (uint64_t)ldb, BN)) !=
-      cudaSuccess)
-    return e;
-  const int per_image =
-      g.sym ? gemm_sym_ctas(g.M, 1) : ceil_div(g.Nn, BN) * ceil_div(g.M, GM);
+namespace {
+int gemm_sms() {
   static int sms = 0;
   if (sms == 0) {
     int dev = 0;
@@ -366,6 +357,28 @@ static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_
       sms = 152;
     }
   }
+  return sms;
+}
+
+// Tiles of an image in symmetric mode.
+template <int BN> int sym_tiles(int N) {
+  int nt = 0;
+  for (int I = 0; I < ceil_div(N, GM); ++I) nt += ceil_div(N, BN) - sym_first_col<BN>(I);
+  return nt;
+}
+}  // namespace
+
+template <int BN>
+static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_rows, int lda,
+                                  const void* Bm, long long b_rows, int ldb, cudaStream_t st) {
+  CUtensorMap am, bm;
+  cudaError_t e = make_tmap_bf16(&am, A, (uint64_t)g.Kd, (uint64_t)a_rows, (uint64_t)lda, GM);
+  if (e != cudaSuccess) return e;
+  if ((e = make_tmap_bf16(&bm, Bm, (uint64_t)g.Kd, (uint64_t)b_rows, (uint64_t)ldb, BN)) !=
+      cudaSuccess)
+    return e;
+  const int per_image = g.sym ? sym_tiles<BN>(g.M) : ceil_div(g.Nn, BN) * ceil_div(g.M, GM);
+  const int sms = gemm_sms();
   const long long tiles = (long long)per_image * g.B;
   if (tiles > 0x7fffffffLL - sms) return cudaErrorInvalidValue;
   constexpr size_t smem = gemm_smem<BN>();
@@ -375,11 +388,7 @@ static cudaError_t launch_gemm_bn(const GemmArgs& g, const void* A, long long a_
   return cudaGetLastError();
 }
 
-int gemm_sym_ctas(int N, int B) {  // symmetric Grams use 128 x 256 tiles (N > 128)
-  int nt = 0;
-  for (int I = 0; I < ceil_div(N, GM); ++I) nt += ceil_div(N, 256) - sym_first_col<256>(I);
-  return nt * B;
-}
+int gemm_sym_ctas(int N, int B) { return sym_tiles<256>(N) * B; }
 
 cudaError_t launch_gemm_tc(const GemmArgs& g, const void* A, long long a_rows, int lda,
                            const void* Bm, long long b_rows, int ldb, cudaStream_t st) {
@@ -390,7 +399,18 @@ cudaError_t launch_gemm_tc(const GemmArgs& g, const void* A, long long a_rows, i
   // rows (the buffer may end right after the last image's text rows)
   if ((g.a_text && g.M < GM) || (g.b_text && g.Nn < (g.Nn <= 128 ? 128 : 256)))
     return cudaErrorInvalidValue;
-  if (g.Nn <= 128) return launch_gemm_bn<128>(g, A, a_rows, lda, Bm, b_rows, ldb, st);
+  bool narrow = g.Nn <= 128;
+  if (g.sym) {
+    // 128 x 128 tiles where they take no more turns of the SMs than 128 x 256 ones (each
+    // turn is then shorter): a call of gmc_cosine, 4 images of N = 1,296 67 us, 57 so; 20 of
+    // 576 88 and 75; 80 of 256 (D = 256) 36 and 26.  With one turn more the wide tiles
+    // win (5 of 1,296: 69 and 76; 32: 276 and 327).
+    const int sms = gemm_sms();
+    const long long wide = (long long)sym_tiles<256>(g.M) * g.B;
+    const long long half = (long long)sym_tiles<128>(g.M) * g.B;
+    narrow = (half + sms - 1) / sms <= (wide + sms - 1) / sms;
+  }
+  if (narrow) return launch_gemm_bn<128>(g, A, a_rows, lda, Bm, b_rows, ldb, st);
   return launch_gemm_bn<256>(g, A, a_rows, lda, Bm, b_rows, ldb, st);
 }
 

@@ -311,7 +311,7 @@ struct GemmArgs {
                              // or above the diagonal computed, the rest mirrored
   int m_fast;                // 1: consecutive CTAs walk the row tiles (B is the larger operand)
 };
-int gemm_sym_ctas(int N, int B);  // CTAs of the symmetric mode for N x N Grams of B images
+int gemm_sym_ctas(int N, int B);  // 128 x 256 tiles of the symmetric mode, N x N Grams of B images
 // a_rows / b_rows: rows declared in the operand's tensor map (reads past them
 // return zeros); lda / ldb: row pitch in elements (a multiple of 8).
 cudaError_t launch_gemm_tc(const GemmArgs&, const void* A, long long a_rows, int lda,

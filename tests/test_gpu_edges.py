@@ -312,10 +312,10 @@ def test_assignment_gates(shape, K, gate_scale, weight, margin, twins):
 
 
 # tensor-core Gram: one tile a CTA and several (both accumulators, the stage ring over
-# tile boundaries), rows of C on 16 bytes and not, a last tile that is shifted inward,
+# tile boundaries), tiles of 128 and of 256 columns, rows of C on 16 bytes and not, a last tile that is shifted inward,
 # blocks on, above and mirrored below the diagonal, K that ends inside a slice
 @pytest.mark.parametrize("B,gh,gw,D,T", [
-    (80, 16, 16, 64, 3), (31, 12, 25, 1000, 5), (12, 23, 31, 264, 2), (2, 47, 49, 72, 7),
+    (80, 16, 16, 64, 3), (4, 36, 36, 200, 2), (14, 24, 24, 64, 5), (90, 17, 17, 136, 1), (31, 12, 25, 1000, 5), (12, 23, 31, 264, 2), (2, 47, 49, 72, 7),
     (1, 64, 65, 512, 1), (3, 36, 36, 3584, 9), (1, 79, 77, 136, 4)])
 def test_cosine_gram_tiles(B, gh, gw, D, T):
     from paper_2608_02134_gb300 import gmc
