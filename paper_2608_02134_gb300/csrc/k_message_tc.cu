@@ -17,11 +17,12 @@
 // is appendix Eq. (cond-native-message): the visual slice of the native causal
 // softmax, not renormalised over the image.
 //
-// Roles: warp 8 / lane 0 loads the query tile once and streams key tiles with
-// TMA through a 4-stage ring; warp 9 / lane 0 issues tcgen05.mma into two
-// 128-column TMEM accumulators (double buffered); warps 0..7 read the
-// accumulators (warp w: TMEM lanes 32*(w%4).., columns 64*(w/4)..) and do the
+// Roles: warp 16 / lane 0 loads the query tile once and streams key tiles with
+// TMA through a 2-stage ring; warp 17 / lane 0 issues tcgen05.mma into two
+// 128-column TMEM accumulators (double buffered); warps 0..15 read the
+// accumulators (warp w: TMEM lanes 32*(w%4).., columns 32*(w/4)..) and do the
 // softmax arithmetic.  Every wait is clock-bounded.
+// k_message_fused does the same in one launch where msg_split says so.
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       if (!ok) ctl->abort = 1;
     }
     __syncwarp();
-  } else {  // ---------------- epilogue warps 0..7
+  } else {  // ---------------- epilogue warps
     const int quarter = warp & 3, cpart = warp >> 2;  // TMEM lane quarter, 32-column part
     const int r = quarter * 32 + lane;           // tile row == TMEM lane
     const int R = tile * BM + r;                 // packed row
@@ -749,9 +750,9 @@ cudaError_t launch_message_tc(const Dims& dm, const void* keys, const void* quer
   }
   if (launches) *launches = 2;
   for (int mode = 0; mode < 2; ++mode) {
-    launch_k(k_message_tc, grid, THREADS, msg_smem_bytes(nkb, mode), st, 1, qmap, kmap, dm.toff, dm.B, dm.N, dm.T, dm.H, dm.Hkv,
-                                              dm.d, RQ, mode, sp.n, s.mpart, s.zn2,
-                                              s.sigma, s.A, s.rs, s.status);
+    launch_k(k_message_tc, grid, THREADS, msg_smem_bytes(nkb, mode), st, 1, qmap, kmap, dm.toff,
+             dm.B, dm.N, dm.T, dm.H, dm.Hkv, dm.d, RQ, mode, sp.n, s.mpart, s.zn2, s.sigma, s.A,
+             s.rs, s.status);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
